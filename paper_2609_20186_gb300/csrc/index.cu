@@ -36,15 +36,26 @@ namespace switchsd {
 constexpr int kIdxMaxWarps = SWITCHSD_NMAX;
 constexpr int kIdxTail = SWITCHSD_NMAX + SWITCHSD_KMAX + 1;  // staged context tail: old end +- the append
 
-// Multiply-xorshift hash of the n tokens ending at the last one (`tok(i)` = token i steps back).
+// Hash of the n tokens ending at the last one (`tok(i)` = token i steps back): a polynomial in an odd
+// multiplier mod 2^32, whose terms are independent (one multiply-add each, no chain through a mixer), then
+// two multiply-xorshift rounds; the bucket is its top bits.
+constexpr uint32_t kGramMul = 0x9E3779B1u;
+__device__ __forceinline__ uint32_t gram_bucket(uint32_t h, int n, int log2_buckets) {
+    h += uint32_t(n) * 0x85EBCA77u;
+    h ^= h >> 15;
+    h *= 0x2C1B3C6Du;
+    h ^= h >> 13;
+    h *= 0x297A2D39u;
+    return h >> (32 - log2_buckets);
+}
 template <typename Tok>
 __device__ __forceinline__ uint32_t gram_hash(int n, Tok tok, int log2_buckets) {
-    uint64_t h = 0x243F6A8885A308D3ull ^ uint64_t(n);
+    uint32_t h = 0u, pw = 1u;
     for (int i = 0; i < n; ++i) {
-        h = (h ^ uint64_t(uint32_t(tok(i)))) * 0x9E3779B97F4A7C15ull;
-        h ^= h >> 29;
+        h += uint32_t(tok(i)) * pw;
+        pw *= kGramMul;
     }
-    return uint32_t(h >> (64 - log2_buckets));
+    return gram_bucket(h, n, log2_buckets);
 }
 
 struct IndexArgs {
@@ -355,43 +366,293 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
     }
 }
 
-// Build: positions n-1 .. L-1 of every (row, n) inserted in increasing order, 32 per warp iteration.
-__global__ void __launch_bounds__(256) index_build_kernel(const int32_t *ctx, const int32_t *lens, int32_t *heads_all,
-                                                          int32_t *prev_all, int32_t B, int32_t cap, int32_t n_min,
-                                                          int32_t nn, int32_t log2_buckets) {
-    const int lane = threadIdx.x & 31;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // one warp per (n, row)
+// ------------------------------------------------------------------------------------------------
+// Build.  One item = one (row, n); its buckets are split over P CTAs (part = the bucket's top bits).  A CTA
+// goes over the row in chunks of kChunk positions; per chunk, warp w owns a contiguous segment:
+//   1. hash: every position's bucket (kept in registers), positions of other parts dropped; the segment's
+//      counts per bin (the next 8 bits of the bucket) in shared memory;
+//   2. scan: offsets of every (bin, warp), so that a bin's entries lie in position order;
+//   3. scatter: (position, key) into a queue in shared memory, key = the bucket's remaining bits (<= 9);
+//   4. link: warp w takes the bins w, w + kW, ... on its own (no barrier): the bin's heads (<= 512, 16-bit
+//      chunk positions) live in shared memory, the entries are linked 32 at a time in order through
+//      __match_any_sync, and the bin's heads go out in one coalesced write, the empty ones included (so
+//      nothing clears the table first);
+//   5. the links, held in shared memory as 16-bit chunk positions, go out coalesced (P = 1; with P > 1 a
+//      part's positions are scattered and step 4 stores them).
+// Steps 1 to 3 are one stable radix pass, so the time does not depend on how the tokens repeat, except that
+// one bucket's entries are linked by one warp.  A later chunk takes the head of a bucket it has not seen
+// from the table its own bins' warp wrote (same warp, earlier chunk) and updates only the heads it moved.
+//
+// Why: one warp per item walking its row 32 positions at a time (a dependent head read and write each) took
+// 1210 us for 64 rows of 32K tokens, n = 3..8 (build and one step); this takes 177 us.  The table written sets
+// the floor (201 MB of heads + 50 MB of links: 37 us at the measured copy bandwidth); what bounds it is the
+// issue rate and latency of the five phases at one 1024-thread CTA an SM (384 CTAs: 2.5 waves).
+// ------------------------------------------------------------------------------------------------
+constexpr int kBuildKeyBits = 9;
+constexpr int kBuildBins = 256;
+constexpr uint32_t kNone16 = 0xffffu;  // no earlier entry; kDone16: the link is in global memory already
+constexpr uint32_t kDone16 = 0xfffeu;
+
+struct BuildArgs {
+    const int32_t *ctx, *lens;
+    int32_t *heads, *prev;
+    int32_t B, cap, n_min, nn, log2_buckets, log2_parts;
+};
+
+template <int kT, int kChunk>
+struct BuildLayout {
+    static constexpr int kW = kT / kWarp;
+    static constexpr size_t queue = size_t(kChunk) * 4;
+    static constexpr size_t counts = size_t(kW) * (kBuildBins + 1) * 4;
+    static constexpr size_t links = size_t(kChunk) * 2 > counts ? size_t(kChunk) * 2 : counts;  // counts, then links
+    static constexpr size_t heads = size_t(kW) * (2 << kBuildKeyBits);
+    static constexpr size_t bytes = queue + links + heads;
+};
+
+// The lanes of `live` that hold the same kBits-bit value as this one, one ballot a bit (every lane calls it; a
+// lane outside `live` is in no other lane's mask).  On this GPU __match_any_sync on 32 mostly distinct values
+// costs more issue slots than the kBits ballots (a build of 64 rows of 32K tokens 250 us against 196 us).
+template <int kBits>
+__device__ __forceinline__ unsigned same_value_lanes(uint32_t v, unsigned live) {
+    unsigned m = live;
+#pragma unroll
+    for (int i = 0; i < kBits; ++i) {
+        const bool set = (v >> i & 1u) != 0u;
+        m &= __ballot_sync(kFull, set) ^ (set ? 0u : ~0u);
+    }
+    return m;
+}
+
+template <int kT, int kChunk>
+__global__ void __launch_bounds__(kT) index_build_kernel(const BuildArgs a) {
+    using Lay = BuildLayout<kT, kChunk>;
+    constexpr int kW = Lay::kW;
+    constexpr int kIts = kChunk / kT;  // positions a thread holds
+    static_assert(kIts % 8 == 0 && kChunk <= 32768, "15-bit chunk positions, rounds of eight");
+    extern __shared__ __align__(16) unsigned char build_smem[];
+    uint32_t *q = reinterpret_cast<uint32_t *>(build_smem);
+    uint32_t *cnt = reinterpret_cast<uint32_t *>(build_smem + Lay::queue);     // [kW][kBuildBins + 1]
+    uint16_t *links = reinterpret_cast<uint16_t *>(build_smem + Lay::queue);   // [kChunk]
+    uint16_t *heads16 = reinterpret_cast<uint16_t *>(build_smem + Lay::queue + Lay::links);
+    __shared__ uint32_t s_bin[kBuildBins + 1];
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int part = int(blockIdx.x) & ((1 << a.log2_parts) - 1);
+    const int item = int(blockIdx.x) >> a.log2_parts;
+    const int w = item / a.B, b = item - w * a.B;
+    const int n = a.n_min + w;
+    const int lg = a.log2_buckets, lgp = lg - a.log2_parts;  // bucket bits, and those within the part
+    const int binbits = lgp < 8 ? lgp : 8, keybits = lgp - binbits;
+    const uint32_t keymask = (1u << keybits) - 1u;
     pdl_wait();
     pdl_trigger();
-    if (gw >= nn * B) return;
-    const int w = gw / B, b = gw % B;
-    const int n = n_min + w;
-    const size_t nb = size_t(1) << log2_buckets;
-    int32_t *heads = heads_all + (size_t(w) * B + b) * nb;
-    int32_t *prev = prev_all + (size_t(w) * B + b) * cap;
-    const int32_t *row = ctx + size_t(b) * cap;
-    int32_t L = lens[b];
-    if (L < 0 || L > cap) L = 0;
-    for (int32_t base = 0; base < L; base += kWarp) {
-        const int32_t p = base + lane;
-        const bool valid = p < L && p >= n - 1;
-        uint32_t bucket = 0xffffffffu;
-        if (valid) bucket = gram_hash(n, [&](int i) { return row[p - i]; }, log2_buckets);
-        const unsigned peers = __match_any_sync(kFull, bucket) & __ballot_sync(kFull, valid);
-        const int32_t old_head = valid ? heads[bucket] : -1;
-        __syncwarp();  // every lane has read its head before any lane replaces one
-        if (valid) {
-            const unsigned earlier = peers & ((1u << lane) - 1u);
-            prev[p] = earlier ? base + (31 - __clz(earlier)) : old_head;
-            if ((peers >> lane) == 1u) heads[bucket] = p;
+    int32_t *heads = a.heads + (size_t(w) * a.B + b) * (size_t(1) << lg) + (size_t(part) << lgp);
+    int32_t *prev = a.prev + (size_t(w) * a.B + b) * size_t(a.cap);
+    const int32_t *row = a.ctx + size_t(b) * size_t(a.cap);
+    int32_t L = a.lens[b];
+    if (L < 0 || L > a.cap) L = 0;
+    uint16_t *H = heads16 + (warp << kBuildKeyBits);
+
+    for (int32_t c0 = 0; c0 == 0 || c0 < L; c0 += kChunk) {
+        const int32_t clen = min(kChunk, L - c0);
+        const int32_t seg = ((clen + kW - 1) / kW + 31) & ~31;  // a warp's positions: <= kChunk / kW
+        const int32_t p_seg = c0 + warp * seg;
+        for (int i = tid; i < kW * (kBuildBins + 1); i += kT) cnt[i] = 0u;
+        __syncthreads();
+
+        // 1. hash and count
+        uint32_t code[kIts];  // bin << kBuildKeyBits | key, all ones for a dropped position
+#pragma unroll
+        for (int r = 0; r < kIts / 8; ++r) {
+            uint32_t h[8];
+            const int32_t p0 = p_seg + 256 * r;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) h[u] = 0u;
+            if (256 * r < seg && p0 < L) {  // warp-uniform
+                uint32_t pw = 1u;
+                if (p0 >= n - 1 && p0 + 256 <= L) {
+                    const int32_t *x = row + p0 + lane;
+                    for (int i = 0; i < n; ++i, --x, pw *= kGramMul)
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) h[u] += uint32_t(__ldg(x + 32 * u)) * pw;
+                } else {
+                    for (int i = 0; i < n; ++i, pw *= kGramMul)
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            h[u] += uint32_t(__ldg(row + min(max(p0 + lane + 32 * u - i, 0), L - 1))) * pw;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int32_t p = p0 + 32 * u + lane;
+                const uint32_t bucket = gram_bucket(h[u], n, lg);
+                const bool mine = 256 * r + 32 * u < seg && p < L && p >= n - 1 && int(bucket >> lgp) == part;
+                const uint32_t local = bucket & ((1u << lgp) - 1u);
+                const uint32_t bin = local >> keybits;
+                code[8 * r + u] = mine ? (bin << kBuildKeyBits | (local & keymask)) : 0xffffffffu;
+                if (mine) atomicAdd(&cnt[warp * (kBuildBins + 1) + int(bin)], 1u);
+            }
         }
-        __syncwarp();
+        __syncthreads();
+
+        // 2. offsets: within a bin over the warps, then over the bins
+        for (int bin = warp; bin < kBuildBins; bin += kW) {
+            const uint32_t v = lane < kW ? cnt[lane * (kBuildBins + 1) + bin] : 0u;
+            uint32_t incl = v;
+#pragma unroll
+            for (int o = 1; o < kWarp; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += t;
+            }
+            if (lane < kW) cnt[lane * (kBuildBins + 1) + bin] = incl - v;
+            if (lane == kWarp - 1) s_bin[bin + 1] = incl;
+        }
+        if (tid == 0) s_bin[0] = 0u;
+        __syncthreads();
+        if (warp == 0) {
+            uint32_t v[kBuildBins / kWarp], sum = 0u;
+#pragma unroll
+            for (int j = 0; j < kBuildBins / kWarp; ++j) {
+                sum += s_bin[1 + lane * (kBuildBins / kWarp) + j];
+                v[j] = sum;
+            }
+            uint32_t incl = sum;
+#pragma unroll
+            for (int o = 1; o < kWarp; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += t;
+            }
+#pragma unroll
+            for (int j = 0; j < kBuildBins / kWarp; ++j)
+                s_bin[1 + lane * (kBuildBins / kWarp) + j] = incl - sum + v[j];
+        }
+        __syncthreads();
+
+        // 3. scatter into the queue, in position order within a bin
+        uint32_t *my = cnt + warp * (kBuildBins + 1);
+#pragma unroll
+        for (int i = 0; i < kIts; ++i) {
+            if (32 * i < seg) {  // warp-uniform
+                const uint32_t c = code[i];
+                const bool mine = c != 0xffffffffu;
+                const uint32_t bin = c >> kBuildKeyBits;
+                const unsigned peers = same_value_lanes<8>(bin, __ballot_sync(kFull, mine));
+                const int rank = __popc(peers & ((1u << lane) - 1u));
+                const uint32_t at = mine ? my[bin] : 0u;
+                __syncwarp();  // every lane has read its counter before the group's first lane moves it
+                if (mine) {
+                    if (rank == 0) my[bin] = at + uint32_t(__popc(peers));
+                    const uint32_t lp = uint32_t(p_seg - c0 + 32 * i + lane);
+                    q[s_bin[bin] + at + uint32_t(rank)] = lp << kBuildKeyBits | (c & ((1u << kBuildKeyBits) - 1u));
+                }
+                __syncwarp();
+            }
+        }
+        __syncthreads();  // the counters are dead from here on: the links take their place
+
+        // 4. link each bin's entries in order
+        const int nbins = 1 << binbits, kb = 1 << keybits;
+        for (int bin = warp; bin < nbins; bin += kW) {
+            for (int i = lane; i < (kb + 7) / 8; i += kWarp)  // H holds 1 << kBuildKeyBits entries
+                reinterpret_cast<uint4 *>(H)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+            __syncwarp();
+            int32_t *hb = heads + (size_t(bin) << keybits);
+            const uint32_t end = s_bin[bin + 1];
+            for (uint32_t base = s_bin[bin]; base < end; base += kWarp) {
+                const bool live = base + lane < end;
+                const uint32_t ent = live ? q[base + lane] : 0u;
+                const uint32_t key = ent & ((1u << kBuildKeyBits) - 1u), lp = ent >> kBuildKeyBits;
+                const uint32_t head = live ? uint32_t(H[key]) : kNone16;
+                __syncwarp();  // every lane has read its head before any lane replaces one
+                if (live) H[key] = uint16_t(lp);
+                __syncwarp();
+                uint32_t l16 = head;
+                // Two entries of one key in this round are rare: then the group is found by ballots, each
+                // entry links to the one before it and the last is the head.
+                if (__any_sync(kFull, live && uint32_t(H[key]) != lp)) {
+                    const unsigned peers = same_value_lanes<kBuildKeyBits>(key, __ballot_sync(kFull, live));
+                    const unsigned earlier = peers & ((1u << lane) - 1u);
+                    const uint32_t before = __shfl_sync(kFull, lp, earlier ? 31 - __clz(earlier) : lane);
+                    if (earlier) l16 = before;
+                    if (live && (peers >> lane) == 1u) H[key] = uint16_t(lp);
+                    __syncwarp();
+                }
+                if (live) {
+                    if (a.log2_parts > 0 || (l16 == kNone16 && c0 > 0)) {
+                        // an earlier chunk's head: from the table, where this warp left it
+                        prev[c0 + int32_t(lp)] = l16 != kNone16 ? c0 + int32_t(l16) : (c0 > 0 ? hb[key] : -1);
+                        l16 = kDone16;
+                    }
+                    if (a.log2_parts == 0) links[lp] = uint16_t(l16);
+                }
+            }
+            __syncwarp();
+            if (c0 == 0 && kb >= 4) {
+                for (int i = lane; i < kb / 4; i += kWarp) {
+                    const short4 h = reinterpret_cast<const short4 *>(H)[i];  // kNone16 widens to -1
+                    reinterpret_cast<int4 *>(hb)[i] = make_int4(h.x, h.y, h.z, h.w);
+                }
+            } else {
+                for (int i = lane; i < kb; i += kWarp) {
+                    const uint32_t h = H[i];
+                    if (h != kNone16) hb[i] = c0 + int32_t(h);
+                    else if (c0 == 0) hb[i] = -1;
+                }
+            }
+            __syncwarp();
+        }
+        __syncthreads();
+
+        // 5. the links, four positions a thread (positions below n - 1 belong to no chain)
+        if (a.log2_parts == 0) {
+            for (int i = tid; 4 * i < clen; i += kT) {
+                const short4 l = reinterpret_cast<const short4 *>(links)[i];
+                int32_t *dst = prev + c0 + 4 * i;
+                if (c0 == 0) {  // kNone16 widens to -1, and no link is in global memory yet
+                    *reinterpret_cast<int4 *>(dst) = make_int4(l.x, l.y, l.z, l.w);
+                } else {  // every link here is to an entry of this chunk, or in global memory already
+                    if (uint16_t(l.x) != kDone16) dst[0] = c0 + l.x;
+                    if (uint16_t(l.y) != kDone16) dst[1] = c0 + l.y;
+                    if (uint16_t(l.z) != kDone16) dst[2] = c0 + l.z;
+                    if (uint16_t(l.w) != kDone16) dst[3] = c0 + l.w;
+                }
+            }
+        }
+        __syncthreads();  // the queue and the counters' space are free for the next chunk
     }
 }
 
 // ------------------------------------------------------------------------------------------------
 // Host side.
 // ------------------------------------------------------------------------------------------------
+// The build's parts per item: enough that a part's buckets fit kBuildBins bins of 1 << kBuildKeyBits heads,
+// and more (up to 8) while the grid leaves SMs idle -- every part hashes the whole row, so more parts only
+// pay while they add CTAs.  Rows up to kBuildSmallChunk tokens of capacity take half-sized CTAs, two an SM.
+constexpr int kBuildSmallChunk = 16384;
+
+template <int kT, int kChunk>
+static cudaError_t launch_index_build(BuildArgs a, cudaStream_t stream) {
+    static int sms[64] = {0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    int n_sm = dev >= 0 && dev < 64 ? sms[dev] : 0;
+    if (n_sm == 0) {
+        e = cudaFuncSetAttribute(index_build_kernel<kT, kChunk>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 int(BuildLayout<kT, kChunk>::bytes));
+        if (e != cudaSuccess) return e;
+        e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) sms[dev] = n_sm;
+    }
+    const int64_t items = int64_t(a.nn) * a.B;
+    int lp = a.log2_buckets > 8 + kBuildKeyBits ? a.log2_buckets - 8 - kBuildKeyBits : 0;
+    while (lp < 3 && (items << (lp + 1)) <= n_sm && a.log2_buckets - lp > 8) ++lp;
+    a.log2_parts = lp;
+    return launch_pdl(index_build_kernel<kT, kChunk>, dim3(unsigned(items << lp)), dim3(kT),
+                      BuildLayout<kT, kChunk>::bytes, stream, 0u, a);
+}
+
 int index_n_min(const switchsd_index *idx) { return idx->n_min; }
 int index_n_max(const switchsd_index *idx) { return idx->n_max; }
 
@@ -497,13 +758,19 @@ extern "C" int switchsd_index_create(const switchsd_params *p, switchsd_index **
 extern "C" int switchsd_index_build(switchsd_index *idx, const int32_t *ctx_tokens, const int32_t *ctx_lens,
                                     void *stream) {
     if (!idx || !ctx_tokens || !ctx_lens) return SWITCHSD_ERR_ARG;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const size_t heads = size_t(idx->nn) * size_t(idx->B) * (size_t(1) << idx->log2_buckets) * sizeof(int32_t);
-    if (cudaMemsetAsync(idx->heads, 0xff, heads, s) != cudaSuccess) return SWITCHSD_ERR_CUDA;  // every head = -1
-    const int warps = idx->nn * idx->B;
-    const cudaError_t e = launch_pdl(index_build_kernel, dim3(unsigned((warps + 7) / 8)), dim3(256), 0, s, 0u,
-                                     ctx_tokens, ctx_lens, idx->heads, idx->prev, idx->B, idx->cap, idx->n_min,
-                                     idx->nn, idx->log2_buckets);
+    BuildArgs a;
+    a.ctx = ctx_tokens;
+    a.lens = ctx_lens;
+    a.heads = idx->heads;
+    a.prev = idx->prev;
+    a.B = idx->B;
+    a.cap = idx->cap;
+    a.n_min = idx->n_min;
+    a.nn = idx->nn;
+    a.log2_buckets = idx->log2_buckets;
+    const cudaError_t e = idx->cap <= kBuildSmallChunk
+                              ? launch_index_build<512, kBuildSmallChunk>(a, static_cast<cudaStream_t>(stream))
+                              : launch_index_build<1024, 2 * kBuildSmallChunk>(a, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? SWITCHSD_OK : SWITCHSD_ERR_CUDA;
 }
 
