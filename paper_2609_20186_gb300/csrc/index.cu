@@ -369,8 +369,10 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
 // ------------------------------------------------------------------------------------------------
 // Build.  One item = one (row, n); its buckets are split over P CTAs (part = the bucket's top bits).  A CTA
 // goes over the row in chunks of kChunk positions; per chunk, warp w owns a contiguous segment:
-//   1. hash: every position's bucket (kept in registers), positions of other parts dropped; the segment's
-//      counts per bin (the next 8 bits of the bucket) in shared memory;
+//   1. hash and rank: every position's bucket, positions of other parts dropped, and its rank within the
+//      segment's positions of its bin (the next 8 bits of the bucket), kept in registers; the lanes of a bin
+//      find each other through a mask per bin in shared memory (an atomicOr, a read), and the segment's counts
+//      per bin run along;
 //   2. scan: offsets of every (bin, warp), so that a bin's entries lie in position order;
 //   3. scatter: (position, key) into a queue in shared memory, key = the bucket's remaining bits (<= 9);
 //   4. link: warp w takes the bins w, w + kW, ... on its own (no barrier): the bin's heads (<= 512, 16-bit
@@ -384,12 +386,14 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
 // from the table its own bins' warp wrote (same warp, earlier chunk) and updates only the heads it moved.
 //
 // Why: one warp per item walking its row 32 positions at a time (a dependent head read and write each) took
-// 1210 us for 64 rows of 32K tokens, n = 3..8 (build and one step); this takes 177 us.  The table written sets
+// 1210 us for 64 rows of 32K tokens, n = 3..8 (build and one step); this takes 155 us (177 us with the ranks taken by
+// eight ballots a position and counted in a pass of their own).  The table written sets
 // the floor (201 MB of heads + 50 MB of links: 37 us at the measured copy bandwidth); what bounds it is the
 // issue rate and latency of the five phases at one 1024-thread CTA an SM (384 CTAs: 2.5 waves).
 // ------------------------------------------------------------------------------------------------
 constexpr int kBuildKeyBits = 9;
 constexpr int kBuildBins = 256;
+constexpr int kRankShift = kBuildKeyBits + 8;  // a segment's rank within a bin (at most 1024) above bin and key
 constexpr uint32_t kNone16 = 0xffffu;  // no earlier entry; kDone16: the link is in global memory already
 constexpr uint32_t kDone16 = 0xfffeu;
 
@@ -405,13 +409,14 @@ struct BuildLayout {
     static constexpr size_t queue = size_t(kChunk) * 4;
     static constexpr size_t counts = size_t(kW) * (kBuildBins + 1) * 4;
     static constexpr size_t links = size_t(kChunk) * 2 > counts ? size_t(kChunk) * 2 : counts;  // counts, then links
-    static constexpr size_t heads = size_t(kW) * (2 << kBuildKeyBits);
+    static constexpr size_t heads = size_t(kW) * (2 << kBuildKeyBits);  // step 1's masks, then the bins' heads
+    static_assert(heads == size_t(kW) * kBuildBins * 4, "a mask per bin and warp");
     static constexpr size_t bytes = queue + links + heads;
 };
 
 // The lanes of `live` that hold the same kBits-bit value as this one, one ballot a bit (every lane calls it; a
 // lane outside `live` is in no other lane's mask).  On this GPU __match_any_sync on 32 mostly distinct values
-// costs more issue slots than the kBits ballots (a build of 64 rows of 32K tokens 250 us against 196 us).
+// costs more issue slots than the kBits ballots.
 template <int kBits>
 __device__ __forceinline__ unsigned same_value_lanes(uint32_t v, unsigned live) {
     unsigned m = live;
@@ -458,10 +463,12 @@ __global__ void __launch_bounds__(kT) index_build_kernel(const BuildArgs a) {
         const int32_t seg = ((clen + kW - 1) / kW + 31) & ~31;  // a warp's positions: <= kChunk / kW
         const int32_t p_seg = c0 + warp * seg;
         for (int i = tid; i < kW * (kBuildBins + 1); i += kT) cnt[i] = 0u;
+        for (int i = tid; i < kW * kBuildBins; i += kT) reinterpret_cast<uint32_t *>(heads16)[i] = 0u;
         __syncthreads();
 
-        // 1. hash and count
-        uint32_t code[kIts];  // bin << kBuildKeyBits | key, all ones for a dropped position
+        // 1. hash and rank
+        uint32_t *mask = reinterpret_cast<uint32_t *>(H), *my = cnt + warp * (kBuildBins + 1);
+        uint32_t code[kIts];  // rank << kRankShift | bin << kBuildKeyBits | key, all ones for a dropped position
 #pragma unroll
         for (int r = 0; r < kIts / 8; ++r) {
             uint32_t h[8];
@@ -489,8 +496,19 @@ __global__ void __launch_bounds__(kT) index_build_kernel(const BuildArgs a) {
                 const bool mine = 256 * r + 32 * u < seg && p < L && p >= n - 1 && int(bucket >> lgp) == part;
                 const uint32_t local = bucket & ((1u << lgp) - 1u);
                 const uint32_t bin = local >> keybits;
-                code[8 * r + u] = mine ? (bin << kBuildKeyBits | (local & keymask)) : 0xffffffffu;
-                if (mine) atomicAdd(&cnt[warp * (kBuildBins + 1) + int(bin)], 1u);
+                if (mine) atomicOr(&mask[bin], 1u << lane);
+                __syncwarp();
+                const uint32_t peers = mine ? mask[bin] : 0u, at = mine ? my[bin] : 0u;
+                const uint32_t below = peers & ((1u << lane) - 1u);
+                __syncwarp();  // every lane has read its bin before the bin's first lane moves it on
+                if (mine && below == 0u) {
+                    my[bin] = at + uint32_t(__popc(peers));
+                    mask[bin] = 0u;
+                }
+                code[8 * r + u] = mine ? ((at + uint32_t(__popc(below))) << kRankShift | bin << kBuildKeyBits |
+                                          (local & keymask))
+                                       : 0xffffffffu;
+                __syncwarp();
             }
         }
         __syncthreads();
@@ -529,23 +547,13 @@ __global__ void __launch_bounds__(kT) index_build_kernel(const BuildArgs a) {
         __syncthreads();
 
         // 3. scatter into the queue, in position order within a bin
-        uint32_t *my = cnt + warp * (kBuildBins + 1);
 #pragma unroll
         for (int i = 0; i < kIts; ++i) {
-            if (32 * i < seg) {  // warp-uniform
-                const uint32_t c = code[i];
-                const bool mine = c != 0xffffffffu;
-                const uint32_t bin = c >> kBuildKeyBits;
-                const unsigned peers = same_value_lanes<8>(bin, __ballot_sync(kFull, mine));
-                const int rank = __popc(peers & ((1u << lane) - 1u));
-                const uint32_t at = mine ? my[bin] : 0u;
-                __syncwarp();  // every lane has read its counter before the group's first lane moves it
-                if (mine) {
-                    if (rank == 0) my[bin] = at + uint32_t(__popc(peers));
-                    const uint32_t lp = uint32_t(p_seg - c0 + 32 * i + lane);
-                    q[s_bin[bin] + at + uint32_t(rank)] = lp << kBuildKeyBits | (c & ((1u << kBuildKeyBits) - 1u));
-                }
-                __syncwarp();
+            const uint32_t c = code[i];
+            if (c != 0xffffffffu) {
+                const uint32_t bin = c >> kBuildKeyBits & uint32_t(kBuildBins - 1);
+                const uint32_t lp = uint32_t(p_seg - c0 + 32 * i + lane);
+                q[s_bin[bin] + my[bin] + (c >> kRankShift)] = lp << kBuildKeyBits | (c & ((1u << kBuildKeyBits) - 1u));
             }
         }
         __syncthreads();  // the counters are dead from here on: the links take their place
@@ -558,17 +566,17 @@ __global__ void __launch_bounds__(kT) index_build_kernel(const BuildArgs a) {
             __syncwarp();
             int32_t *hb = heads + (size_t(bin) << keybits);
             const uint32_t end = s_bin[bin + 1];
-            for (uint32_t base = s_bin[bin]; base < end; base += kWarp) {
-                const bool live = base + lane < end;
+            // one round of 32 entries: (position, link), the link kNone16 when the bin holds no earlier entry
+            auto round = [&](uint32_t base, bool live, uint32_t &key, uint32_t &lp) {
                 const uint32_t ent = live ? q[base + lane] : 0u;
-                const uint32_t key = ent & ((1u << kBuildKeyBits) - 1u), lp = ent >> kBuildKeyBits;
-                const uint32_t head = live ? uint32_t(H[key]) : kNone16;
+                key = ent & ((1u << kBuildKeyBits) - 1u);
+                lp = ent >> kBuildKeyBits;
+                uint32_t l16 = live ? uint32_t(H[key]) : kNone16;
                 __syncwarp();  // every lane has read its head before any lane replaces one
                 if (live) H[key] = uint16_t(lp);
                 __syncwarp();
-                uint32_t l16 = head;
-                // Two entries of one key in this round are rare: then the group is found by ballots, each
-                // entry links to the one before it and the last is the head.
+                // Two entries of one key in a round are rare: then the group is found by ballots, each entry
+                // links to the one before it and the last is the head.
                 if (__any_sync(kFull, live && uint32_t(H[key]) != lp)) {
                     const unsigned peers = same_value_lanes<kBuildKeyBits>(key, __ballot_sync(kFull, live));
                     const unsigned earlier = peers & ((1u << lane) - 1u);
@@ -577,13 +585,27 @@ __global__ void __launch_bounds__(kT) index_build_kernel(const BuildArgs a) {
                     if (live && (peers >> lane) == 1u) H[key] = uint16_t(lp);
                     __syncwarp();
                 }
-                if (live) {
-                    if (a.log2_parts > 0 || (l16 == kNone16 && c0 > 0)) {
-                        // an earlier chunk's head: from the table, where this warp left it
-                        prev[c0 + int32_t(lp)] = l16 != kNone16 ? c0 + int32_t(l16) : (c0 > 0 ? hb[key] : -1);
-                        l16 = kDone16;
+                return l16;
+            };
+            uint32_t key, lp;
+            if (c0 == 0 && a.log2_parts == 0) {
+                for (uint32_t base = s_bin[bin]; base < end; base += kWarp) {
+                    const bool live = base + lane < end;
+                    const uint32_t l16 = round(base, live, key, lp);
+                    if (live) links[lp] = uint16_t(l16);
+                }
+            } else {
+                for (uint32_t base = s_bin[bin]; base < end; base += kWarp) {
+                    const bool live = base + lane < end;
+                    uint32_t l16 = round(base, live, key, lp);
+                    if (live) {
+                        if (a.log2_parts > 0 || l16 == kNone16) {
+                            // an earlier chunk's head: from the table, where this warp left it
+                            prev[c0 + int32_t(lp)] = l16 != kNone16 ? c0 + int32_t(l16) : (c0 > 0 ? hb[key] : -1);
+                            l16 = kDone16;
+                        }
+                        if (a.log2_parts == 0) links[lp] = uint16_t(l16);
                     }
-                    if (a.log2_parts == 0) links[lp] = uint16_t(l16);
                 }
             }
             __syncwarp();
