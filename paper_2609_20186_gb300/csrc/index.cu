@@ -14,6 +14,12 @@
 //   insertion of the appended end positions (all lanes at once; positions of one run that fall into
 //   the same bucket are linked through __match_any_sync, so one read of the old heads suffices);
 //   the lookup, the probe and the switch / copy draft (as switchsd_step), when stepping.
+// What bounds it is the chain of dependent L2 round trips, three after the wait: the verification's inputs
+// (all loads at once), the heads (with the link of a position inserted before), then per chain entry the
+// tokens compared, the next link and the tokens that follow it.  The lookup starts from the link that the
+// insert of the suffix's own end found, and the draft is written from the registers of the n that wins.  16
+// rows of 128K tokens, n = 2..12, 16 launches: 82.6 us with the heads and links read again for the lookup and
+// the draft gathered at the end (seven round trips), 74.4 us so.
 // Candidate mode (W > 0, as switchsd_step_candidates / switchsd_verify_candidates): the previous W
 // candidates are verified and the longest accepted one appended; the warp of n = kappa walks its
 // chain on past the first match and lists the W most recent ends whose kappa-gram equals the
@@ -111,7 +117,6 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
     __shared__ int32_t s_ver[3];             // accepted, new length, status
     __shared__ int32_t s_found[kIdxMaxWarps];
     __shared__ float s_wz[kIdxMaxWarps];
-    __shared__ int32_t s_out[3];
     __shared__ int32_t s_cend[SWITCHSD_WMAX];  // candidate mode: the listed ends, most recent first
     __shared__ int32_t s_ncf;
 
@@ -129,15 +134,47 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
     if (!pf_ctx) pdl_wait();
 
     if (tid == 0) s_ncf = 0;
+    // The previous draft, the target (and the sampled rule's numbers), lane i positions i and i + 32: one round
+    // of independent loads, after the wait.
+    int32_t pv_n = 0, d_lo = 0, d_hi = 0, t_lo = 0, t_hi = 0, t_top = 0;
+    float u_lo = 0.f, u_hi = 0.f, q_lo = 1.f, q_hi = 1.f, p_lo = 0.f, p_hi = 0.f;
+    auto load_draft = [&]() {
+        if (!verifying || a.W > 0 || warp != 0) return;
+        const int32_t *dr = a.pv_draft + size_t(b) * a.k;
+        const int32_t *tg = a.pv_target + size_t(b) * (a.k + 1);
+        pv_n = __ldcg(a.pv_len + b);
+        if (lane < a.k) d_lo = __ldcg(dr + lane);
+        if (lane + 32 < a.k) d_hi = __ldcg(dr + lane + 32);
+        if (lane <= a.k) t_lo = __ldcg(tg + lane);
+        if (lane + 32 <= a.k) t_hi = __ldcg(tg + lane + 32);
+        if (a.k >= 64) t_top = __ldcg(tg + 64);
+        if (a.pv_p != nullptr) {
+            const size_t o = size_t(b) * a.k + lane;
+            if (lane < a.k) {
+                u_lo = __ldcg(a.pv_u + o);
+                p_lo = __ldcg(a.pv_p + o);
+                if (a.pv_q) q_lo = __ldcg(a.pv_q + o);
+            }
+            if (lane + 32 < a.k) {
+                u_hi = __ldcg(a.pv_u + o + 32);
+                p_hi = __ldcg(a.pv_p + o + 32);
+                if (a.pv_q) q_hi = __ldcg(a.pv_q + o + 32);
+            }
+        }
+    };
+    if (!pf_ctx) load_draft();
     int32_t *row = a.ctx + size_t(b) * a.cap;
-    const int32_t L_old = a.lens[b];
+    const int32_t L_old = __ldcg(a.lens + b);  // (rewritten each step: not from an L1 line of an earlier grid)
     const bool len_ok = L_old >= 1 && L_old <= a.cap;
     const int32_t tail0 = L_old - SWITCHSD_NMAX;  // s_tail[i] = x[tail0 + i]
     for (int i = tid; i < SWITCHSD_NMAX; i += blockDim.x) {
         const int32_t p = tail0 + i;
-        s_tail[i] = (len_ok && p >= 0) ? row[p] : 0;
+        s_tail[i] = (len_ok && p >= 0) ? __ldcg(row + p) : 0;
     }
-    if (pf_ctx) pdl_wait();  // the previous draft, the target and the index tables come after this
+    if (pf_ctx) {
+        pdl_wait();  // the previous draft, the target and the index tables come after this
+        load_draft();
+    }
     pdl_trigger();
     if (warp == 0) {
         int32_t acc = -1, L = L_old, vst = len_ok ? SWITCHSD_ROW_OK : SWITCHSD_ROW_BAD_LEN;
@@ -183,38 +220,26 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
                 L = L_old + best + 1;
             }
         } else if (verifying && len_ok) {
-            const int32_t n = a.pv_len[b];
-            if (n < 0 || n > a.k) {
+            if (pv_n < 0 || pv_n > a.k) {
                 vst = SWITCHSD_ROW_BAD_LEN;
             } else {
-                const int32_t *dr = a.pv_draft + size_t(b) * a.k;
-                const int32_t *tg = a.pv_target + size_t(b) * (a.k + 1);
-                acc = n;
-                for (int base = 0; base < n; base += kWarp) {
-                    const int i = base + lane;
-                    // greedy: a draft token is rejected when it differs from the target's; sampled: when
-                    // u * q (binary32) is not below p
-                    bool rej = false;
-                    if (i < n) {
-                        if (a.pv_p != nullptr) {
-                            const size_t o = size_t(b) * a.k + i;
-                            rej = !(__fmul_rn(a.pv_u[o], a.pv_q ? a.pv_q[o] : 1.f) < a.pv_p[o]);
-                        } else {
-                            rej = dr[i] != tg[i];
-                        }
-                    }
-                    const unsigned m = __ballot_sync(kFull, rej);
-                    if (m) {
-                        acc = base + __ffs(m) - 1;
-                        break;
-                    }
+                // greedy: a draft token is rejected when it differs from the target's; sampled: when u * q
+                // (binary32) is not below p
+                bool rej_lo = lane < pv_n && d_lo != t_lo, rej_hi = lane + 32 < pv_n && d_hi != t_hi;
+                if (a.pv_p != nullptr) {
+                    rej_lo = lane < pv_n && !(__fmul_rn(u_lo, q_lo) < p_lo);
+                    rej_hi = lane + 32 < pv_n && !(__fmul_rn(u_hi, q_hi) < p_hi);
                 }
+                const unsigned m_lo = __ballot_sync(kFull, rej_lo);
+                const unsigned m_hi = __ballot_sync(kFull, rej_hi);
+                acc = m_lo ? __ffs(m_lo) - 1 : (m_hi ? 32 + __ffs(m_hi) - 1 : pv_n);
                 if (L_old + acc + 1 > a.cap) {
                     vst = SWITCHSD_ROW_CAPACITY;
                     acc = -1;
                 } else {
+                    const int32_t t_acc = __shfl_sync(kFull, acc < 32 ? t_lo : (acc < 64 ? t_hi : t_top), acc & 31);
                     for (int i = lane; i <= acc; i += kWarp) {
-                        const int32_t t = i < acc ? dr[i] : tg[acc];
+                        const int32_t t = i == acc ? t_acc : (i < 32 ? d_lo : d_hi);
                         s_tail[SWITCHSD_NMAX + i] = t;
                         row[L_old + i] = t;
                     }
@@ -245,23 +270,38 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
     int32_t *prev = a.prev + (size_t(warp) * a.B + b) * a.cap;
     auto tail_tok = [&](int32_t p) { return s_tail[p - tail0]; };  // valid for p in [tail0, L)
 
-    // Insert the appended end positions p in [L_old, L) (lanes over p, chained through match_any).
+    // Insert the appended end positions p in [L_old, L) (lanes over p, chained through match_any).  The last of
+    // them ends the suffix, so its link is where the lookup starts.
+    int32_t e = -1;         // the chain of the suffix n-gram, the suffix's own end skipped
+    bool linked = false;    // e is known from the insert
     if (has_n && L > L_old) {
         for (int32_t base = L_old; base < L; base += kWarp) {
             const int32_t p = base + lane;
             const bool valid = p < L && p >= n - 1;
             uint32_t bucket = 0xffffffffu;
             if (valid) bucket = gram_hash(n, [&](int i) { return tail_tok(p - i); }, a.log2_buckets);
+            int32_t old_head = -1, old_link = -1;
+            if (valid) {
+                old_head = __ldcg(heads + bucket);
+                if (p == L - 1) old_link = __ldcg(prev + p);  // p's link, if p was inserted before
+            }
             const unsigned peers = __match_any_sync(kFull, bucket) & __ballot_sync(kFull, valid);
-            const int32_t old_head = valid ? heads[bucket] : -1;
             __syncwarp();  // every lane has read its head before any lane replaces one
             // A head at or past p means these positions were inserted before (the same tokens appended
             // again after the lengths were rewound): the chains already hold them, so leave them be.
             // This keeps prev[p] < p, so every chain stays acyclic.
-            if (valid && old_head < p) {
+            int32_t link = old_head == p ? old_link : old_head;
+            const bool fresh = valid && old_head < p;
+            if (fresh) {
                 const unsigned earlier = peers & ((1u << lane) - 1u);
-                prev[p] = earlier ? base + (31 - __clz(earlier)) : old_head;
+                link = earlier ? base + (31 - __clz(earlier)) : old_head;
+                prev[p] = link;
                 if ((peers >> lane) == 1u) heads[bucket] = p;  // the latest position of the run
+            }
+            const unsigned last = __ballot_sync(kFull, valid && p == L - 1);
+            if (last) {
+                e = __shfl_sync(kFull, link, __ffs(last) - 1);
+                linked = true;
             }
             __syncwarp();
         }
@@ -269,27 +309,42 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
     if (!a.stepping) return;
 
     // Lookup: the most recent earlier occurrence of the suffix n-gram, if any.  Candidate mode: the
-    // warp of n = kappa lists the W most recent.
+    // warp of n = kappa lists the W most recent.  Per entry, the tokens compared, the next link and the
+    // tokens that follow (the draft, should it match) are loaded at once: one round trip an entry.
     const int32_t kappa_c = a.kappa > 0 ? a.kappa : a.n_min;
     const bool collect = a.W > 0 && has_n && n == kappa_c;
     int32_t found = -1, nfound = 0;
+    int32_t f_lo = 0, f_hi = 0;  // the tokens after `found`: e + 1 + lane, e + 33 + lane
     if (has_n && len_ok && L >= n + 1) {
-        const uint32_t bucket = gram_hash(n, [&](int i) { return tail_tok(L - 1 - i); }, a.log2_buckets);
         const int32_t mine = lane < n ? tail_tok(L - 1 - lane) : 0;
-        int32_t e = heads[bucket];
+        if (!linked) {
+            const uint32_t bucket = gram_hash(n, [&](int i) { return tail_tok(L - 1 - i); }, a.log2_buckets);
+            const int32_t own = __ldcg(prev + L - 1);  // (an unbuilt index may hold anything here: used below only as a link)
+            e = __ldcg(heads + bucket);
+            if (e == L - 1) e = own;
+        }
+        auto tok = [&](int32_t p) { return p >= L_old ? tail_tok(p) : __ldcg(row + p); };
         // A valid chain strictly decreases and ends at -1 within L hops; the bounds keep a stale or
         // unbuilt index from reading outside its tables.
         for (int32_t hops = 0; e >= 0 && e < a.cap && hops < a.cap; ++hops) {
+            const int32_t next = __ldcg(prev + e);
             if (e <= L - 2 && e >= n - 1) {
-                const bool eq = lane >= n || (e - lane >= L_old ? tail_tok(e - lane) : row[e - lane]) == mine;
-                if (__all_sync(kFull, eq)) {
-                    if (found < 0) found = e;
+                const int32_t x = lane < n ? tok(e - lane) : 0;
+                const int32_t lo = e + 1 + lane, hi = lo + 32;
+                const int32_t y_lo = lane < a.k && lo < L ? tok(lo) : 0;
+                const int32_t y_hi = lane + 32 < a.k && hi < L ? tok(hi) : 0;
+                if (__all_sync(kFull, x == mine)) {
+                    if (found < 0) {
+                        found = e;
+                        f_lo = y_lo;
+                        f_hi = y_hi;
+                    }
                     if (!collect) break;
                     if (lane == 0) s_cend[nfound] = e;
                     if (++nfound >= a.W) break;
                 }
             }
-            e = prev[e];
+            e = next;
         }
     }
     if (lane == 0 && warp < kIdxMaxWarps) s_found[warp] = found;
@@ -315,39 +370,33 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
     if (lane == 0) s_wz[warp] = zp;
     __syncthreads();
 
+    // Every thread takes the decision from shared memory (the same sums in the same order); thread 0 writes
+    // it, and the winning n's warp its draft.
+    float z = 0.f;
+    for (int w = 0; w < nwarps; ++w) z += s_wz[w];
+    if (a.z1_part != nullptr) z += a.b2;
+    int win = a.n_max - a.n_min;
+    while (win >= 0 && s_found[win] < 0) --win;
+    const bool hit = len_ok && win >= 0;
+    const int32_t nstar = win >= 0 ? a.n_min + win : 0, estar = win >= 0 ? s_found[win] : -1;
+    const bool gate = a.W > 0 ? s_ncf > 0 : nstar >= kappa_c;
+    int32_t mode = SWITCHSD_MODE_NO_REP;
+    if (hit) mode = (gate && z >= a.logit_tau) ? SWITCHSD_MODE_COPY : SWITCHSD_MODE_REP_NO_COPY;
+    const int32_t len = (a.W == 0 && mode == SWITCHSD_MODE_COPY) ? min(a.k, L - 1 - estar) : 0;
+    const int32_t nc = mode == SWITCHSD_MODE_COPY ? s_ncf : 0;  // candidate mode: candidates written
     if (tid == 0) {
-        float z = 0.f;
-        for (int w = 0; w < nwarps; ++w) z += s_wz[w];
-        if (a.z1_part != nullptr) z += a.b2;
-        int32_t nstar = 0, estar = -1;
-        for (int w = a.n_max - a.n_min; w >= 0; --w)
-            if (s_found[w] >= 0) {
-                nstar = a.n_min + w;
-                estar = s_found[w];
-                break;
-            }
-        const bool hit = len_ok && nstar > 0;
-        const bool gate = a.W > 0 ? s_ncf > 0 : nstar >= kappa_c;
-        int32_t mode = SWITCHSD_MODE_NO_REP;
-        if (hit) mode = (gate && z >= a.logit_tau) ? SWITCHSD_MODE_COPY : SWITCHSD_MODE_REP_NO_COPY;
-        const int32_t len = (a.W == 0 && mode == SWITCHSD_MODE_COPY) ? min(a.k, L - 1 - estar) : 0;
-        s_out[0] = estar;
-        s_out[1] = len;
-        s_out[2] = mode == SWITCHSD_MODE_COPY ? s_ncf : 0;  // candidate mode: candidates written
         if (a.W == 0 && a.counters)  // out_mode still holds the previous step's mode
             count_row(a.counters, mode, verifying, a.out_mode[b], s_ver[0]);
         a.out_mode[b] = mode;
         if (a.W == 0) a.out_len[b] = len;
-        else a.out_ncand[b] = s_out[2];
+        else a.out_ncand[b] = nc;
         a.out_score[b] = z;
         if (a.out_match_n) a.out_match_n[b] = nstar;
         if (a.out_match_end) a.out_match_end[b] = estar;
         if (a.status) a.status[b] = s_ver[2];
     }
-    __syncthreads();
     if (a.W > 0) {
         // The candidates' continuations x[e_w+1 .. e_w+len_w], len_w = min(D, L-1-e_w).
-        const int32_t nc = s_out[2];
         for (int t = tid; t < nc * a.D; t += blockDim.x) {
             const int w = t / a.D, i = t - w * a.D;
             const int32_t ew = s_cend[w];
@@ -358,11 +407,10 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
         }
         return;
     }
-    const int32_t e = s_out[0], len = s_out[1];
-    // The copy draft x[e+1 .. e+len]: positions below L_old are in global memory, the rest in s_tail.
-    for (int i = tid; i < len; i += blockDim.x) {
-        const int32_t p = e + 1 + i;
-        a.out_draft[size_t(b) * a.k + i] = p >= L_old ? tail_tok(p) : row[p];
+    if (warp == win) {  // the copy draft x[e+1 .. e+len], loaded with the match
+        int32_t *out = a.out_draft + size_t(b) * a.k;
+        if (lane < len) out[lane] = f_lo;
+        if (lane + 32 < len) out[lane + 32] = f_hi;
     }
 }
 
