@@ -44,10 +44,10 @@ constexpr int kKeyShift = 25;
 constexpr uint32_t kKeyEndMask = (1u << kKeyShift) - 1u;
 constexpr uint32_t kKeyTimeout = 1u << 31;
 static_assert(SWITCHSD_NMAX < (1 << (31 - kKeyShift)), "m must fit below the timeout bit");
-// The scan: kScanWords words per thread per round; a thread's rounds of a CTA range fit the 32 bits of its
+// The scan: kScanWords words per thread per round; a thread's words of a CTA range fit the 32 bits of its
 // pass mask.
 constexpr int kScanWords = 4;
-static_assert(kRescanTileMax / 4 / (kScanWords * kRescanThreads) <= 32, "a thread's rounds fit its pass mask");
+static_assert(kRescanTileMax / 4 / kRescanThreads <= 32, "a thread's words fit its pass mask");
 
 // The scan of a CTA's old ends [e_lo, e_end) against the new suffix (suf[-q] = its q-th token from the end)
 // for the longest-then-most-recent match: the largest key m << kKeyShift | e over the ends with
@@ -56,17 +56,18 @@ static_assert(kRescanTileMax / 4 / (kScanWords * kRescanThreads) <= 32, "a threa
 // Filter depth F = min(n_min, 3): end e can match only if its last F tokens equal the suffix's.  Pass 1
 // tests a hash of them, h(e) = x[e] + x[e-1] A + x[e-2] B (the first F terms, mod 2^32), against the
 // suffix's: equal tokens give equal hashes, so no end that matches is missed, and the few that collide
-// are dropped by pass 2's exact test.  Two multiply-adds per end and a running three-input min test a
-// round of sixteen ends; the shared-memory reads, not the arithmetic, set the pace.
+// are dropped by pass 2's exact test.  Two multiply-adds per end and two mins a word of four ends; the
+// shared-memory reads, not the arithmetic, set the pace.
 //
-// Pass 1: rounds of kScanWords words per thread (word g0 + u kT, g0 = tid + kScanWords kT r: consecutive
-// lanes read consecutive words), each with the two tokens before it (unset before position 0, where
-// lim < F drops the end); a round with an end that passes only sets its bit.  No branch and no backward
-// compare in the hot loop.
-// Pass 2 (rare): the rounds that passed, in warp-synchronous steps (each step every lane with a round left
+// Pass 1: rounds of kScanWords words per thread (word tid + i kT for i = 0, 1, ...: consecutive lanes read
+// consecutive words), each with the two tokens before it (unset before position 0, where lim < F drops the
+// end); a word with an end that passes sets bit i.  No branch and no backward compare in the hot loop.
+// Pass 2 (rare): the words that passed, in warp-synchronous steps (each step every lane with a word left
 // takes its next one, so the compares of a hot suffix run side by side), reloaded from shared memory;
 // their ends that pass the exact test (x[e-i] = suf[-i] for i < F) take the backward compare from m = F,
-// eight positions per step with independent loads.
+// eight positions per step with independent loads.  (A bit a round of four words instead made every step
+// of pass 2 test sixteen ends: 16 launches on the 32K rows 73.6 us against 69.7 us, 8 on the 128K rows 46.3
+// against 43.2 us.)
 constexpr uint32_t kHashA = 0x9E3779B1u, kHashB = 0x85EBCA77u;  // odd multipliers
 
 // The F-token hash of end e (x0 = x[e], x1 = x[e-1], x2 = x[e-2]; the first F terms, mod 2^32).
@@ -114,21 +115,21 @@ __device__ __forceinline__ uint32_t scan_ends(const int32_t *stage, int32_t e_lo
     const int32_t n4 = (e_end - e_lo + 3) >> 2;
     const int4 *g4 = reinterpret_cast<const int4 *>(stage + kHalo);
     const int32_t off = kHalo - e_lo;
-    uint32_t passed = 0u;
+    uint32_t passed = 0u;  // bit i: word tid + i * kRescanThreads holds an end that passes
     int rnd = 0;
     if constexpr (kPre) {
-        for (int32_t g0 = tid; g0 - lane < n4; g0 += kScanWords * kRescanThreads, ++rnd) {
-            uint32_t z = 0u;
+        for (int32_t g0 = tid; g0 - lane < n4; g0 += kScanWords * kRescanThreads, rnd += kScanWords) {
+            uint32_t hit = 0u;
 #pragma unroll
             for (int u = 0; u < kScanWords; ++u) {
                 const int32_t g = g0 + u * kRescanThreads;
-                z |= g < n4 ? has_zero_byte(hb[g] ^ hs4) : 0u;
+                if (g < n4 && has_zero_byte(hb[g] ^ hs4) != 0u) hit |= 1u << u;
             }
-            passed |= uint32_t(z != 0u) << (rnd & 31);
+            passed |= hit << (rnd & 31);
         }
     } else {
         auto hash = [&](int32_t x0, int32_t x1, int32_t x2) { return end_hash<F>(x0, x1, x2) ^ hs; };
-        for (int32_t g0 = tid; g0 - lane < n4; g0 += kScanWords * kRescanThreads, ++rnd) {
+        for (int32_t g0 = tid; g0 - lane < n4; g0 += kScanWords * kRescanThreads, rnd += kScanWords) {
             int4 v[kScanWords];
             int2 pv[kScanWords];  // x[4g - 2], x[4g - 1]
 #pragma unroll
@@ -137,14 +138,14 @@ __device__ __forceinline__ uint32_t scan_ends(const int32_t *stage, int32_t e_lo
                 v[u] = g < n4 ? g4[g] : make_int4(0, 0, 0, 0);
                 pv[u] = (F >= 2 && g < n4) ? *reinterpret_cast<const int2 *>(stage + kHalo + 4 * g - 2) : make_int2(0, 0);
             }
-            uint32_t mn = 0xffffffffu;
+            uint32_t hit = 0u;
 #pragma unroll
             for (int u = 0; u < kScanWords; ++u) {
                 const uint32_t h0 = hash(v[u].x, pv[u].y, pv[u].x), h1 = hash(v[u].y, v[u].x, pv[u].y);
                 const uint32_t h2 = hash(v[u].z, v[u].y, v[u].x), h3 = hash(v[u].w, v[u].z, v[u].y);
-                mn = __vimin3_u32(mn, __vimin3_u32(h0, h1, h2), h3);
+                if (min(__vimin3_u32(h0, h1, h2), h3) == 0u) hit |= 1u << u;
             }
-            passed |= uint32_t(mn == 0u) << (rnd & 31);
+            passed |= hit << (rnd & 31);
         }
     }
     uint32_t mine = 0u;
@@ -176,56 +177,44 @@ __device__ __forceinline__ uint32_t scan_ends(const int32_t *stage, int32_t e_lo
     };
     while (__any_sync(kFull, passed != 0u)) {
         if (passed == 0u) continue;
-        const int r = __ffs(passed) - 1;
+        const int32_t g = tid + (__ffs(passed) - 1) * kRescanThreads;
         passed &= passed - 1u;
+        if (g >= n4) continue;  // (a lane past the range read zeros)
         if constexpr (kPre) {
-            // the round's ends whose hash byte matches: bit 4u + j for end j of word u
-            uint32_t cand = 0u;
-#pragma unroll
-            for (int u = 0; u < kScanWords; ++u) {
-                const int32_t g = tid + r * kScanWords * kRescanThreads + u * kRescanThreads;
-                const uint32_t eq = g < n4 ? __vcmpeq4(hb[g], hs4) : 0u;  // 0xff in each matching byte
-                cand |= ((eq & 1u) | (eq >> 7 & 2u) | (eq >> 14 & 4u) | (eq >> 21 & 8u)) << (4 * u);
-            }
-            while (cand) {
-                const int i = __ffs(cand) - 1;
-                cand &= cand - 1u;
-                const int32_t g = tid + r * kScanWords * kRescanThreads + (i >> 2) * kRescanThreads;
-                const int32_t e = e_lo + 4 * g + (i & 3);
+            // the word's ends whose hash byte matches: the lowest byte flagged is an exact match, and is then
+            // made nonzero
+            uint32_t x = hb[g] ^ hs4;
+            for (uint32_t z = has_zero_byte(x); z != 0u; z = has_zero_byte(x)) {
+                const int j = (__ffs(z) - 1) >> 3;
+                x |= 1u << (8 * j);
+                const int32_t e = e_lo + 4 * g + j;
                 if (e >= e_end) break;
                 const int32_t lim = min(n_max, e + 1);
-                if (lim < F) continue;  // the hash read a token before position 0
-                bool ok = stage[off + e] == s0;
-                if (F >= 2) ok = ok && stage[off + e - 1] == s1;
-                if (F >= 3) ok = ok && stage[off + e - 2] == s2;
-                if (ok) take(e, match_len(e, lim));
+                const int32_t x0 = stage[off + e], x1 = F >= 2 ? stage[off + e - 1] : s1, x2 = F >= 3 ? stage[off + e - 2] : s2;
+                // (lim < F: the hash read a token before position 0)
+                if (((x0 ^ s0) | (x1 ^ s1) | (x2 ^ s2)) == 0 && lim >= F) take(e, match_len(e, lim));
             }
         } else {
-#pragma unroll 1
-            for (int u = 0; u < kScanWords; ++u) {
-                const int32_t g = tid + r * kScanWords * kRescanThreads + u * kRescanThreads;
-                if (g >= n4) break;
-                const int4 v = g4[g];
-                const int2 pv = *reinterpret_cast<const int2 *>(stage + kHalo + 4 * g - 2);
-                // exact test of the last F tokens of each end
-                const int32_t x[6] = {pv.x, pv.y, v.x, v.y, v.z, v.w};
-                uint32_t hall = 0u;
+            const int4 v = g4[g];
+            const int2 pv = *reinterpret_cast<const int2 *>(stage + kHalo + 4 * g - 2);
+            // exact test of the last F tokens of each end
+            const int32_t x[6] = {pv.x, pv.y, v.x, v.y, v.z, v.w};
+            uint32_t hall = 0u;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    bool ok = x[j + 2] == s0;
-                    if (F >= 2) ok = ok && x[j + 1] == s1;
-                    if (F >= 3) ok = ok && x[j] == s2;
-                    hall |= uint32_t(ok) << j;
-                }
-                while (hall) {
-                    const int j = __ffs(hall) - 1;
-                    hall &= hall - 1;
-                    const int32_t e = e_lo + 4 * g + j;
-                    if (e >= e_end) break;
-                    const int32_t lim = min(n_max, e + 1);
-                    if (lim < F) continue;  // the test read a token before position 0
-                    take(e, match_len(e, lim));
-                }
+            for (int j = 0; j < 4; ++j) {
+                bool ok = x[j + 2] == s0;
+                if (F >= 2) ok = ok && x[j + 1] == s1;
+                if (F >= 3) ok = ok && x[j] == s2;
+                hall |= uint32_t(ok) << j;
+            }
+            while (hall) {
+                const int j = __ffs(hall) - 1;
+                hall &= hall - 1;
+                const int32_t e = e_lo + 4 * g + j;
+                if (e >= e_end) break;
+                const int32_t lim = min(n_max, e + 1);
+                if (lim < F) continue;  // the test read a token before position 0
+                take(e, match_len(e, lim));
             }
         }
     }
