@@ -112,3 +112,41 @@ def test_long_runs_and_short_periods(n):
         L = int(lens[b])
         assert np.array_equal(got[b, :L], oracle.copy_labels(ctx[b, :L], n)), b
         assert not got[b, L:].any()
+
+
+def _first_occurrence_labels(x: np.ndarray, n: int) -> np.ndarray:
+    """Every position of one row from a dictionary of the windows' first starts (the oracle's definition, in
+    time linear in the row)."""
+    y = np.zeros(len(x), np.uint8)
+    seen = {}
+    raw = np.ascontiguousarray(x, np.int32).tobytes()
+    for s in range(len(x) - n + 1):
+        if seen.setdefault(raw[4 * s:4 * (s + n)], s) < s:
+            y[s:s + n] = 1
+    return y
+
+
+# (rows, capacity, n): one and several CTAs a row, tables of every size class, capacities that are no multiple
+# of 16, the largest capacity of the one-kernel form and the first one past it
+@pytest.mark.parametrize("B,cap,n", [(200, 3001, 5), (3, 513, 32), (40, 8209, 2), (2, 32769, 5), (70, 16389, 3),
+                                     (1, 131075, 5), (2, 262144, 7), (1, 262145, 5)])
+def test_size_classes(B, cap, n):
+    rng = np.random.default_rng(cap)
+    ctx = np.zeros((B, cap), np.int32)
+    for b in range(B):
+        kind = b % 3
+        if kind == 0:                                   # ids that differ in their high bits alone, copies
+            ctx[b] = rng.integers(-128, 128, cap) << 24
+        elif kind == 1:
+            ctx[b] = np.minimum(rng.zipf(1.2, cap), 120000)
+        else:
+            ctx[b] = np.tile(rng.integers(0, 9, 5), cap // 5 + 1)[:cap]
+        if cap > 2000:
+            ctx[b, cap - 900:] = ctx[b, 100:1000]
+    lens = rng.integers(max(1, cap - 40), cap + 1, B).astype(np.int32)
+    assert np.array_equal(_first_occurrence_labels(ctx[0, :400], n), oracle.copy_labels(ctx[0, :400], n))
+    got = _labels(ctx, lens, n)
+    for b in list(range(min(B, 6))) + [B - 1]:
+        L = int(lens[b])
+        assert np.array_equal(got[b, :L], _first_occurrence_labels(ctx[b, :L], n)), b
+        assert not got[b, L:].any()
