@@ -30,6 +30,7 @@
 // length read and waited on just before the first message, so the leader's message barrier is
 // initialised before anyone ships to it and no CTA reads the length after the leader rewrites it.
 #include <mutex>
+#include <type_traits>
 
 #include "mlp.cuh"
 #include "step.cuh"
@@ -117,37 +118,40 @@ __device__ __forceinline__ uint32_t scan_ends(const int32_t *stage, int32_t e_lo
     const int32_t off = kHalo - e_lo;
     uint32_t passed = 0u;  // bit i: word tid + i * kRescanThreads holds an end that passes
     int rnd = 0;
-    if constexpr (kPre) {
-        for (int32_t g0 = tid; g0 - lane < n4; g0 += kScanWords * kRescanThreads, rnd += kScanWords) {
-            uint32_t hit = 0u;
+    int32_t g0 = tid;
+    // One round: words g0, g0 + kT, ...; kAll: every lane's words lie in the range (the hot rounds: no
+    // predicates, one base address), else the words past it read as no match.
+    auto round = [&](auto all) {
+        constexpr bool kAll = decltype(all)::value;
+        uint32_t hit = 0u;
+        if constexpr (kPre) {
+            const uint32_t *w = hb + g0;
 #pragma unroll
-            for (int u = 0; u < kScanWords; ++u) {
-                const int32_t g = g0 + u * kRescanThreads;
-                if (g < n4 && has_zero_byte(hb[g] ^ hs4) != 0u) hit |= 1u << u;
-            }
-            passed |= hit << (rnd & 31);
-        }
-    } else {
-        auto hash = [&](int32_t x0, int32_t x1, int32_t x2) { return end_hash<F>(x0, x1, x2) ^ hs; };
-        for (int32_t g0 = tid; g0 - lane < n4; g0 += kScanWords * kRescanThreads, rnd += kScanWords) {
+            for (int u = 0; u < kScanWords; ++u)
+                if ((kAll || g0 + u * kRescanThreads < n4) && has_zero_byte(w[u * kRescanThreads] ^ hs4) != 0u) hit |= 1u << u;
+        } else {
+            const int4 *w = g4 + g0;
             int4 v[kScanWords];
             int2 pv[kScanWords];  // x[4g - 2], x[4g - 1]
 #pragma unroll
             for (int u = 0; u < kScanWords; ++u) {
-                const int32_t g = g0 + u * kRescanThreads;
-                v[u] = g < n4 ? g4[g] : make_int4(0, 0, 0, 0);
-                pv[u] = (F >= 2 && g < n4) ? *reinterpret_cast<const int2 *>(stage + kHalo + 4 * g - 2) : make_int2(0, 0);
+                const bool in = kAll || g0 + u * kRescanThreads < n4;
+                v[u] = in ? w[u * kRescanThreads] : make_int4(0, 0, 0, 0);
+                pv[u] = (F >= 2 && in) ? reinterpret_cast<const int2 *>(w + u * kRescanThreads)[-1] : make_int2(0, 0);
             }
-            uint32_t hit = 0u;
 #pragma unroll
             for (int u = 0; u < kScanWords; ++u) {
-                const uint32_t h0 = hash(v[u].x, pv[u].y, pv[u].x), h1 = hash(v[u].y, v[u].x, pv[u].y);
-                const uint32_t h2 = hash(v[u].z, v[u].y, v[u].x), h3 = hash(v[u].w, v[u].z, v[u].y);
-                if (min(__vimin3_u32(h0, h1, h2), h3) == 0u) hit |= 1u << u;
+                const uint32_t h0 = end_hash<F>(v[u].x, pv[u].y, pv[u].x), h1 = end_hash<F>(v[u].y, v[u].x, pv[u].y);
+                const uint32_t h2 = end_hash<F>(v[u].z, v[u].y, v[u].x), h3 = end_hash<F>(v[u].w, v[u].z, v[u].y);
+                if ((h0 == hs) | (h1 == hs) | (h2 == hs) | (h3 == hs)) hit |= 1u << u;
             }
-            passed |= hit << (rnd & 31);
         }
-    }
+        passed |= hit << (rnd & 31);
+        g0 += kScanWords * kRescanThreads;
+        rnd += kScanWords;
+    };
+    while (g0 - lane + (kScanWords - 1) * kRescanThreads + kWarp <= n4) round(std::true_type{});
+    while (g0 - lane < n4) round(std::false_type{});
     uint32_t mine = 0u;
     // m(e) from F for an end whose last F tokens match: x[e - q] against suf[-q], eight positions per step,
     // every load issued unconditionally (q clamped to lim - 1; the sentinel bit ends the run at the count)
