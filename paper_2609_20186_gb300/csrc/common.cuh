@@ -213,7 +213,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity
 }
 
 // Launches `kernel` on `stream` with programmatic stream serialization and, when cluster_x >= 1, an
-// explicit cluster shape of cluster_x CTAs (1 included: the cluster instructions of the step kernel,
+// explicit cluster shape of cluster_x CTAs (1 included: the cluster instructions of the rescan kernel,
 // st.async into shared::cluster in particular, need an explicit cluster launch).
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
@@ -254,15 +254,6 @@ __device__ __forceinline__ void count_row(unsigned long long *ctr, int32_t mode,
 
 __device__ __forceinline__ float bf16_lo(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
-
-__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        unsigned long long w = __shfl_xor_sync(kFull, v, o);
-        v = w > v ? w : v;
-    }
-    return v;
-}
 
 __device__ __forceinline__ float warp_sum_f32(float v) {
 #pragma unroll

@@ -105,11 +105,13 @@ __device__ __forceinline__ void hash_ends(const int32_t *stage, uint32_t *hb, in
 // one byte per end against the suffix's (four ends a 4-byte load), and pass 2 takes only the ends whose
 // byte matches.  The byte filter passes every end that matches and about 1 in 256 of the others, which
 // the exact test drops.
+//
+// The key holds e - key0, the bitmap starts at end bm_lo (a ring of tiles scans one tile at a time: e_lo is
+// then the tile's first end).
 template <int F, bool kCand, bool kPre>
 __device__ __forceinline__ uint32_t scan_ends(const int32_t *stage, int32_t e_lo, int32_t e_end, const int32_t *suf,
-                                              int32_t n_min, int32_t n_max, int tid, int lane,
-                                              uint32_t *bm = nullptr, int32_t kappa_c = 0,
-                                              const uint32_t *hb = nullptr) {
+                                              int32_t n_min, int32_t n_max, int tid, int lane, uint32_t *bm,
+                                              int32_t kappa_c, const uint32_t *hb, int32_t key0, int32_t bm_lo) {
     const int32_t s0 = suf[0], s1 = F >= 2 ? suf[-1] : 0, s2 = F >= 3 ? suf[-2] : 0;
     const uint32_t hs = end_hash<F>(s0, s1, s2);
     const uint32_t hs4 = hash_byte(hs) * 0x01010101u;
@@ -174,10 +176,10 @@ __device__ __forceinline__ uint32_t scan_ends(const int32_t *stage, int32_t e_lo
     };
     auto take = [&](int32_t e, int32_t m) {
         if (m >= n_min) {
-            const uint32_t key = (uint32_t(m) << kKeyShift) | uint32_t(e);
+            const uint32_t key = (uint32_t(m) << kKeyShift) | uint32_t(e - key0);
             mine = key > mine ? key : mine;
         }
-        if (kCand && m >= kappa_c) atomicOr(&bm[(e - e_lo) >> 5], 1u << ((e - e_lo) & 31));
+        if (kCand && m >= kappa_c) atomicOr(&bm[(e - bm_lo) >> 5], 1u << ((e - bm_lo) & 31));
     };
     while (__any_sync(kFull, passed != 0u)) {
         if (passed == 0u) continue;
@@ -228,7 +230,8 @@ __device__ __forceinline__ uint32_t scan_ends(const int32_t *stage, int32_t e_lo
 constexpr int kVerifyLoads = 4;  // candidate verification: staging loads a thread has in flight at once
 
 // Candidate mode's shared memory beyond the single-draft layout: per CTA one candidate message of cslot
-// bytes -- a 16-byte header (count), the ends (W, most recent first), their continuations [W][D] -- the
+// bytes -- a 16-byte header (count), the ends (W, most recent first), their continuations [W][D] (not from
+// a ring, whose tiles are gone by then: the leader reads them from the row) -- the
 // leader receiving C of them and every CTA staging its own; a bitmap of the CTA's marked ends; the
 // verification's staging of the previous candidates (drafts [W][D], targets [W][D+1], lengths [W], count).
 struct CandLayout {
@@ -236,19 +239,30 @@ struct CandLayout {
     int bm_words;    // bitmap words (a multiple of 4)
     int v_ints;      // verification staging (a multiple of 4)
 };
-__host__ __device__ inline CandLayout cand_layout(int tile, int W, int D) {
+__host__ __device__ inline CandLayout cand_layout(int range, int W, int D, bool ring) {
     CandLayout c;
-    c.cslot = 16u * uint32_t(1 + (W + 3) / 4 + (W * D + 3) / 4);
-    c.bm_words = ((tile + 31) / 32 + 3) & ~3;
+    c.cslot = 16u * uint32_t(1 + (W + 3) / 4 + (ring ? 0 : (W * D + 3) / 4));
+    c.bm_words = ((range + 31) / 32 + 3) & ~3;
     c.v_ints = (W * D + W * (D + 1) + W + 1 + 3) & ~3;
     return c;
 }
 
-// kPre: the pre-wait hash table (a.hash_words > 0); kMlp: the two-layer probe's finish (a.z1_part set).
+// kScan: how a CTA's old ends are staged and scanned -- one copy, filtered on the tokens (kScanTokens) or on
+// the pre-wait hash bytes (kScanHashed, a.hash_words > 0); or, for ranges above kRescanTileMax ends, a ring
+// of a.stages tiles filtered on the tokens (kScanRing).  kMlp: the two-layer probe's finish (a.z1_part set).
 // Separate instances, so that each carries only its own scan and its own probe code and registers.
-template <bool kSampled, bool kCand, bool kPre, bool kMlp>
-__global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_kernel(const StepArgs a) {
+//
+// The ring: every warp scans its share of each tile as it lands, keeps its best match's continuation while
+// that tile is staged, and counts itself out of the stage; the last warp out refills it.  No CTA barrier and
+// no producer warp: the warps drift by up to the ring's depth.
+enum { kScanTokens = 0, kScanHashed = 1, kScanRing = 2 };
+template <bool kSampled, bool kCand, int kScan, bool kMlp>
+__global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaunchBlocks : kRescanLaunchBlocks)
+    rescan_kernel(const StepArgs a) {
+    constexpr bool kPre = kScan == kScanHashed, kRing = kScan == kScanRing;
     extern __shared__ __align__(128) int32_t dsm[];
+    __shared__ __align__(8) uint64_t ring[kRing ? kRingStages : 1];  // a tile of the ring landed
+    __shared__ int s_out_of[kRing ? kRingStages : 1];                // warps done with a stage, counted on and on
     __shared__ __align__(8) uint64_t bars[5];              // tile, tail, probe slices, messages (leader),
                                                            // pre-wait hashes
     __shared__ __align__(16) int32_t s_tail[kHalo + 8];    // x[tail_lo .. L_old), tail_lo = roundown4(L_old - kHalo)
@@ -264,7 +278,7 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
     const int b = blockIdx.y;
     const int stage_ints = kHalo + a.tile + kFwd;
     int32_t *stage = dsm;
-    uint32_t *hb = reinterpret_cast<uint32_t *>(dsm + ((stage_ints + 3) & ~3));  // [hash_words]
+    uint32_t *hb = reinterpret_cast<uint32_t *>(dsm + (kRing ? a.stages : 1) * ((stage_ints + 3) & ~3));  // [hash_words]
     uint4 *s_pw = reinterpret_cast<uint4 *>(hb + a.hash_words);
     uint4 *s_ph = s_pw + a.probe_words;
     unsigned char *msgs = reinterpret_cast<unsigned char *>(s_ph + a.probe_words);
@@ -272,7 +286,7 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
     const int kw = kCand ? 0 : (a.k + 3) >> 2;             // 16-byte words of a message's continuation
     const uint32_t slot_bytes = 16u * uint32_t(1 + kw);
     const int nmsg = int(C) * kRescanWarps;
-    const CandLayout cl = cand_layout(kCand ? a.tile : 0, kCand ? a.W : 0, kCand ? a.D : 0);
+    const CandLayout cl = cand_layout(kCand ? a.range : 0, kCand ? a.W : 0, kCand ? a.D : 0, kRing);
     unsigned char *cmsgs = msgs + size_t(nmsg) * slot_bytes;                  // [C][cslot] (leader)
     unsigned char *cstage = cmsgs + size_t(C) * cl.cslot;                     // this CTA's message
     uint32_t *bm = reinterpret_cast<uint32_t *>(cstage + cl.cslot);           // [bm_words]
@@ -285,6 +299,11 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
         mbar_init(&bars[1], 1);
         mbar_init(&bars[2], 1);
         mbar_init(&bars[4], kRescanThreads - kWarp);
+        if (kRing)
+            for (int s = 0; s < a.stages; ++s) {
+                mbar_init(&ring[s], 1);
+                s_out_of[s] = 0;
+            }
         if (rank == lead) {
             mbar_init(&bars[3], 1);
             mbar_arrive_expect_tx(&bars[3], slot_bytes * uint32_t(nmsg) + (kCand ? cl.cslot * C : 0u));
@@ -324,7 +343,20 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
     }
     auto tile_hi = [&]() { return e_hi > e_lo ? min((e_hi + kFwd + 3) & ~3, a.cap) : lo; };
     const uint64_t pol = l2_evict_first_policy();
+    // Ring: tile t of the range (ends [t0, t0 + a.tile)) into stage s = t mod a.stages, x[p] at [kHalo + p - t0].
+    auto issue_ring = [&](int t, int s) {
+        const int32_t t0 = e_lo + t * a.tile, t1 = min(e_hi, t0 + a.tile);
+        const int32_t lo_t = max(0, t0 - kHalo), hi_t = min((t1 + kFwd + 3) & ~3, a.cap);
+        const uint32_t bytes = uint32_t(hi_t - lo_t) * 4u;
+        mbar_expect_tx_relaxed(&ring[s], bytes);
+        bulk_g2s_hint(stage + s * stage_ints + (kHalo + lo_t - t0), row + lo_t, bytes, &ring[s], pol);
+    };
+    auto ring_tiles = [&]() { return e_hi > e_lo ? (e_hi - e_lo - 1) / a.tile + 1 : 0; };
     auto issue_tile = [&](int32_t hi_) {  // positions [lo, hi_) land at stage[kHalo + p - e_lo]
+        if (kRing) {
+            for (int t = 0; t < min(ring_tiles(), a.stages); ++t) issue_ring(t, t);
+            return;
+        }
         const uint32_t bytes = uint32_t(hi_ - lo) * 4u;
         mbar_expect_tx_relaxed(&bars[0], bytes);
         if (bytes > 0) bulk_g2s_hint(stage + (kHalo + lo - e_lo), row + lo, bytes, &bars[0], pol);
@@ -584,18 +616,78 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
     // key = m << kKeyShift | e (e < 2^kKeyShift, m <= 32): the largest key is the longest match, then the
     // most recent; 0 = no match; kKeyTimeout marks a copy that did not land.
     uint32_t mine = 0;
-    const bool tile_in = hi == lo || mbar_wait(&bars[0], 0);
+    const bool tile_in = kRing || hi == lo || mbar_wait(&bars[0], 0);
     const bool hashed = !pre || mbar_wait(&bars[4], 0);
     bool timed_out = !tail_in || !tile_in || !hashed;
     const int32_t off = kHalo - e_lo;  // stage[off + p] = x[p] over the staged range
-    if (!timed_out && len_ok && L >= 2) {
-        // (n_min and kappa are uniform over the launch: one instance runs)
-        // the filter depth may test no more than a candidate needs (fdepth <= kappa in candidate mode)
+    // (n_min and kappa are uniform over the launch: one instance runs)
+    // the filter depth may test no more than a candidate needs (fdepth <= kappa in candidate mode)
+    auto scan = [&](const int32_t *st, int32_t lo_e, int32_t end_e, int32_t key0) {
         const int fdepth = filter_depth();
-        mine = fdepth >= 3 ? scan_ends<3, kCand, kPre>(stage, e_lo, e_end, suf, n_min, n_max, tid, lane, bm, kappa_c, hb)
-                           : (fdepth == 2
-                                  ? scan_ends<2, kCand, kPre>(stage, e_lo, e_end, suf, n_min, n_max, tid, lane, bm, kappa_c, hb)
-                                  : scan_ends<1, kCand, kPre>(stage, e_lo, e_end, suf, n_min, n_max, tid, lane, bm, kappa_c, hb));
+        return fdepth >= 3
+                   ? scan_ends<3, kCand, kPre>(st, lo_e, end_e, suf, n_min, n_max, tid, lane, bm, kappa_c, hb, key0, e_lo)
+                   : (fdepth == 2 ? scan_ends<2, kCand, kPre>(st, lo_e, end_e, suf, n_min, n_max, tid, lane, bm, kappa_c,
+                                                              hb, key0, e_lo)
+                                  : scan_ends<1, kCand, kPre>(st, lo_e, end_e, suf, n_min, n_max, tid, lane, bm, kappa_c,
+                                                              hb, key0, e_lo));
+    };
+    // the continuation of a match ending at e: lane j (1..kw) gathers tokens 4(j-1) .. +3, from the staged
+    // tile (tl[o_ + p] = x[p]) or past the old length from this warp's window
+    uint4 cw = make_uint4(0, 0, 0, 0);
+    auto gather_next = [&](int32_t e, const int32_t *tl, int32_t o_) {
+        if (lane < 1 || lane > kw) return;
+        const int32_t len = min(a.k, L - 1 - e);
+        int32_t t4[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int32_t i = 4 * (lane - 1) + q;
+            const int32_t p = e + 1 + i;
+            t4[q] = i < len ? (p < L_old ? tl[o_ + p] : y[kHalo + p - L_old]) : 0;
+        }
+        cw = make_uint4(uint32_t(t4[0]), uint32_t(t4[1]), uint32_t(t4[2]), uint32_t(t4[3]));
+    };
+    // ring: this warp's best match so far (m_b = 0: none), warp-uniform; its continuation is in cw
+    int32_t m_b = 0, e_b = -1;
+    if constexpr (kRing) {
+        const int nt = ring_tiles();
+        int s = 0;
+        uint32_t phase = 0u;
+        for (int t = 0; t < nt; ++t) {
+            if (!__all_sync(kFull, mbar_wait(&ring[s], phase))) {
+                timed_out = true;
+                // copies still in flight get a second bounded wait before the CTA's memory goes away
+                if (lane == 0)
+                    for (int u = t; u < min(nt, t + a.stages); ++u)
+                        (void)mbar_wait(&ring[u % a.stages], uint32_t(u / a.stages) & 1u);
+                break;
+            }
+            const int32_t t0 = e_lo + t * a.tile;
+            const int32_t *tl = stage + s * stage_ints;
+            uint32_t k_t = 0u;
+            if (tail_in && len_ok && t0 < e_end) k_t = scan(tl, t0, min(e_end, t0 + a.tile), t0);
+            k_t = __reduce_max_sync(kFull, k_t);
+            if (k_t != 0u && int32_t(k_t >> kKeyShift) >= m_b) {  // a later tile's ends are the more recent
+                m_b = int32_t(k_t >> kKeyShift);
+                e_b = t0 + int32_t(k_t & kKeyEndMask);
+                gather_next(e_b, tl, kHalo - t0);
+            }
+            __syncwarp();
+            if (lane == 0 && t + a.stages < nt) {
+                __threadfence_block();  // this warp's reads of the stage, before the last warp out refills it
+                if ((atomicAdd(&s_out_of[s], 1) + 1) % kRescanWarps == 0) {
+                    __threadfence_block();
+                    fence_proxy_async();
+                    issue_ring(t + a.stages, s);
+                }
+            }
+            if (++s == a.stages) {
+                s = 0;
+                phase ^= 1u;
+            }
+        }
+    }
+    if (!timed_out && len_ok && L >= 2) {
+        if (!kRing) mine = scan(stage, e_lo, e_end, 0);
         // The ends the append creates, [L_old - 1, L - 1), lie in the window: the leader's warp 0.  In
         // candidate mode new_c[t] bit i marks end L_old - 1 + 32 t + i as a candidate (warp-uniform).
         if (kCand && rank == lead && warp == 0 && acc >= 0) {
@@ -610,7 +702,7 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
 #pragma unroll 1
                     while (m < lim && y[kHalo - 1 + j - m] == suf[-m]) ++m;
                     if (m >= n_min) {
-                        const uint32_t key = (uint32_t(m) << kKeyShift) | uint32_t(e);
+                        const uint32_t key = (uint32_t(m) << kKeyShift) | uint32_t(kRing ? j : e);
                         mine = key > mine ? key : mine;
                     }
                     qual = m >= kappa_c;
@@ -626,13 +718,22 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
 #pragma unroll 1
                 while (m < lim && y[kHalo - 1 + j - m] == suf[-m]) ++m;
                 if (m >= n_min) {
-                    const uint32_t key = (uint32_t(m) << kKeyShift) | uint32_t(e);
+                    const uint32_t key = (uint32_t(m) << kKeyShift) | uint32_t(kRing ? j : e);
                     mine = key > mine ? key : mine;
                 }
             }
         }
     }
     uint32_t key = __reduce_max_sync(kFull, mine);
+    if constexpr (kRing) {
+        // the appended ends (the leader's warp 0) are more recent than every old one
+        if (key != 0u && int32_t(key >> kKeyShift) >= m_b) {
+            m_b = int32_t(key >> kKeyShift);
+            e_b = L_old - 1 + int32_t(key & kKeyEndMask);
+            gather_next(e_b, stage, 0);  // every token of it is in the window
+        }
+        key = uint32_t(m_b) << kKeyShift;  // the message carries the end beside it
+    }
     if (timed_out) key = kKeyTimeout;
 
     // ---- candidate mode: this CTA's W most recent marked ends and their continuations (warp 0) ----
@@ -682,7 +783,7 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
             if (lane < nsel) ce[lane] = s_sel[lane];
             const int dw = kWarp / a.D, di = kWarp - dw * a.D;  // (candidate, token) step of 32 slots
             int w = lane / a.D, i = lane - w * a.D;
-            for (int t = lane; t < nsel * a.D; t += kWarp) {
+            for (int t = lane; !kRing && t < nsel * a.D; t += kWarp) {  // (the ring's tiles are gone)
                 const int32_t ew = s_sel[w];
                 const int32_t p = ew + 1 + i;
                 ct[t] = i < min(a.D, L - 1 - ew) ? (p < L_old ? stage[off + p] : y[kHalo + p - L_old]) : 0;
@@ -716,20 +817,8 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
     if (!probe_ok) key = kKeyTimeout;
     const float z_w = warp_sum_f32(zp);
 
-    // ---- the continuation of this warp's best match: lane j (1..kw) gathers tokens 4(j-1) .. +3 ----
-    uint4 cw = make_uint4(0, 0, 0, 0);
-    if (key != 0u && key != kKeyTimeout && lane >= 1 && lane <= kw) {
-        const int32_t e = int32_t(key & kKeyEndMask);
-        const int32_t len = min(a.k, L - 1 - e);
-        int32_t t4[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int32_t i = 4 * (lane - 1) + q;
-            const int32_t p = e + 1 + i;
-            t4[q] = i < len ? (p < L_old ? stage[off + p] : y[kHalo + p - L_old]) : 0;
-        }
-        cw = make_uint4(uint32_t(t4[0]), uint32_t(t4[1]), uint32_t(t4[2]), uint32_t(t4[3]));
-    }
+    // ---- the continuation of this warp's best match (the ring has it already) ----
+    if (!kRing && key != 0u && key != kKeyTimeout) gather_next(int32_t(key & kKeyEndMask), stage, off);
 
     // ---- ship to the leader ----
     cluster_wait_acquire();  // every CTA has read the length and the leader's barrier is initialised
@@ -739,7 +828,7 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
         uint4 h;
         h.x = key;
         h.y = __float_as_uint(z_w);
-        h.z = 0u;
+        h.z = uint32_t(e_b);
         h.w = 0u;
         st_async_v4(map_to_rank(slot, lead), h, done_addr);
     } else if (lane <= kw) {
@@ -750,7 +839,7 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
     if (rank != lead || warp != 0) {
         if (kCand && warp == 0 && lane == 0) bulk_wait_read();  // the message has been read out
         if (timed_out && lane == 0) {  // copies still in flight get a second bounded wait
-            (void)mbar_wait(&bars[0], 0);
+            if (!kRing) (void)mbar_wait(&bars[0], 0);
             (void)mbar_wait(&bars[1], 0);
         }
         if (!probe_ok && lane == 0) (void)mbar_wait(&bars[2], 0);
@@ -766,28 +855,30 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
         }
     }
     const bool all_in = __all_sync(kFull, mbar_wait_polls(&bars[3], 0, a.msg_wait_polls));
-    uint32_t k_r = 0u;
+    uint32_t k_r = 0u, e_r = 0u;
     int32_t i_r = 0;
     float z_r = 0.f;
     if (all_in) {
         for (int i = lane; i < nmsg; i += kWarp) {  // lane j: messages j, j + 32, ... in order
-            const uint2 hv = *reinterpret_cast<const uint2 *>(msgs + size_t(i) * slot_bytes);
+            const uint4 hv = *reinterpret_cast<const uint4 *>(msgs + size_t(i) * slot_bytes);
             z_r += __uint_as_float(hv.y);
-            if (hv.x > k_r) {
+            if (hv.x > k_r || (kRing && hv.x == k_r && hv.x != 0u && hv.z > e_r)) {
                 k_r = hv.x;
+                e_r = hv.z;
                 i_r = i;
             }
         }
     }
     const uint32_t best = all_in ? __reduce_max_sync(kFull, k_r) : kKeyTimeout;
-    const unsigned at = __ballot_sync(kFull, k_r == best);
+    // ring: the keys hold the lengths alone, the most recent end decides among them
+    const uint32_t best_e = kRing ? __reduce_max_sync(kFull, k_r == best ? e_r : 0u) : 0u;
+    const unsigned at = __ballot_sync(kFull, k_r == best && (!kRing || e_r == best_e));
     const int32_t win = __shfl_sync(kFull, i_r, at != 0u ? __ffs(at) - 1 : 0);
     const float z = warp_sum_f32(z_r) + (mlp ? a.b2 : 0.f);
     const bool timeout = best == kKeyTimeout;
     const bool hit = len_ok && !timeout && best != 0u;
     const int32_t n = hit ? int32_t(best >> kKeyShift) : 0;
-    const int32_t e = hit ? int32_t(best & kKeyEndMask) : -1;
-    const int32_t kappa = a.kappa > 0 ? a.kappa : a.n_min;
+    const int32_t e = hit ? int32_t(kRing ? best_e : best & kKeyEndMask) : -1;
     if constexpr (kCand) {
         // The row's candidates, most recent first: the appended ends (highest first), then the CTAs' lists
         // from the leader's (the most recent range) down to CTA 0's.  s_sel[w] is merged candidate w's
@@ -850,6 +941,9 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
                 int32_t tok;
                 if (src < 0) {
                     tok = y[kHalo + ew + 1 + i - L_old];
+                } else if (kRing) {
+                    const int32_t p = ew + 1 + i;
+                    tok = p < L_old ? __ldcg(row + p) : y[kHalo + p - L_old];
                 } else {
                     const int r = src / kMaxCand;
                     tok = reinterpret_cast<const int32_t *>(cmsgs + size_t(r) * cl.cslot + 16 + 16 * cwE)
@@ -898,7 +992,7 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
     }
     if (!all_in && lane == 0) (void)mbar_wait(&bars[3], 0);  // messages still in flight: a second bounded wait
     if (timed_out && lane == 0) {
-        (void)mbar_wait(&bars[0], 0);
+        if (!kRing) (void)mbar_wait(&bars[0], 0);
         (void)mbar_wait(&bars[1], 0);
     }
     if (!probe_ok && lane == 0) (void)mbar_wait(&bars[2], 0);
@@ -906,42 +1000,42 @@ __global__ void __launch_bounds__(kRescanThreads, kRescanLaunchBlocks) rescan_ke
 
 size_t rescan_smem_bytes(const StepArgs &args, int split) {
     const bool cand = args.W > 0;
-    const size_t stage = size_t((kHalo + args.tile + kFwd + 3) & ~3) * sizeof(int32_t);
+    const size_t stage = size_t(args.stages) * size_t((kHalo + args.tile + kFwd + 3) & ~3) * sizeof(int32_t);
     const size_t probe = 2 * size_t(args.probe_words) * 16 + size_t(args.hash_words) * 4;
     const size_t msgs = size_t(split) * kRescanWarps * 16 * size_t(1 + (cand ? 0 : ((args.k + 3) >> 2)));
     if (!cand) return stage + probe + msgs;
-    const CandLayout c = cand_layout(args.tile, args.W, args.D);
+    const CandLayout c = cand_layout(args.range, args.W, args.D, args.ring != 0);
     return stage + probe + msgs + size_t(split + 1) * c.cslot + size_t(c.bm_words + c.v_ints) * sizeof(int32_t);
 }
 
-template <bool kSampled, bool kCand, bool kPre, bool kMlp>
+template <bool kSampled, bool kCand, int kScan, bool kMlp>
 static cudaError_t rescan_attrs() {
     static bool attr_done[64] = {false};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(rescan_kernel<kSampled, kCand, kPre, kMlp>,
+        cudaError_t e = cudaFuncSetAttribute(rescan_kernel<kSampled, kCand, kScan, kMlp>,
                                              cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(rescan_kernel<kSampled, kCand, kPre, kMlp>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 int(kRescanSmemBudget));
+        e = cudaFuncSetAttribute(rescan_kernel<kSampled, kCand, kScan, kMlp>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 int(kScan == kScanRing ? kRingSmemBudget : kRescanSmemBudget));
         if (e != cudaSuccess) return e;
         attr_done[dev] = true;
     }
     return cudaSuccess;
 }
 
-template <bool kSampled, bool kCand, bool kPre, bool kMlp>
+template <bool kSampled, bool kCand, int kScan, bool kMlp>
 static cudaError_t launch_rescan(const StepArgs &args, int split, cudaStream_t stream) {
-    const cudaError_t e = rescan_attrs<kSampled, kCand, kPre, kMlp>();
+    const cudaError_t e = rescan_attrs<kSampled, kCand, kScan, kMlp>();
     if (e != cudaSuccess) return e;
-    return launch_pdl(rescan_kernel<kSampled, kCand, kPre, kMlp>, dim3(unsigned(split), unsigned(args.B), 1),
+    return launch_pdl(rescan_kernel<kSampled, kCand, kScan, kMlp>, dim3(unsigned(split), unsigned(args.B), 1),
                       dim3(kRescanThreads, 1, 1), rescan_smem_bytes(args, split), stream, unsigned(split), args);
 }
 
 // Resident CTAs per SM of an instance at a dynamic shared-memory size (cached: the occupancy calculator
 // runs once per instance, device and size).
-template <bool kSampled, bool kCand, bool kPre, bool kMlp>
+template <bool kSampled, bool kCand, int kScan, bool kMlp>
 static cudaError_t rescan_per_sm(size_t smem, int &out) {
     struct Entry {
         int dev;
@@ -961,10 +1055,10 @@ static cudaError_t rescan_per_sm(size_t smem, int &out) {
                 return cudaSuccess;
             }
     }
-    cudaError_t e = rescan_attrs<kSampled, kCand, kPre, kMlp>();
+    cudaError_t e = rescan_attrs<kSampled, kCand, kScan, kMlp>();
     if (e != cudaSuccess) return e;
     int n = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, rescan_kernel<kSampled, kCand, kPre, kMlp>, kRescanThreads, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, rescan_kernel<kSampled, kCand, kScan, kMlp>, kRescanThreads, smem);
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lk(mu);
     if (used < 32) cache[used++] = Entry{dev, smem, n};
@@ -981,13 +1075,13 @@ static cudaError_t choose_hash(StepArgs &args, int split, int sms) {
     // launch with it, the 32K rows (512 CTAs) gain 0.1 us and the 128K rows (256 CTAs of 8.5K ends) 0.8 us.
     if (int64_t(split) * args.B < int64_t(sms)) return cudaSuccess;
     int without = 0, with = 0;
-    cudaError_t e = rescan_per_sm<kSampled, kCand, false, kMlp>(rescan_smem_bytes(args, split), without);
+    cudaError_t e = rescan_per_sm<kSampled, kCand, kScanTokens, kMlp>(rescan_smem_bytes(args, split), without);
     if (e != cudaSuccess) return e;
     StepArgs h = args;
     h.hash_words = words;
     const size_t bytes = rescan_smem_bytes(h, split);
     if (bytes > kRescanSmemBudget) return cudaSuccess;
-    e = rescan_per_sm<kSampled, kCand, true, kMlp>(bytes, with);
+    e = rescan_per_sm<kSampled, kCand, kScanHashed, kMlp>(bytes, with);
     if (e != cudaSuccess) return e;
     if (with >= 1 && with >= (without < kRescanMinBlocks ? without : kRescanMinBlocks)) args.hash_words = words;
     return cudaSuccess;
@@ -1005,14 +1099,17 @@ cudaError_t rescan_choose_hash(StepArgs &args, int split, int sms) {
                                 : choose_hash2<false, false>(args, split, sms);
 }
 
+template <bool kSampled, bool kCand, bool kMlp>
+static cudaError_t launch_rescan3(const StepArgs &args, int split, cudaStream_t stream) {
+    if (args.ring) return launch_rescan<kSampled, kCand, kScanRing, kMlp>(args, split, stream);
+    return args.hash_words > 0 ? launch_rescan<kSampled, kCand, kScanHashed, kMlp>(args, split, stream)
+                               : launch_rescan<kSampled, kCand, kScanTokens, kMlp>(args, split, stream);
+}
+
 template <bool kSampled, bool kCand>
 static cudaError_t launch_rescan2(const StepArgs &args, int split, cudaStream_t stream) {
-    const bool mlp = args.z1_part != nullptr;
-    if (args.hash_words > 0)
-        return mlp ? launch_rescan<kSampled, kCand, true, true>(args, split, stream)
-                   : launch_rescan<kSampled, kCand, true, false>(args, split, stream);
-    return mlp ? launch_rescan<kSampled, kCand, false, true>(args, split, stream)
-               : launch_rescan<kSampled, kCand, false, false>(args, split, stream);
+    return args.z1_part != nullptr ? launch_rescan3<kSampled, kCand, true>(args, split, stream)
+                                 : launch_rescan3<kSampled, kCand, false>(args, split, stream);
 }
 
 cudaError_t launch_rescan_kernel(const StepArgs &args, int split, cudaStream_t stream) {

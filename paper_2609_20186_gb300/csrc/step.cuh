@@ -1,4 +1,4 @@
-// step.cuh -- the step kernel's constants, arguments and launcher (step.cu), shared with the entry
+// step.cuh -- the rescan kernel's constants, arguments and launcher (rescan.cu), shared with the entry
 // points (step_api.cu).
 #pragma once
 
@@ -6,16 +6,9 @@
 
 namespace switchsd {
 
-constexpr int kStepThreads = 256;
-constexpr int kStepWarps = kStepThreads / kWarp;
-constexpr int kTileMax = 8192;        // tile of the ring of stages, for ranges above kSingleTileMax
-constexpr int kSingleTileMax = 16384; // a CTA range up to this many ends is staged by one copy
 constexpr int kHalo = 32;             // look-back staged before a tile: >= SWITCHSD_NMAX, multiple of 4
 constexpr int kFwd = SWITCHSD_KMAX;   // look-ahead staged after a tile: the longest copy draft
-constexpr int kMaxStages = 6;          // staged tiles in flight per CTA (bounded by shared memory)
-constexpr size_t kStageSmemBudget = 200 * 1024;
 constexpr int kMaxSplit = 16;
-constexpr unsigned long long kTimeoutBit = 1ull << 62;
 constexpr int kMaxCand = SWITCHSD_WMAX; // candidate mode: largest W
 constexpr int kProbeStage = 256;      // probe words (8 bf16) of w and of h staged per CTA; the rest is read directly
 // The rescan kernel (rescan.cu): four warps, at most 64 registers a thread (eight CTAs' worth of an SM's
@@ -27,10 +20,19 @@ constexpr int kRescanMinBlocks = 7;
 constexpr int kRescanLaunchBlocks = 8;  // the launch bound: 65,536 / (8 x 128) = 64 registers a thread
 constexpr int kRescanTileMax = 16384;  // largest CTA range of the rescan kernel (one bulk copy)
 constexpr size_t kRescanSmemBudget = 100 * 1024;
-constexpr int kRescanCapMax = 1 << 25;  // the rescan kernel's match keys hold an end below 2^25
+constexpr int kRescanCapMax = 1 << 25;  // one copy a range: the match keys hold an end below 2^25
+// The ring instance, for larger ranges: tiles of a CTA's range in flight, the launch bound (six CTAs an SM,
+// 80 registers a thread), the largest tile, and the shared memory a CTA may take.
+constexpr int kRingStages = 4;
+constexpr int kRingLaunchBlocks = 6;
+constexpr int kRingTileMin = 1024, kRingTileMax = 8192;
+constexpr size_t kRingSmemBudget = 222 * 1024;
+constexpr int kRingCtas = 3;              // CTAs an SM the ring's split aims at
+constexpr int kSmSharedBytes = 228 * 1024;  // an SM's shared memory, and what a CTA takes beside the dynamic part
+constexpr int kCtaSharedReserve = 3 * 1024 + 256;
 
 static_assert(kHalo >= SWITCHSD_NMAX && kHalo % 4 == 0, "halo must cover the longest n-gram");
-static_assert(kFwd % 4 == 0 && kTileMax % 4 == 0, "stages must stay 16-byte aligned");
+static_assert(kFwd % 4 == 0 && kRingTileMax % 4 == 0, "stages must stay 16-byte aligned");
 
 struct StepArgs {
     int32_t *ctx;            // read through TMA; written (append) by the leader when verifying
@@ -48,7 +50,9 @@ struct StepArgs {
     const float *pv_p, *pv_q, *pv_u;  // sampled verification (T > 0): null = greedy; pv_target then holds
                                       // the residual / bonus draws and pv_q may be null (copy drafts)
     int32_t *out_accept;
-    int32_t B, cap, d, k, n_min, n_max, kappa, tile, stages;
+    int32_t B, cap, d, k, n_min, n_max, kappa;
+    int32_t tile, stages, range, ring;  // ends a copy holds and copies in flight (1 without the ring); the largest CTA
+                                        // range; whether the ranges are staged through a ring of tiles
     int32_t prefetch;        // SWITCHSD_PREFETCH_* bits: reads that may precede the grid-dependency wait
     int32_t hidden_rows;     // > 1: hidden is [B, hidden_rows, d] and the probe reads row a_b (verifying)
     int32_t len_bound;       // > 0: every row's length is at most this; the ranges are split on it
@@ -56,7 +60,7 @@ struct StepArgs {
     int32_t *out_draft, *out_len, *out_mode;
     float *out_score;
     int32_t *out_match_n, *out_match_end, *status;
-    int32_t W, D, bm_words;   // candidate mode: W candidates of up to D tokens; bitmap words per CTA
+    int32_t W, D;             // candidate mode: W candidates of up to D tokens
     int32_t *out_cand, *out_cand_len, *out_ncand;
     const int32_t *pv_cand_len;  // candidate mode, verifying: the previous candidates' lengths [B, W]
                                  // (pv_draft [B, W, D], pv_target [B, W, D+1], pv_len = their count [B])
@@ -84,16 +88,8 @@ __device__ __forceinline__ float dot8_bf16(uint4 w, uint4 h, float acc) {
     return acc;
 }
 
-__device__ __forceinline__ void st_cluster_i32(uint32_t addr, int32_t v) {
-    asm volatile("st.shared::cluster.s32 [%0], %1;\n" ::"r"(addr), "r"(v) : "memory");
-}
-
-// Launches step_kernel<cand> on grid (split, B) as clusters of `split` CTAs, with the shared memory
-// that args.stages / args.tile / args.bm_words call for.
-cudaError_t launch_step_kernel(const StepArgs &args, bool cand, int split, cudaStream_t stream);
-
-// The rescan kernel (rescan.cu) on grid (split, B): the linear probe, greedy or sampled verification (or
-// none), no candidates, no length bound; args.tile >= the largest CTA range, args.probe_words set.
+// The rescan kernel (rescan.cu) on grid (split, B): every step without the index.  args.tile, stages, range,
+// ring, probe_words and (without the ring) hash_words set.
 cudaError_t launch_rescan_kernel(const StepArgs &args, int split, cudaStream_t stream);
 size_t rescan_smem_bytes(const StepArgs &args, int split);
 // Sets args.hash_words: the pre-wait hash table when the grid has at least one CTA per SM (`sms` SMs) and

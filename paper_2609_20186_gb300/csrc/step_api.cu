@@ -1,8 +1,8 @@
 // step_api.cu -- the step entry points of the C ABI: switchsd_step, switchsd_verify_step,
 // switchsd_verify_sampled_step, switchsd_step_candidates, switchsd_verify_candidates_step and
 // switchsd_workspace_bytes.  Host-side validation, the choice of the split, the shared-memory tiling of
-// each CTA's range, the two-layer probe's kernels and the index's kernel; the step kernel itself is
-// in step.cu.
+// each CTA's range, the two-layer probe's kernels and the index's kernel; the rescan kernel itself is
+// in rescan.cu.
 #include <cstdlib>
 
 #include "common.cuh"
@@ -29,17 +29,6 @@ static int sm_count_cached() {
 
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// CTAs per row: the largest power of two, at most kMaxSplit, that leaves every CTA at least 4096
-// candidate ends and keeps the grid within one wave of four CTAs per SM (the step kernel's register
-// limit); 1 at least.  Measured on this GPU, per-CTA ranges of 4K-9K ends in a single wave beat both
-// smaller ranges (more CTAs per row to reduce and ship) and a second wave.
-static int choose_split(int B, int cap) {
-    const int sms = sm_count_cached() > 0 ? sm_count_cached() : 148;
-    int c = 1;
-    while (c < kMaxSplit && cap / (2 * c) >= 4096 && int64_t(B) * (2 * c) <= 4ll * sms) c *= 2;
-    return c;
-}
-
 // CTAs per row of the rescan kernel: the largest power of two, at most kMaxSplit, that leaves every CTA
 // at least 4096 candidate ends while two launches' grids fit on the GPU at once (seven of its CTAs per
 // SM), so the next launch's copies are in flight while this one finishes; 1 at least.  Measured in the
@@ -52,6 +41,38 @@ static int choose_rescan_split(int B, int cap) {
     while (c < kMaxSplit && cap / (2 * c) >= 4096 && 2 * int64_t(B) * (2 * c) <= int64_t(kRescanMinBlocks) * sms)
         c *= 2;
     return c;
+}
+
+// CTAs per row when the rescan kernel's one-copy ranges would not fit: the ring's, the largest power of two, at
+// most kMaxSplit, with at most kRingCtas CTAs per SM.  Measured on 96 rows of 100K..200K tokens, per launch at
+// two tiles of 8192 ends a CTA: 4 CTAs a row 13.5 us, 2: 18.1; 8 (two tiles of 4096): 16.1.
+static int choose_ring_split(int B) {
+    const int sms = sm_count_cached() > 0 ? sm_count_cached() : 148;
+    int c = 1;
+    while (c < kMaxSplit && int64_t(B) * (2 * c) <= int64_t(kRingCtas) * sms) c *= 2;
+    return c;
+}
+
+// The ring's tile and stages: as much shared memory as lets the whole grid (up to kRingCtas CTAs per SM) be
+// resident at once -- and the next launch's, when an SM has one CTA -- in the largest tiles of which it holds two
+// (at most kRingTileMax ends).  Larger tiles beat more of them: the same rows
+// took 13.5 us a launch with two tiles of 8192 ends, 15.9 with three of 4096, 16.4 with three of 2048 (8 CTAs a
+// row) -- a tile's fixed cost (its wait, the second pass, the refill) is paid by every warp.
+static void choose_ring_tiles(StepArgs &a, int split) {
+    const int sms = sm_count_cached() > 0 ? sm_count_cached() : 148;
+    a.ring = 1;
+    const int64_t ctas = (int64_t(a.B) * split + sms - 1) / sms;  // a SM's share of the grid
+    const int64_t share = int64_t(kSmSharedBytes) / (ctas < 2 ? 2 : (ctas < kRingCtas ? ctas : kRingCtas)) - kCtaSharedReserve;
+    StepArgs z = a;
+    z.stages = 0;
+    const int64_t fixed = int64_t(rescan_smem_bytes(z, split));
+    const int64_t budget = (share < int64_t(kRingSmemBudget) ? share : int64_t(kRingSmemBudget)) - fixed;
+    const int64_t words = budget / (2 * int64_t(sizeof(int32_t))) - (kHalo + kFwd);  // a tile, when two fit
+    a.tile = int32_t(words < kRingTileMax ? words : kRingTileMax) & ~127;
+    if (a.tile < kRingTileMin) a.tile = kRingTileMin;
+    a.stages = budget > 0 ? int32_t(budget / int64_t((kHalo + a.tile + kFwd) * sizeof(int32_t))) : 0;
+    if (a.stages < 2) a.stages = 2;
+    if (a.stages > kRingStages) a.stages = kRingStages;
 }
 
 // Polls of the rescan kernel's wait for the row's messages: kWaitLimit, or the value of the environment
@@ -216,61 +237,46 @@ static int step_entry(int32_t *ctx_tokens, int32_t *ctx_lens, const uint16_t *hi
     args.counters = cs == nullptr ? reinterpret_cast<unsigned long long *>(p->counters) : nullptr;
     args.msg_wait_polls = kWaitLimit;
     args.wait_late = 0;
+    args.tile = args.stages = args.range = args.ring = 0;
 
     args.probe_words = 0;
     args.hash_words = 0;
-    const int split = p->split > 0 ? p->split : choose_split(p->B, p->cap);
-    // Tile: the largest CTA range (the last CTA may also cover a k + 1 token append), in one stage
-    // up to kSingleTileMax ends (64 KB; one copy, and few enough bytes that a grid of two or four
-    // CTAs per SM stays resident in one wave), else a ring of kTileMax stages, as many as the range
-    // needs up to kMaxStages and the shared-memory budget.
-    const int64_t range = ((int64_t(p->cap) - 1 + split - 1) / split + 3) / 4 * 4 + args.k + 1;
-    // candidate mode: a bit per end of the CTA's range, after the stages
     args.W = cs ? cs->W : 0;
     args.D = cs ? cs->D : 0;
-    args.bm_words = cs ? int32_t((range + 31) / 32) : 0;
     args.out_cand = cs ? cs->cand : nullptr;
     args.out_cand_len = cs ? cs->cand_len : nullptr;
     args.out_ncand = cs ? cs->ncand : nullptr;
     args.pv_cand_len = cs ? cs->pv_cand_len : nullptr;
     args.out_choice = cs ? cs->out_choice : nullptr;
-    const size_t budget = kStageSmemBudget - size_t(args.bm_words) * sizeof(uint32_t);
-    if (range <= kSingleTileMax) {
-        args.tile = int32_t((range + 3) / 4 * 4);
-        args.stages = 1;
-    } else {
-        args.tile = kTileMax;
-        const int64_t need = (range + kTileMax - 1) / kTileMax;
-        const int64_t fit = int64_t(budget / ((kHalo + kTileMax + kFwd) * sizeof(int32_t)));
-        args.stages = int32_t(need < fit ? need : fit);
-        if (args.stages > kMaxStages) args.stages = kMaxStages;
-        if (args.stages < 2) args.stages = 2;
-    }
 
     args.b2 = p->b2;
-    // The rescan kernel takes the step without the index -- single draft or W candidates, linear probe or
-    // the two-layer probe's finish after its first-layer kernel -- when the row's range fits its shared
-    // memory; the step kernel takes the rest.
+    // The rescan kernel takes the step without the index -- single draft or W candidates, linear probe or the
+    // two-layer probe's finish after its first-layer kernel: one copy a CTA range when that fits its shared memory, else a
+    // ring of tiles.
     const bool mlp_probe = p->probe_kind == SWITCHSD_PROBE_MLP;
-    const int rsplit = p->split > 0 ? p->split : choose_rescan_split(p->B, p->cap);
-    StepArgs ra = args;
-    bool rescan = false;
-    if (p->index == nullptr && p->cap <= kRescanCapMax) {
-        const int64_t rrange = ((int64_t(p->cap) - 1 + rsplit - 1) / rsplit + 3) / 4 * 4;
+    int split = 1;
+    if (p->index == nullptr) {
         const int nv = p->d >> 3;
-        const int vper = (nv + rsplit - 1) / rsplit;
-        ra.tile = int32_t(rrange);
-        ra.stages = 1;
-        ra.probe_words = mlp_probe ? 0 : (vper < kProbeStage ? vper : kProbeStage);
-        ra.msg_wait_polls = msg_wait_polls();
-        ra.bm_words = 0;  // the rescan kernel sizes its own bitmap from the tile
-        if (cs == nullptr) {
-            ra.W = ra.D = 0;
-            ra.out_cand = ra.out_cand_len = ra.out_ncand = ra.out_choice = nullptr;
-            ra.pv_cand_len = nullptr;
+        auto ranges = [&](int c) {
+            split = c;
+            args.range = int32_t(((int64_t(p->cap) - 1 + c - 1) / c + 3) / 4 * 4);
+            const int vper = (nv + c - 1) / c;
+            args.probe_words = mlp_probe ? 0 : (vper < kProbeStage ? vper : kProbeStage);
+        };
+        ranges(p->split > 0 ? p->split : choose_rescan_split(p->B, p->cap));
+        args.ring = 0;
+        args.stages = 1;
+        args.tile = args.range;
+        args.msg_wait_polls = msg_wait_polls();
+        if (p->cap > kRescanCapMax || args.range > kRescanTileMax || rescan_smem_bytes(args, split) > kRescanSmemBudget) {
+            if (p->split == 0) ranges(choose_ring_split(p->B));
+            choose_ring_tiles(args, split);
+            // a candidate bitmap too large beside two tiles: more CTAs per row
+            while (p->split == 0 && split < kMaxSplit && rescan_smem_bytes(args, split) > kRingSmemBudget) {
+                ranges(2 * split);
+                choose_ring_tiles(args, split);
+            }
         }
-        ra.hash_words = 0;
-        rescan = rrange <= kRescanTileMax && rescan_smem_bytes(ra, rsplit) <= kRescanSmemBudget;
     }
     bool mlp_early = false;  // the first-layer kernel releases the step kernel at its start
     if (mlp_probe) {
@@ -303,7 +309,7 @@ static int step_entry(int32_t *ctx_tokens, int32_t *ctx_lens, const uint16_t *hi
         // Beside the rescan kernel the first layer stages two chunks at a time, so that every CTA of the
         // rescan kernel fits on the GPU while it runs (that kernel verifies and scans meanwhile).
         if (launch_mlp_tc(probe_in, probe_w, part, p->B, p->d, p->probe_hidden, probe_pf, stream,
-                          rescan ? kMlpStagesBeside : 0) != cudaSuccess)
+                          p->index == nullptr ? kMlpStagesBeside : 0) != cudaSuccess)
             return SWITCHSD_ERR_CUDA;
         args.z1_part = part;
         mlp_early = probe_pf;
@@ -330,27 +336,15 @@ static int step_entry(int32_t *ctx_tokens, int32_t *ctx_lens, const uint16_t *hi
                             p->n_min, p->n_max, p->kappa, p->logit_tau, true, stream, pv_p, pv_q, pv_u,
                             args.hidden_rows, cs != nullptr ? &ic : nullptr, p->prefetch, args.counters);
     }
-    if (rescan) {
-        ra.z1_part = args.z1_part;
-        ra.b1 = args.b1;
-        ra.w2 = args.w2;
-        ra.mlp_S = args.mlp_S;
-        ra.H1 = args.H1;
-        ra.H1p = args.H1p;
-        ra.hidden_rows = args.hidden_rows;
-        // Without the probe prefetch the first-layer kernel launched just above waits for every earlier
-        // kernel before it releases this one, so only its own output, the partial sums, needs this
-        // launch's wait.  With it, that kernel releases this one at its start: this launch then reads
-        // before its wait only what the caller's prefetch bits cover, and everything else after it.
-        ra.wait_late = (args.z1_part != nullptr && !mlp_early) ? 1 : 0;
-        if (rescan_choose_hash(ra, rsplit, sm_count_cached() > 0 ? sm_count_cached() : 148) != cudaSuccess)
-            return SWITCHSD_ERR_CUDA;
-        if (launch_rescan_kernel(ra, rsplit, stream) != cudaSuccess) return SWITCHSD_ERR_CUDA;
-        return SWITCHSD_OK;
-    }
-    const cudaError_t e = launch_step_kernel(args, cs != nullptr, split, stream);
-    if (e != cudaSuccess) return SWITCHSD_ERR_CUDA;
-    return SWITCHSD_OK;
+    // Without the probe prefetch the first-layer kernel launched just above waits for every earlier
+    // kernel before it releases this one, so only its own output, the partial sums, needs this
+    // launch's wait.  With it, that kernel releases this one at its start: this launch then reads
+    // before its wait only what the caller's prefetch bits cover, and everything else after it.
+    args.wait_late = (args.z1_part != nullptr && !mlp_early) ? 1 : 0;
+    if (!args.ring &&
+        rescan_choose_hash(args, split, sm_count_cached() > 0 ? sm_count_cached() : 148) != cudaSuccess)
+        return SWITCHSD_ERR_CUDA;
+    return launch_rescan_kernel(args, split, stream) == cudaSuccess ? SWITCHSD_OK : SWITCHSD_ERR_CUDA;
 }
 
 }  // namespace switchsd
