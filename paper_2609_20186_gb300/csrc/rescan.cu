@@ -362,6 +362,36 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
         if (bytes > 0) bulk_g2s_hint(stage + (kHalo + lo - e_lo), row + lo, bytes, &bars[0], pol);
     };
     if (bounded && tid == 0) issue_tile(tile_hi());
+    // The verification's inputs (lane i: positions i and i + 32) are loaded as soon as the wait allows -- before
+    // the length when that is read after the wait too, so that the two round trips overlap (8 launches on 37
+    // ragged rows of 9K tokens: 38.9 -> 37.6 us).
+    int32_t pv_n = 0, d_lo = 0, d_hi = 0, t_lo = 0, t_hi = 0, t_top = 0;
+    float pv_lo[3] = {0.f, 1.f, 0.f}, pv_hi[3] = {0.f, 1.f, 0.f};  // sampled: u, q, p
+    auto load_draft = [&]() {
+        if (kCand || !verifying) return;
+        const int32_t *dr = a.pv_draft + size_t(b) * a.k;
+        const int32_t *tg = a.pv_target + size_t(b) * (a.k + 1);
+        pv_n = __ldcg(a.pv_len + b);
+        if (lane < a.k) d_lo = __ldcg(dr + lane);
+        if (lane + 32 < a.k) d_hi = __ldcg(dr + lane + 32);
+        if (lane <= a.k) t_lo = __ldcg(tg + lane);
+        if (lane + 32 <= a.k) t_hi = __ldcg(tg + lane + 32);
+        if (lane == 0 && a.k >= 64) t_top = __ldcg(tg + 64);
+        if (kSampled) {
+            const size_t o = size_t(b) * a.k + lane;
+            if (lane < a.k) {
+                pv_lo[0] = __ldcg(a.pv_u + o);
+                if (a.pv_q) pv_lo[1] = __ldcg(a.pv_q + o);
+                pv_lo[2] = __ldcg(a.pv_p + o);
+            }
+            if (lane + 32 < a.k) {
+                pv_hi[0] = __ldcg(a.pv_u + o + 32);
+                if (a.pv_q) pv_hi[1] = __ldcg(a.pv_q + o + 32);
+                pv_hi[2] = __ldcg(a.pv_p + o + 32);
+            }
+        }
+    };
+    if (!pf_ctx) load_draft();
     // Every thread reads the length itself (one L2 request per warp), then arrives on the cluster
     // barrier.  The arrive is relaxed: the barrier only has to publish the leader's message barrier (its
     // initialisation fence is a release), and each warp's read of the length is ordered before the leader
@@ -441,6 +471,7 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
         mbar_arrive(&bars[4]);  // every thread of warps 1.., whether or not it hashed
     }
     if (pf_ctx && !late) pdl_wait();
+    if (pf_ctx) load_draft();
     pdl_trigger();
     if (!pf_probe && !gather && !mlp && tid == 0) issue_probe();
 
@@ -479,7 +510,7 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
 
     // ---- verification of the previous draft (every warp) ----
     int32_t acc = -1, L = L_old, vst = len_ok ? SWITCHSD_ROW_OK : SWITCHSD_ROW_BAD_LEN;
-    int32_t d_lo = 0, d_hi = 0, t_acc = 0;
+    int32_t t_acc = 0;
     int32_t choice = 0;  // candidate mode: the kept candidate
     if (kCand && verifying) {
         // The W previous candidates verified at once (§3.3): the CTA stages every slot's draft, target and
@@ -537,26 +568,14 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
         }
     }
     if (!kCand && verifying && len_ok) {
-        const int32_t *dr = a.pv_draft + size_t(b) * a.k;
-        const int32_t *tg = a.pv_target + size_t(b) * (a.k + 1);
-        const int32_t pv_n = __ldcg(a.pv_len + b);
-        d_lo = lane < a.k ? __ldcg(dr + lane) : 0;
-        d_hi = lane + 32 < a.k ? __ldcg(dr + lane + 32) : 0;
-        const int32_t t_lo = lane <= a.k ? __ldcg(tg + lane) : 0;
-        const int32_t t_hi = lane + 32 <= a.k ? __ldcg(tg + lane + 32) : 0;
-        const int32_t t_top = (lane == 0 && a.k >= 64) ? __ldcg(tg + 64) : 0;
         if (pv_n < 0 || pv_n > a.k) {
             vst = SWITCHSD_ROW_BAD_LEN;
         } else {
             bool rej_lo, rej_hi;
             if (kSampled) {
                 // T > 0: draft token i is rejected when u_i * q_i (binary32) is not below p_i
-                const size_t o = size_t(b) * a.k;
-                rej_lo = lane < pv_n && !(__fmul_rn(__ldcg(a.pv_u + o + lane), a.pv_q ? __ldcg(a.pv_q + o + lane) : 1.f) <
-                                          __ldcg(a.pv_p + o + lane));
-                rej_hi = lane + 32 < pv_n &&
-                         !(__fmul_rn(__ldcg(a.pv_u + o + lane + 32), a.pv_q ? __ldcg(a.pv_q + o + lane + 32) : 1.f) <
-                           __ldcg(a.pv_p + o + lane + 32));
+                rej_lo = lane < pv_n && !(__fmul_rn(pv_lo[0], pv_lo[1]) < pv_lo[2]);
+                rej_hi = lane + 32 < pv_n && !(__fmul_rn(pv_hi[0], pv_hi[1]) < pv_hi[2]);
             } else {
                 rej_lo = lane < pv_n && d_lo != t_lo;
                 rej_hi = lane + 32 < pv_n && d_hi != t_hi;
