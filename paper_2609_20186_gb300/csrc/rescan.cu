@@ -27,7 +27,7 @@
 //    (the last one) with asynchronous DSMEM stores completing on the leader's mbarrier, and is done.
 // The leader's warp 0 publishes the append, waits (bounded) for the C x kRescanWarps messages, reduces
 // them in a fixed order and writes the outputs.  The only cluster barrier is arrived on right after the
-// length read and waited on just before the first message, so the leader's message barrier is
+// length read and waited on beside the verification's loads, so the leader's message barrier is
 // initialised before anyone ships to it and no CTA reads the length after the leader rewrites it.
 #include <mutex>
 #include <type_traits>
@@ -452,7 +452,10 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     };
     // A prefetched probe is finished before the wait by warps 1.. (its inputs are not written by the
     // preceding kernel); warp 0 goes straight to the wait and releases the next launch.
-    if (pf_probe && warp >= 1) probe_dot(h4);
+    if (pf_probe) {
+        if (warp >= 1) probe_dot(h4);
+        zp = warp_sum_f32(zp);
+    }
     // Warps 1.. hash this CTA's old ends once the tile has landed -- before the wait when the context is
     // prefetched -- so that the scan after it compares one byte per end (scan_ends, kPre).
     constexpr bool pre = kPre;
@@ -473,6 +476,9 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     if (pf_ctx && !late) pdl_wait();
     if (pf_ctx) load_draft();
     pdl_trigger();
+    // Every CTA has read the length and the leader's message barrier is initialised once this returns; the arrive
+    // was long before, so it costs little beside the loads in flight (on the way out it cost the row's chain).
+    cluster_wait_acquire();
     if (!pf_probe && !gather && !mlp && tid == 0) issue_probe();
 
     // Two-layer probe: this CTA finishes units [u0m, u1m) (the S partial sums in order, b1, ReLU, w2);
@@ -834,13 +840,12 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
         }
     }
     if (!probe_ok) key = kKeyTimeout;
-    const float z_w = warp_sum_f32(zp);
+    const float z_w = pf_probe ? zp : warp_sum_f32(zp);
 
     // ---- the continuation of this warp's best match (the ring has it already) ----
     if (!kRing && key != 0u && key != kKeyTimeout) gather_next(int32_t(key & kKeyEndMask), stage, off);
 
     // ---- ship to the leader ----
-    cluster_wait_acquire();  // every CTA has read the length and the leader's barrier is initialised
     const uint32_t done_addr = map_to_rank(&bars[3], lead);
     unsigned char *slot = msgs + size_t(rank * kRescanWarps + warp) * slot_bytes;
     if (lane == 0) {
