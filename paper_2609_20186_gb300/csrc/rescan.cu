@@ -111,7 +111,8 @@ __device__ __forceinline__ void hash_ends(const int32_t *stage, uint32_t *hb, in
 template <int F, bool kCand, bool kPre>
 __device__ __forceinline__ uint32_t scan_ends(const int32_t *stage, int32_t e_lo, int32_t e_end, const int32_t *suf,
                                               int32_t n_min, int32_t n_max, int tid, int lane, uint32_t *bm,
-                                              int32_t kappa_c, const uint32_t *hb, int32_t key0, int32_t bm_lo) {
+                                              int32_t kappa_c, const uint32_t *hb, int32_t key0, int32_t bm_lo,
+                                              bool *marked) {
     const int32_t s0 = suf[0], s1 = F >= 2 ? suf[-1] : 0, s2 = F >= 3 ? suf[-2] : 0;
     const uint32_t hs = end_hash<F>(s0, s1, s2);
     const uint32_t hs4 = hash_byte(hs) * 0x01010101u;
@@ -179,7 +180,10 @@ __device__ __forceinline__ uint32_t scan_ends(const int32_t *stage, int32_t e_lo
             const uint32_t key = (uint32_t(m) << kKeyShift) | uint32_t(e - key0);
             mine = key > mine ? key : mine;
         }
-        if (kCand && m >= kappa_c) atomicOr(&bm[(e - bm_lo) >> 5], 1u << ((e - bm_lo) & 31));
+        if (kCand && m >= kappa_c) {
+            atomicOr(&bm[(e - bm_lo) >> 5], 1u << ((e - bm_lo) & 31));
+            *marked = true;
+        }
     };
     while (__any_sync(kFull, passed != 0u)) {
         if (passed == 0u) continue;
@@ -233,7 +237,7 @@ constexpr int kVerifyLoads = 4;  // candidate verification: staging loads a thre
 // bytes -- a 16-byte header (count), the ends (W, most recent first), their continuations [W][D] (not from
 // a ring, whose tiles are gone by then: the leader reads them from the row) -- the
 // leader receiving C of them and every CTA staging its own; a bitmap of the CTA's marked ends; the
-// verification's staging of the previous candidates (drafts [W][D], targets [W][D+1], lengths [W], count).
+// verification's staging of the previous candidates (drafts [W][D], targets [W][D+1]).
 struct CandLayout {
     uint32_t cslot;  // bytes of a candidate message
     int bm_words;    // bitmap words (a multiple of 4)
@@ -243,7 +247,7 @@ __host__ __device__ inline CandLayout cand_layout(int range, int W, int D, bool 
     CandLayout c;
     c.cslot = 16u * uint32_t(1 + (W + 3) / 4 + (ring ? 0 : (W * D + 3) / 4));
     c.bm_words = ((range + 31) / 32 + 3) & ~3;
-    c.v_ints = (W * D + W * (D + 1) + W + 1 + 3) & ~3;
+    c.v_ints = (W * D + W * (D + 1) + 3) & ~3;
     return c;
 }
 
@@ -270,6 +274,8 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     __shared__ int32_t s_sel[kMaxCand];                    // candidate mode: the CTA's selected ends / the
                                                            // leader's merged candidates' sources
     __shared__ int32_t s_wtot[kRescanWarps];               // candidate mode: marks per warp in a pass
+    __shared__ int32_t s_miss[kMaxCand];                   // candidate mode: the first position of each previous
+                                                           // candidate that differs from the target
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t rank = cluster_ctarank();
@@ -292,7 +298,6 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     uint32_t *bm = reinterpret_cast<uint32_t *>(cstage + cl.cslot);           // [bm_words]
     int32_t *vc = reinterpret_cast<int32_t *>(bm + cl.bm_words);              // previous drafts [W][D]
     int32_t *vt = vc + a.W * a.D;                                             // their targets [W][D+1]
-    int32_t *vl = vt + a.W * (a.D + 1);                                       // their lengths [W]
 
     if (tid == 0) {
         mbar_init(&bars[0], 1);
@@ -310,8 +315,10 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
         }
         fence_mbar_init();
     }
-    if (kCand)
+    if (kCand) {
         for (int i = tid; i < cl.bm_words; i += kRescanThreads) bm[i] = 0u;
+        if (tid < kMaxCand) s_miss[tid] = SWITCHSD_KMAX;
+    }
     __syncthreads();  // the barriers are initialised (and the bitmap cleared) before any thread uses them
 
     const bool pf_ctx = (a.prefetch & SWITCHSD_PREFETCH_CONTEXT) != 0;
@@ -519,50 +526,53 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     int32_t t_acc = 0;
     int32_t choice = 0;  // candidate mode: the kept candidate
     if (kCand && verifying) {
-        // The W previous candidates verified at once (§3.3): the CTA stages every slot's draft, target and
-        // length (one round of independent L2 reads, whatever the count), then each warp takes, per
-        // candidate, the first position where draft and target differ; the longest accepted candidate is
-        // kept, the lowest index on a tie.  A count of 0 (a neural draft) uses slot 0 with length 0.
+        // The W previous candidates verified at once (§3.3): thread i takes the positions i, i + kRescanThreads, ... of the
+        // candidates laid end to end, stages their draft and target tokens and notes the first position of each
+        // candidate that differs; each warp then takes the accepted lengths with lane w on candidate w.  The
+        // longest is kept, the lowest index on a tie.  A count of 0 (a neural draft) uses slot 0 with length 0.
         const int W = a.W, D = a.D;
         const size_t o = size_t(b) * size_t(W);
-        // one index space over drafts, targets, lengths and the count (vl[W]); each thread issues all of
-        // its loads before its first store, so they share one round trip
-        const int n_d = W * D, n_t = W * (D + 1), n_all = n_d + n_t + W + 1;
-        for (int base = tid; base < n_all; base += kVerifyLoads * kRescanThreads) {
-            int32_t v[kVerifyLoads];
+        const int n_d = W * D;
+        const int32_t ncv = __ldcg(a.pv_len + b);
+        const int32_t lenv = lane < W ? __ldcg(a.pv_cand_len + o + lane) : 0;
+        const int32_t topv = tid < W ? __ldcg(a.pv_target + (o + tid) * (D + 1) + D) : 0;  // after a whole candidate
+        // each thread issues its loads before its first store, so they share one round trip
+        for (int base = tid; base < n_d; base += kVerifyLoads * kRescanThreads) {
+            int32_t c[kVerifyLoads], t[kVerifyLoads];
 #pragma unroll
             for (int u = 0; u < kVerifyLoads; ++u) {
                 const int i = base + u * kRescanThreads;
-                v[u] = 0;
-                if (i < n_d) v[u] = __ldcg(a.pv_draft + o * D + i);
-                else if (i < n_d + n_t) v[u] = __ldcg(a.pv_target + o * (D + 1) + (i - n_d));
-                else if (i < n_d + n_t + W) v[u] = __ldcg(a.pv_cand_len + o + (i - n_d - n_t));
-                else if (i < n_all) v[u] = __ldcg(a.pv_len + b);
-            }
-#pragma unroll
-            for (int u = 0; u < kVerifyLoads; ++u)
-                if (base + u * kRescanThreads < n_all) vc[base + u * kRescanThreads] = v[u];  // vc, vt, vl contiguous
-        }
-        __syncthreads();
-        const int32_t nc = vl[W];
-        if (len_ok) {
-            bool badlen = nc < 0 || nc > W;
-            const int ncx = badlen ? 0 : (nc > 0 ? nc : 1);
-            int32_t best = -1, best_w = 0;
-            for (int w = 0; w < ncx; ++w) {
-                const int32_t len = nc > 0 ? vl[w] : 0;
-                badlen |= len < 0 || len > D;
-                const int32_t lc = (len >= 0 && len <= D) ? len : 0;
-                const int32_t *cw_ = vc + w * D, *tw_ = vt + w * (D + 1);
-                const unsigned m_lo = __ballot_sync(kFull, lane < lc && cw_[lane] != tw_[lane]);
-                const unsigned m_hi = __ballot_sync(kFull, lane + 32 < lc && cw_[lane + 32] != tw_[lane + 32]);
-                const int32_t acc_w = m_lo ? __ffs(m_lo) - 1 : (m_hi ? 32 + __ffs(m_hi) - 1 : lc);
-                if (acc_w > best) {
-                    best = acc_w;
-                    best_w = w;
+                c[u] = t[u] = 0;
+                if (i < n_d) {
+                    c[u] = __ldcg(a.pv_draft + o * D + i);
+                    t[u] = __ldcg(a.pv_target + o * (D + 1) + i + i / D);
                 }
             }
-            choice = best_w;
+#pragma unroll
+            for (int u = 0; u < kVerifyLoads; ++u) {
+                const int i = base + u * kRescanThreads;
+                if (i < n_d) {
+                    const int w = i / D;
+                    vc[i] = c[u];
+                    vt[i + w] = t[u];
+                    if (c[u] != t[u]) atomicMin(&s_miss[w], i - w * D);
+                }
+            }
+        }
+        if (tid < W) vt[tid * (D + 1) + D] = topv;
+        __syncthreads();
+        const int32_t nc = ncv;
+        if (len_ok) {
+            const bool nc_ok = nc >= 0 && nc <= W;
+            const int ncx = !nc_ok ? 0 : (nc > 0 ? nc : 1);
+            const int32_t len = nc > 0 ? lenv : 0;
+            const bool used = lane < ncx;
+            const bool len_bad = used && (len < 0 || len > D);
+            const bool badlen = __any_sync(kFull, len_bad) || !nc_ok;
+            const int32_t acc_w = used && !len_bad ? min(s_miss[lane], len) : 0;
+            const uint32_t rank_w = __reduce_max_sync(kFull, used ? (uint32_t(acc_w) << 5 | uint32_t(31 - lane)) + 1u : 0u);
+            const int32_t best = rank_w != 0u ? int32_t((rank_w - 1u) >> 5) : -1;
+            choice = rank_w != 0u ? 31 - int32_t((rank_w - 1u) & 31u) : 0;
             if (badlen) {
                 vst = SWITCHSD_ROW_BAD_LEN;
             } else if (L_old + best + 1 > a.cap) {
@@ -647,14 +657,15 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     const int32_t off = kHalo - e_lo;  // stage[off + p] = x[p] over the staged range
     // (n_min and kappa are uniform over the launch: one instance runs)
     // the filter depth may test no more than a candidate needs (fdepth <= kappa in candidate mode)
+    bool marked = false;  // candidate mode: this thread marked an end
     auto scan = [&](const int32_t *st, int32_t lo_e, int32_t end_e, int32_t key0) {
         const int fdepth = filter_depth();
         return fdepth >= 3
-                   ? scan_ends<3, kCand, kPre>(st, lo_e, end_e, suf, n_min, n_max, tid, lane, bm, kappa_c, hb, key0, e_lo)
+                   ? scan_ends<3, kCand, kPre>(st, lo_e, end_e, suf, n_min, n_max, tid, lane, bm, kappa_c, hb, key0, e_lo, &marked)
                    : (fdepth == 2 ? scan_ends<2, kCand, kPre>(st, lo_e, end_e, suf, n_min, n_max, tid, lane, bm, kappa_c,
-                                                              hb, key0, e_lo)
+                                                              hb, key0, e_lo, &marked)
                                   : scan_ends<1, kCand, kPre>(st, lo_e, end_e, suf, n_min, n_max, tid, lane, bm, kappa_c,
-                                                              hb, key0, e_lo));
+                                                              hb, key0, e_lo, &marked));
     };
     // the continuation of a match ending at e: lane j (1..kw) gathers tokens 4(j-1) .. +3, from the staged
     // tile (tl[o_ + p] = x[p]) or past the old length from this warp's window
@@ -763,11 +774,12 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
 
     // ---- candidate mode: this CTA's W most recent marked ends and their continuations (warp 0) ----
     if constexpr (kCand) {
-        __syncthreads();  // every warp's marks are in the bitmap
+        // every warp's marks are in the bitmap after this barrier; most CTAs have none to rank
+        const bool any_marked = __syncthreads_or(marked);
         // Bitmap words from the top, kRescanThreads per pass: thread t holds word top - t; prefix sums of
         // the popcounts (within the warp, then over the warps) rank its bits after those of higher words.
         // `found` is CTA-uniform.
-        const int nwords = (e_end - e_lo + 31) >> 5;
+        const int nwords = any_marked ? (e_end - e_lo + 31) >> 5 : 0;
         int found = 0;
         for (int top = nwords - 1; top >= 0 && found < a.W; top -= kRescanThreads) {
             const int idx = top - tid;
@@ -819,8 +831,7 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
                     ++w;
                 }
             }
-            fence_proxy_async();  // the bulk copy below reads the message through the async proxy
-            __syncwarp();
+            __syncwarp();  // the message is shipped below, a word a lane
         }
     }
 
@@ -858,10 +869,12 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     } else if (lane <= kw) {
         st_async_v4(map_to_rank(slot + 16 * lane, lead), cw, done_addr);
     }
-    if (kCand && warp == 0 && lane == 0)  // this CTA's candidates, in one bulk copy
-        bulk_s2c(map_to_rank(cmsgs + size_t(rank) * cl.cslot, lead), cstage, cl.cslot, done_addr);
+    if (kCand && warp == 0) {  // this CTA's candidates
+        const uint32_t to = map_to_rank(cmsgs + size_t(rank) * cl.cslot, lead);
+        for (uint32_t i = lane; i < cl.cslot / 16; i += kWarp)
+            st_async_v4(to + 16 * i, reinterpret_cast<const uint4 *>(cstage)[i], done_addr);
+    }
     if (rank != lead || warp != 0) {
-        if (kCand && warp == 0 && lane == 0) bulk_wait_read();  // the message has been read out
         if (timed_out && lane == 0) {  // copies still in flight get a second bounded wait
             if (!kRing) (void)mbar_wait(&bars[0], 0);
             (void)mbar_wait(&bars[1], 0);
@@ -907,19 +920,22 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
         // The row's candidates, most recent first: the appended ends (highest first), then the CTAs' lists
         // from the leader's (the most recent range) down to CTA 0's.  s_sel[w] is merged candidate w's
         // source: -1 - j for the appended end L_old - 1 + j, else r kMaxCand + i for entry i of CTA r.
-        auto count_of = [&](int r) {
-            return min(*reinterpret_cast<const int32_t *>(cmsgs + size_t(r) * cl.cslot), a.W);
-        };
+        // Lane r holds CTA r's count; a suffix sum places its entries after those of the more recent CTAs.
         const int n_new = hit ? __popc(new_c[0]) + __popc(new_c[1]) + __popc(new_c[2]) : 0;
-        int total = n_new;
-        if (hit)
-            for (int r = 0; r < int(C); ++r) total += count_of(r);
-        const int ncand = min(total, a.W);
+        int cnt = 0;
+        if (hit && lane < int(C)) cnt = min(*reinterpret_cast<const int32_t *>(cmsgs + size_t(lane) * cl.cslot), a.W);
+        int after = cnt;
+#pragma unroll
+        for (int o_ = 1; o_ < kMaxSplit; o_ <<= 1) {
+            const int t_ = __shfl_down_sync(kFull, after, o_);
+            if (lane + o_ < kWarp) after += t_;
+        }
+        const int first = n_new + after - cnt;  // the rank of CTA `lane`'s first entry
+        const int ncand = min(n_new + __shfl_sync(kFull, after, 0), a.W);
         int32_t mode = SWITCHSD_MODE_NO_REP;
         if (hit) mode = (ncand > 0 && z >= a.logit_tau) ? SWITCHSD_MODE_COPY : SWITCHSD_MODE_REP_NO_COPY;
         const int nc = mode == SWITCHSD_MODE_COPY ? ncand : 0;
         if (lane < nc) {
-            int src = 0;
             if (lane < n_new) {
                 int k = lane, j = -1;
                 for (int t = 2; t >= 0 && j < 0; --t) {
@@ -932,18 +948,10 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
                         k -= pc;
                     }
                 }
-                src = -1 - j;
-            } else {
-                int k = lane - n_new, r = int(C) - 1;
-                for (; r > 0; --r) {
-                    const int cr = count_of(r);
-                    if (k < cr) break;
-                    k -= cr;
-                }
-                src = r * kMaxCand + k;
+                s_sel[lane] = -1 - j;
             }
-            s_sel[lane] = src;
         }
+        for (int i = 0; i < cnt && first + i < nc; ++i) s_sel[first + i] = lane * kMaxCand + i;
         __syncwarp();
         const int cwE = (a.W + 3) / 4;
         auto cand_end = [&](int src) -> int32_t {
@@ -989,7 +997,6 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
                 if (st == SWITCHSD_ROW_OK && timeout) st = SWITCHSD_ROW_TIMEOUT;
                 a.status[b] = st;
             }
-            bulk_wait_read();  // the leader's own message has been read out
         }
         (void)win;
     } else {
