@@ -2,13 +2,18 @@
 //
 // The paper's probe is linear (Eq. 3); this two-layer form is an extension used with probe_kind
 // SWITCHSD_PROBE_MLP.  Its first layer is a real contraction, Z1[B, H1] = H[B, d] . W1[H1, d]^T, so it
-// runs on tcgen05.  K = d is split S ways: CTA (s, n, m) stages its K chunks of H rows [128 m, +128) and
-// W1 units [64 n, +64) in shared memory with TMA (128-byte swizzle, zero fill past the tensor edges), one
-// thread issues tcgen05.mma (bf16 x bf16, fp32 accumulators in 64 TMEM columns), the four warps read
-// their 32 rows back with tcgen05.ld and store them as the split-K partial sums
+// runs on tcgen05.  K = d is split into P = mlp_split(d) parts, of which a CTA takes A = P / S: CTA (s, n, m)
+// stages the K chunks of its parts of H rows [128 m, +128) and W1 units [64 n, +64) in shared memory with TMA
+// (128-byte swizzle, zero fill past the tensor edges), one thread issues tcgen05.mma (bf16 x bf16, fp32
+// accumulators in 64 TMEM columns a part), the four warps read their 32 rows of the A parts back with
+// tcgen05.ld, add them in order and store the partial sums
 //     part[s][b][u]  (fp32, s < S, b < B, u < H1p = H1 rounded up to 64; units >= H1 hold zeros).
 // The step kernel that follows adds the S partials of its row in order, then b1, ReLU, w2 and b2: every
 // sum has a fixed order, so the result is deterministic.  No cluster and no cross-CTA exchange here.
+//
+// S is P, or P / 2 for the larger batches (mlp_ctas_per_tile), so that the partial sums that go through memory --
+// S B H1 floats written, then read by the row's step CTAs, which bound those batches -- stay small.  The parts,
+// and with them the length of every sum in an accumulator, do not depend on S.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -24,7 +29,6 @@ constexpr int kMlpKc = 64;             // K elements per staged chunk: one 128-b
 constexpr int kMlpThreads = 128;       // four warps: one per 32 TMEM lanes
 constexpr uint32_t kAChunk = kMlpM * kMlpKc * 2;    // 16 KB
 constexpr uint32_t kBChunk = kMlpN * kMlpKc * 2;    // 8 KB
-constexpr uint32_t kTmemCols = 64;
 static_assert(kMaxMlpChunks * (kAChunk + kBChunk) + 1024 + 64 <= 227 * 1024,
               "operands, alignment slack and static shared memory must fit one CTA");
 static_assert(kMlpThreads == kMlpM && kMlpN == 64, "one thread per tile row; 16 chunks of 16 bytes per row");
@@ -36,6 +40,8 @@ constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(kMlpN
 struct MlpArgs {
     float *part;   // [S][B][H1p]
     int32_t B, H1p, nchunks, prefetch;
+    int32_t parts;   // P
+    int32_t columns; // TMEM columns: 64 a part of the CTA, a power of two
     int32_t stages;  // operand stages: chunk c goes to stage c % stages, refilled once its MMAs are done
 };
 
@@ -77,9 +83,10 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int S = int(gridDim.x), ks = blockIdx.x;
     const int n_tile = blockIdx.y, m0 = blockIdx.z * kMlpM, n0 = n_tile * kMlpN;
-    const int per = (a.nchunks + S - 1) / S;
-    const int c0 = ks * per;
-    const int nck = max(0, min(a.nchunks, c0 + per) - c0);
+    const int A = a.parts / S;                           // this CTA's parts
+    const int per = (a.nchunks + a.parts - 1) / a.parts;  // chunks of a part (fewer, or none, at the end of K)
+    const int c0 = ks * A * per;
+    const int nck = max(0, min(a.nchunks, c0 + A * per) - c0);
     const int st = a.stages;  // 1 .. kMaxMlpChunks
     // 1024-byte aligned operand stages (the swizzle atom): A chunks, then B chunks.
     uint8_t *base = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
@@ -111,7 +118,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
     if (a.prefetch) pdl_trigger();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_addr(&s_tmem)),
-                     "r"(kTmemCols)
+                     "r"(a.columns)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
@@ -144,14 +151,14 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
             const uint64_t db = sw128_desc(smem_addr(opB + size_t(sg) * kBChunk));
 #pragma unroll
             for (int j = 0; j < kMlpKc / 16; ++j) {
-                const uint32_t acc = (c | j) != 0;
+                const uint32_t acc = ((c % per) | j) != 0;  // a part starts from zero in its own columns
                 // advance both descriptors by j * 32 bytes inside the swizzle row
                 asm volatile(
                     "{\n"
                     ".reg .pred p;\n"
                     "setp.ne.b32 p, %4, 0;\n"
                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
-                    "}\n" ::"r"(tmem),
+                    "}\n" ::"r"(tmem + uint32_t(kMlpN * (c / per))),
                     "l"(da + uint64_t(2 * j)), "l"(db + uint64_t(2 * j)), "r"(kIdesc), "r"(acc)
                     : "memory");
             }
@@ -183,30 +190,40 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     ok = __syncthreads_and(ok && mma_done);
 
-    // Row tid of the tile: its 64 accumulators (zero when this CTA had no K chunk; NaN when a copy or
-    // the MMAs did not complete in time, so the row's logit shows the failure).
-    float v[kMlpN];
-    if (nck > 0 && ok) {
-        const uint32_t taddr = tmem + (uint32_t(warp * 32) << 16);
-        tmem_ld32(taddr, v);
-        tmem_ld32(taddr + 32, v + 32);
-        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-    } else {
-        const float fill = ok ? 0.f : __int_as_float(0x7fc00000);
-#pragma unroll
-        for (int i = 0; i < kMlpN; ++i) v[i] = fill;
-    }
-    // The tile goes out through shared memory (the operand stages are free: every MMA has completed), so
-    // that each warp store writes two whole 256-byte rows instead of one 16-byte piece of 32 rows.  Row r
-    // keeps its 16-byte chunk q at position q ^ (r % 16): both the row-wise writes below and the reads
-    // across rows hit distinct banks.
-    // The partial sums overwrite what an earlier step kernel may still read: with the prefetch bit the
-    // copies and the MMAs above ran before the wait, the stores come after it.
-    if (a.prefetch) pdl_wait();
+    // Row tid of the tile: its 64 accumulators, the parts added in order (zero when this CTA had no K chunk;
+    // NaN when a copy or the MMAs did not complete in time, so the row's logit shows the failure).  The tile
+    // goes out through shared memory (the operand stages are free: every MMA has completed), so that each warp
+    // store writes two whole 256-byte rows instead of one 16-byte piece of 32 rows.  Row r keeps its 16-byte
+    // chunk q at position q ^ (r % 16): both the row-wise writes here and the reads across rows below hit
+    // distinct banks.
     float4 *tile = reinterpret_cast<float4 *>(base);  // [kMlpM rows][16 chunks]
+    const uint32_t taddr = tmem + (uint32_t(warp * 32) << 16);
+#pragma unroll 1
+    for (int g = 0; g < kMlpN; g += 32) {
+        float v[32];
+        if (nck > 0 && ok) {
+            tmem_ld32(taddr + uint32_t(g), v);
+            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll 1
+            for (int p = 1; p * per < nck; ++p) {
+                float w[32];
+                tmem_ld32(taddr + uint32_t(kMlpN * p + g), w);
+                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
-    for (int q = 0; q < kMlpN / 4; ++q)
-        tile[tid * 16 + (q ^ (tid & 15))] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                for (int i = 0; i < 32; ++i) v[i] += w[i];
+            }
+        } else {
+            const float fill = ok ? 0.f : __int_as_float(0x7fc00000);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) v[i] = fill;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            tile[tid * 16 + ((g / 4 + q) ^ (tid & 15))] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    }
+    // The partial sums overwrite what an earlier step kernel may still read: with the prefetch bit the copies
+    // and the MMAs above ran before the wait, the stores come after it.
+    if (a.prefetch) pdl_wait();
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
 #pragma unroll 4
@@ -217,7 +234,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
                 tile[r * 16 + (c ^ (r & 15))];
     }
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(a.columns) : "memory");
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -256,6 +273,25 @@ int mlp_split(int d) {
     return s;
 }
 
+int mlp_ctas_per_tile(int B, int d, int H1) {
+    const int parts = mlp_split(d);
+    // With every part its own CTA, parts x B x H1p floats go through memory.  Past 10 MB two parts a CTA are
+    // faster, below it the shorter CTAs.  A step (probe and rescan kernel), one part a CTA and two: 256 rows x
+    // 256 units (4 MB) 10.3 and 13.6 us, 512 x 256 (8 MB) 11.8 and 14.2, 130 x 1024 (8.5 MB) 13.2 and 14.4,
+    // 768 x 256 (12.6 MB) 18.6 and 17.2, 400 x 512 (13 MB) 20.7 and 15.3, 768 x 512 (25 MB) 25.1 and 21.0 (four
+    // parts a CTA: 23.3).
+    const size_t bytes = size_t(parts) * size_t(B) * size_t(mlp_hidden_padded(H1)) * sizeof(float);
+    return parts > 1 && bytes > 10u * 1000u * 1000u ? parts / 2 : parts;
+}
+
+// A grid of at most half the SMs stages all its chunks at once, one of at most a CTA an SM three, a larger one
+// two: a step of 64 rows x 256 units (64 CTAs) takes 8.4 us with two, 7.3 with all five; 256 x 256 (128 CTAs)
+// 10.3 with two, 9.9 with three, 11.6 with five; 512 x 256 (256 CTAs) 11.9 with two, 13.6 with three.
+int mlp_stages_beside(int B, int H1, int S, int sms) {
+    const int64_t ctas = int64_t((B + kMlpM - 1) / kMlpM) * ((H1 + kMlpN - 1) / kMlpN) * S;
+    return 2 * ctas <= sms ? 0 : (ctas <= sms ? 3 : 2);
+}
+
 bool mlp_shape_ok(int d, int H1) {
     const int nchunks = (d + kMlpKc - 1) / kMlpKc;
     const int s = mlp_split(d);
@@ -264,15 +300,16 @@ bool mlp_shape_ok(int d, int H1) {
 
 int mlp_hidden_padded(int H1) { return (H1 + kMlpN - 1) / kMlpN * kMlpN; }
 
-cudaError_t launch_mlp_tc(const uint16_t *hidden, const uint16_t *W1, float *part, int B, int d, int H1,
+cudaError_t launch_mlp_tc(const uint16_t *hidden, const uint16_t *W1, float *part, int B, int d, int H1, int S,
                           bool prefetch, cudaStream_t stream, int stages) {
     CUtensorMap tm_h, tm_w;
     if (!encode_rows(&tm_h, hidden, B, d, kMlpM) || !encode_rows(&tm_w, W1, H1, d, kMlpN))
         return cudaErrorInvalidValue;
     const int nchunks = (d + kMlpKc - 1) / kMlpKc;
-    const int S = mlp_split(d);
-    const int per = (nchunks + S - 1) / S;
-    const int st = stages >= 1 && stages < per ? stages : per;
+    const int parts = mlp_split(d);
+    const int per = (parts / S) * ((nchunks + parts - 1) / parts);  // a CTA's chunks
+    const int most = stages >= 1 && stages < kMaxMlpChunks ? stages : kMaxMlpChunks;
+    const int st = per < most ? per : most;
     // the operand stages, which also hold the output tile (kMlpM x kMlpN fp32) once the MMAs are done
     const size_t smem = 1024 + std::max(size_t(st) * (kAChunk + kBChunk), size_t(kMlpM) * kMlpN * 4);
     static bool attr_done[64] = {false};
@@ -291,6 +328,8 @@ cudaError_t launch_mlp_tc(const uint16_t *hidden, const uint16_t *W1, float *par
     a.nchunks = nchunks;
     a.prefetch = prefetch ? 1 : 0;
     a.stages = st;
+    a.parts = parts;
+    a.columns = kMlpN * (parts / S);
     const dim3 grid(unsigned(S), unsigned(a.H1p / kMlpN), unsigned((B + kMlpM - 1) / kMlpM));
     // An explicit one-CTA cluster: the copies and the MMA commit address shared::cluster.
     return launch_pdl(mlp_tc_kernel, grid, dim3(kMlpThreads), smem, stream, 1u, tm_h, tm_w, a);

@@ -6,24 +6,28 @@
 
 namespace switchsd {
 
-constexpr int kMaxMlpSplit = 16;    // CTAs splitting K
+constexpr int kMaxMlpSplit = 16;    // parts of K
 constexpr int kMaxMlpChunks = 8;    // 64-element K chunks staged per CTA: d <= 16 * 8 * 64 = 8192
 constexpr int kMaxMlpHidden = 1024; // H1: at most 16 tiles of 64 units
-constexpr int kMlpStagesBeside = 2; // chunks staged at once when the rescan kernel runs beside it
 
-// K split used for hidden size d: the partial sums per (row, unit).
+// Parts of K for hidden size d: the most partial sums per (row, unit).
 int mlp_split(int d);
+// CTAs per tile of 128 rows x 64 units, each with an equal share of the parts: the partial sums per (row, unit)
+// of a launch.  A power of two, at most mlp_split(d).
+int mlp_ctas_per_tile(int B, int d, int H1);
+// Chunks a CTA stages at once when the rescan kernel runs beside the launch (0: all of them).
+int mlp_stages_beside(int B, int H1, int S, int sms);
 // Whether (d, H1) is within the kernel's limits.
 bool mlp_shape_ok(int d, int H1);
 // H1 rounded up to the 64-unit tile: the row stride of the partial sums.
 int mlp_hidden_padded(int H1);
-// part [mlp_split(d)][B][mlp_hidden_padded(H1)] <- split-K partial sums of W1 h (fp32; units >= H1 are
-// zero).  Launched with programmatic stream serialization; prefetch: the hidden states and W1 may be
+// part [S][B][mlp_hidden_padded(H1)] <- split-K partial sums of W1 h (fp32; units >= H1 are zero), S =
+// mlp_ctas_per_tile(...).  Launched with programmatic stream serialization; prefetch: the hidden states and W1 may be
 // read (and the MMAs run) before the preceding kernel finishes (the caller's guarantee,
 // SWITCHSD_PREFETCH_PROBE), and the next kernel is released at once; the stores wait.  stages:
 // operand chunks staged at once per CTA (0 or >= the CTA's chunks: all of them; fewer leave shared memory
 // to a kernel that runs beside this one).
-cudaError_t launch_mlp_tc(const uint16_t *hidden, const uint16_t *W1, float *part, int B, int d, int H1,
+cudaError_t launch_mlp_tc(const uint16_t *hidden, const uint16_t *W1, float *part, int B, int d, int H1, int S,
                           bool prefetch, cudaStream_t stream, int stages = 0);
 
 }  // namespace switchsd

@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     const bool pf_probe = (a.prefetch & SWITCHSD_PREFETCH_PROBE) != 0 && !gather && !mlp;
     // Two-layer probe: every input but the partial sums was written by kernels that completed before the
     // first-layer kernel released this launch (it does so only after its own wait), so verification and
-    // scan run while it computes; warps 1.. wait just before reading the sums.  Reads before that wait
+    // scan run while it computes; the warps wait just before reading the sums.  Reads before that wait
     // go through L2 (bulk copies, ld.global.cg).
     const bool late = mlp && a.wait_late != 0;
     if (!pf_ctx && !late) pdl_wait();
@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     if (!pf_probe && !gather && !mlp && tid == 0) issue_probe();
 
     // Two-layer probe: this CTA finishes units [u0m, u1m) (the S partial sums in order, b1, ReLU, w2);
-    // thread j = tid - 32 of warps 1.. takes units u0m + j, u0m + j + (kT - 32), ...  When this launch's
+    // thread j takes units u0m + j, u0m + j + kT, ...  When this launch's
     // wait already covers the first-layer kernel (not late), the first unit's partial sums are loaded
     // now, so that their round trip overlaps the verification's; the sums are taken after it.
     const int uper = mlp ? (a.H1 + int(C) - 1) / int(C) : 0;
@@ -510,15 +510,15 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     // every partial sum of a unit is loaded before the first add (independent L2 reads), then added in
     // order; the same threads and order either way, so the logit does not depend on when this runs
     auto mlp_finish = [&](int from) {
-        for (int u = from; u < u1m; u += kRescanThreads - kWarp) {
+        for (int u = from; u < u1m; u += kRescanThreads) {
             float pz[kMaxMlpSplit];
             mlp_load(u, pz);
             zp = mlp_unit(u, pz, zp);
         }
     };
-    const bool mlp_early = mlp && !late && warp >= 1;
+    const bool mlp_early = mlp && !late;
     float pz0[kMaxMlpSplit];
-    const int u_first = u0m + tid - kWarp;
+    const int u_first = u0m + tid;
     if (mlp_early && u_first < u1m) mlp_load(u_first, pz0);
 
     // ---- verification of the previous draft (every warp) ----
@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     }
     if (mlp_early && u_first < u1m) {
         zp = mlp_unit(u_first, pz0, zp);
-        mlp_finish(u_first + (kRescanThreads - kWarp));
+        mlp_finish(u_first + kRescanThreads);
     }
     // The probed state of a fused verification with hidden_rows = k + 1: row a_b (row 0 when nothing was
     // appended).  Its words are loaded now and used after the scan.
@@ -836,11 +836,11 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     }
 
     // ---- probe share (unless finished before the wait) ----
-    if (warp >= 1) {
-        if (late) {  // the partial sums only now: this launch waits for the first-layer kernel here
-            pdl_wait();
-            mlp_finish(u0m + tid - kWarp);
-        } else if (mlp) {
+    if (late) {  // the partial sums only now: this launch waits for the first-layer kernel here
+        pdl_wait();
+        mlp_finish(u0m + tid);
+    } else if (warp >= 1) {
+        if (mlp) {
             // finished after the verification (mlp_early)
         } else if (gather) {
             zp = dot8_bf16(gw, gh, 0.f);  // zero words for a thread past the slice

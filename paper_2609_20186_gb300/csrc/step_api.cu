@@ -306,16 +306,17 @@ static int step_entry(int32_t *ctx_tokens, int32_t *ctx_lens, const uint16_t *hi
             probe_pf = false;  // the probe kernel's input was just written by the gather
             args.hidden_rows = 1;
         }
-        // Beside the rescan kernel the first layer stages two chunks at a time, so that every CTA of the
+        // Beside the rescan kernel the first layer stages few chunks at a time, so that every CTA of the
         // rescan kernel fits on the GPU while it runs (that kernel verifies and scans meanwhile).
-        if (launch_mlp_tc(probe_in, probe_w, part, p->B, p->d, p->probe_hidden, probe_pf, stream,
-                          p->index == nullptr ? kMlpStagesBeside : 0) != cudaSuccess)
+        const int sms = sm_count_cached() > 0 ? sm_count_cached() : 148;
+        args.mlp_S = mlp_ctas_per_tile(p->B, p->d, p->probe_hidden);
+        if (launch_mlp_tc(probe_in, probe_w, part, p->B, p->d, p->probe_hidden, args.mlp_S, probe_pf, stream,
+                          p->index == nullptr ? mlp_stages_beside(p->B, p->probe_hidden, args.mlp_S, sms) : 0) != cudaSuccess)
             return SWITCHSD_ERR_CUDA;
         args.z1_part = part;
         mlp_early = probe_pf;
         args.b1 = p->b1;
         args.w2 = probe_w + size_t(p->probe_hidden) * size_t(p->d);
-        args.mlp_S = mlp_split(p->d);
         args.H1 = p->probe_hidden;
         args.H1p = mlp_hidden_padded(p->probe_hidden);
     }
