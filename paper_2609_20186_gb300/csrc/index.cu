@@ -19,7 +19,7 @@
 // tokens compared, the next link and the tokens that follow it.  The lookup starts from the link that the
 // insert of the suffix's own end found, and the draft is written from the registers of the n that wins.  16
 // rows of 128K tokens, n = 2..12, 16 launches: 82.6 us with the heads and links read again for the lookup and
-// the draft gathered at the end (seven round trips), 74.4 us so.
+// the draft gathered at the end (seven round trips), 71.7 us so.
 // Candidate mode (W > 0, as switchsd_step_candidates / switchsd_verify_candidates): the previous W
 // candidates are verified and the longest accepted one appended; the warp of n = kappa walks its
 // chain on past the first match and lists the W most recent ends whose kappa-gram equals the
@@ -42,23 +42,23 @@ namespace switchsd {
 constexpr int kIdxMaxWarps = SWITCHSD_NMAX;
 constexpr int kIdxTail = SWITCHSD_NMAX + SWITCHSD_KMAX + 1;  // staged context tail: old end +- the append
 
-// Hash of the n tokens ending at the last one (`tok(i)` = token i steps back): a polynomial in an odd
-// multiplier mod 2^32, whose terms are independent (one multiply-add each, no chain through a mixer), then
-// two multiply-xorshift rounds; the bucket is its top bits.
+// Hash of the n tokens ending at the last one (`tok(i)` = token i steps back): the sum of their products with
+// the powers of an odd multiplier, whose terms are independent (one multiply-add each, no chain through a
+// mixer), in 64 bits so that tokens that differ in their high bits alone still spread, then one
+// multiply-xorshift round; the bucket is its top bits.
 constexpr uint32_t kGramMul = 0x9E3779B1u;
-__device__ __forceinline__ uint32_t gram_bucket(uint32_t h, int n, int log2_buckets) {
-    h += uint32_t(n) * 0x85EBCA77u;
+__device__ __forceinline__ uint32_t gram_bucket(uint64_t sum, int n, int log2_buckets) {
+    uint32_t h = uint32_t(sum) + uint32_t(sum >> 32) * 0x7FEB352Du + uint32_t(n) * 0x85EBCA77u;
     h ^= h >> 15;
     h *= 0x2C1B3C6Du;
-    h ^= h >> 13;
-    h *= 0x297A2D39u;
     return h >> (32 - log2_buckets);
 }
 template <typename Tok>
 __device__ __forceinline__ uint32_t gram_hash(int n, Tok tok, int log2_buckets) {
-    uint32_t h = 0u, pw = 1u;
+    uint64_t h = 0u;
+    uint32_t pw = 1u;
     for (int i = 0; i < n; ++i) {
-        h += uint32_t(tok(i)) * pw;
+        h += uint64_t(uint32_t(tok(i))) * pw;
         pw *= kGramMul;
     }
     return gram_bucket(h, n, log2_buckets);
@@ -434,14 +434,18 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
 // from the table its own bins' warp wrote (same warp, earlier chunk) and updates only the heads it moved.
 //
 // Why: one warp per item walking its row 32 positions at a time (a dependent head read and write each) took
-// 1210 us for 64 rows of 32K tokens, n = 3..8 (build and one step); this takes 155 us (177 us with the ranks taken by
-// eight ballots a position and counted in a pass of their own).  The table written sets
-// the floor (201 MB of heads + 50 MB of links: 37 us at the measured copy bandwidth); what bounds it is the
-// issue rate and latency of the five phases at one 1024-thread CTA an SM (384 CTAs: 2.5 waves).
+// 1210 us for 64 rows of 32K tokens, n = 3..8 (build and one step); this takes 150 us.  Ranks by eight ballots a
+// position, counted in a pass of their own: 177 us; the groups of equal keys in a round of step 4 by nine ballots
+// (six rounds in ten hold one): 155 us.  The tokens staged in shared memory by one copy made no difference.  The
+// table written sets the floor (201 MB of heads + 50 MB of links: 37 us at the measured copy bandwidth); what
+// bounds it is the issue rate (ALU and shared-memory pipes each at half of their peak) at one 1024-thread CTA an
+// SM, 2.5 waves of them here.
 // ------------------------------------------------------------------------------------------------
 constexpr int kBuildKeyBits = 9;
 constexpr int kBuildBins = 256;
-constexpr int kRankShift = kBuildKeyBits + 8;  // a segment's rank within a bin (at most 1024) above bin and key
+constexpr int kLocalBits = kBuildKeyBits + 8;  // a bucket within its part: bin and key.  A position's rank within
+                                               // its segment and bin (below 1024), and in the queue its place in
+                                               // the chunk (15 bits), stand above it.
 constexpr uint32_t kNone16 = 0xffffu;  // no earlier entry; kDone16: the link is in global memory already
 constexpr uint32_t kDone16 = 0xfffeu;
 
@@ -462,22 +466,8 @@ struct BuildLayout {
     static constexpr size_t bytes = queue + links + heads;
 };
 
-// The lanes of `live` that hold the same kBits-bit value as this one, one ballot a bit (every lane calls it; a
-// lane outside `live` is in no other lane's mask).  On this GPU __match_any_sync on 32 mostly distinct values
-// costs more issue slots than the kBits ballots.
-template <int kBits>
-__device__ __forceinline__ unsigned same_value_lanes(uint32_t v, unsigned live) {
-    unsigned m = live;
-#pragma unroll
-    for (int i = 0; i < kBits; ++i) {
-        const bool set = (v >> i & 1u) != 0u;
-        m &= __ballot_sync(kFull, set) ^ (set ? 0u : ~0u);
-    }
-    return m;
-}
-
 template <int kT, int kChunk>
-__global__ void __launch_bounds__(kT) index_build_kernel(const BuildArgs a) {
+__global__ void __launch_bounds__(kT, 1024 / kT) index_build_kernel(const BuildArgs a) {
     using Lay = BuildLayout<kT, kChunk>;
     constexpr int kW = Lay::kW;
     constexpr int kIts = kChunk / kT;  // positions a thread holds
@@ -496,7 +486,7 @@ __global__ void __launch_bounds__(kT) index_build_kernel(const BuildArgs a) {
     const int n = a.n_min + w;
     const int lg = a.log2_buckets, lgp = lg - a.log2_parts;  // bucket bits, and those within the part
     const int binbits = lgp < 8 ? lgp : 8, keybits = lgp - binbits;
-    const uint32_t keymask = (1u << keybits) - 1u;
+    const uint32_t keymask = (1u << keybits) - 1u, localmask = (1u << lgp) - 1u;
     pdl_wait();
     pdl_trigger();
     int32_t *heads = a.heads + (size_t(w) * a.B + b) * (size_t(1) << lg) + (size_t(part) << lgp);
@@ -516,10 +506,11 @@ __global__ void __launch_bounds__(kT) index_build_kernel(const BuildArgs a) {
 
         // 1. hash and rank
         uint32_t *mask = reinterpret_cast<uint32_t *>(H), *my = cnt + warp * (kBuildBins + 1);
-        uint32_t code[kIts];  // rank << kRankShift | bin << kBuildKeyBits | key, all ones for a dropped position
+        uint32_t code[kIts];  // rank << kLocalBits | the bucket in the part, all ones for a dropped position
+        const int32_t p_end = min(L, p_seg + seg);
 #pragma unroll
         for (int r = 0; r < kIts / 8; ++r) {
-            uint32_t h[8];
+            uint64_t h[8];
             const int32_t p0 = p_seg + 256 * r;
 #pragma unroll
             for (int u = 0; u < 8; ++u) h[u] = 0u;
@@ -529,20 +520,20 @@ __global__ void __launch_bounds__(kT) index_build_kernel(const BuildArgs a) {
                     const int32_t *x = row + p0 + lane;
                     for (int i = 0; i < n; ++i, --x, pw *= kGramMul)
 #pragma unroll
-                        for (int u = 0; u < 8; ++u) h[u] += uint32_t(__ldg(x + 32 * u)) * pw;
+                        for (int u = 0; u < 8; ++u) h[u] += uint64_t(uint32_t(__ldg(x + 32 * u))) * pw;
                 } else {
                     for (int i = 0; i < n; ++i, pw *= kGramMul)
 #pragma unroll
                         for (int u = 0; u < 8; ++u)
-                            h[u] += uint32_t(__ldg(row + min(max(p0 + lane + 32 * u - i, 0), L - 1))) * pw;
+                            h[u] += uint64_t(uint32_t(__ldg(row + min(max(p0 + lane + 32 * u - i, 0), L - 1)))) * pw;
                 }
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int32_t p = p0 + 32 * u + lane;
                 const uint32_t bucket = gram_bucket(h[u], n, lg);
-                const bool mine = 256 * r + 32 * u < seg && p < L && p >= n - 1 && int(bucket >> lgp) == part;
-                const uint32_t local = bucket & ((1u << lgp) - 1u);
+                const bool mine = p >= n - 1 && p < p_end && int(bucket >> lgp) == part;
+                const uint32_t local = bucket & localmask;
                 const uint32_t bin = local >> keybits;
                 if (mine) atomicOr(&mask[bin], 1u << lane);
                 __syncwarp();
@@ -553,9 +544,7 @@ __global__ void __launch_bounds__(kT) index_build_kernel(const BuildArgs a) {
                     my[bin] = at + uint32_t(__popc(peers));
                     mask[bin] = 0u;
                 }
-                code[8 * r + u] = mine ? ((at + uint32_t(__popc(below))) << kRankShift | bin << kBuildKeyBits |
-                                          (local & keymask))
-                                       : 0xffffffffu;
+                code[8 * r + u] = mine ? (at + uint32_t(__popc(below))) << kLocalBits | local : 0xffffffffu;
                 __syncwarp();
             }
         }
@@ -599,9 +588,9 @@ __global__ void __launch_bounds__(kT) index_build_kernel(const BuildArgs a) {
         for (int i = 0; i < kIts; ++i) {
             const uint32_t c = code[i];
             if (c != 0xffffffffu) {
-                const uint32_t bin = c >> kBuildKeyBits & uint32_t(kBuildBins - 1);
+                const uint32_t local = c & ((1u << kLocalBits) - 1u), bin = local >> keybits;
                 const uint32_t lp = uint32_t(p_seg - c0 + 32 * i + lane);
-                q[s_bin[bin] + my[bin] + (c >> kRankShift)] = lp << kBuildKeyBits | (c & ((1u << kBuildKeyBits) - 1u));
+                q[s_bin[bin] + my[bin] + (c >> kLocalBits)] = lp << kLocalBits | local;
             }
         }
         __syncthreads();  // the counters are dead from here on: the links take their place
@@ -617,22 +606,25 @@ __global__ void __launch_bounds__(kT) index_build_kernel(const BuildArgs a) {
             // one round of 32 entries: (position, link), the link kNone16 when the bin holds no earlier entry
             auto round = [&](uint32_t base, bool live, uint32_t &key, uint32_t &lp) {
                 const uint32_t ent = live ? q[base + lane] : 0u;
-                key = ent & ((1u << kBuildKeyBits) - 1u);
-                lp = ent >> kBuildKeyBits;
+                key = ent & keymask;
+                lp = ent >> kLocalBits;
                 uint32_t l16 = live ? uint32_t(H[key]) : kNone16;
                 __syncwarp();  // every lane has read its head before any lane replaces one
                 if (live) H[key] = uint16_t(lp);
                 __syncwarp();
-                // Two entries of one key in a round are rare: then the group is found by ballots, each entry
-                // links to the one before it and the last is the head.
-                if (__any_sync(kFull, live && uint32_t(H[key]) != lp)) {
-                    const unsigned peers = same_value_lanes<kBuildKeyBits>(key, __ballot_sync(kFull, live));
+                // Entries of one key in a round: one of them holds H now, the others see it.  Such a group
+                // (one a round, mostly two entries) links each entry to the one before it; the last is the head.
+                for (unsigned todo = __ballot_sync(kFull, live && uint32_t(H[key]) != lp); todo != 0u;) {
+                    const uint32_t k = __shfl_sync(kFull, key, __ffs(todo) - 1);
+                    const bool in = live && key == k;
+                    const unsigned peers = __ballot_sync(kFull, in);
                     const unsigned earlier = peers & ((1u << lane) - 1u);
                     const uint32_t before = __shfl_sync(kFull, lp, earlier ? 31 - __clz(earlier) : lane);
-                    if (earlier) l16 = before;
-                    if (live && (peers >> lane) == 1u) H[key] = uint16_t(lp);
-                    __syncwarp();
+                    if (in && earlier) l16 = before;
+                    if (in && (peers >> lane) == 1u) H[key] = uint16_t(lp);
+                    todo &= ~peers;
                 }
+                __syncwarp();
                 return l16;
             };
             uint32_t key, lp;
