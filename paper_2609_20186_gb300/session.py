@@ -76,6 +76,7 @@ class Session:
         if d is None:
             d = probe_w_bits.size if probe_kind == bd.PROBE_LINEAR else None
         self.d = d
+        self._hidden_shape = (B, d)  # of a [B, d] hidden state, once d is known
 
         # workspace of the two-layer probe (none for the linear probe)
         probe = bd.switchsd_params()
@@ -109,6 +110,12 @@ class Session:
             p.counters = self.counters.data_ptr() if self.counters is not None else None
             return p
         self._p_dbg, self._p_fast = params(True), params(False)
+        # switchsd_step alone takes hidden as [B, d] whatever hidden_rows is: its own blocks (the calls then only
+        # pick one; both kinds share every buffer)
+        self._ps_dbg, self._ps_fast = params(True), params(False)
+        self._ps_dbg.hidden_rows = self._ps_fast.hidden_rows = 0
+        self._step_fn = self.lib.switchsd_step
+        self._step_refs = (ctypes.byref(self._ps_fast), ctypes.byref(self._ps_dbg))
         self._step_head = (self.ctx.data_ptr(), self.lens.data_ptr())
         self._step_tail = (self.probe_w.data_ptr(),)
         self._step_outs = (self.draft.data_ptr(), self.len.data_ptr(), self.mode.data_ptr(),
@@ -157,6 +164,9 @@ class Session:
     # --- the three calls ---------------------------------------------------------------------
     def _check_hidden(self, hidden: torch.Tensor, rows: int = 1) -> None:
         """hidden: bf16 [B, d], or [B, rows, d] when rows > 1 (the fused verification's gather)."""
+        if (rows <= 1 and hidden.shape == self._hidden_shape and hidden.dtype == torch.bfloat16
+                and hidden.is_contiguous() and hidden.device == self.device):
+            return
         shape_ok = hidden.shape[0] == self.B and (
             (rows <= 1 and hidden.dim() == 2) or (rows > 1 and hidden.dim() == 3 and hidden.shape[1] == rows))
         if (hidden.dtype != torch.bfloat16 or hidden.device != self.device
@@ -164,17 +174,16 @@ class Session:
                 or (self.d is not None and hidden.shape[-1] != self.d)):
             raise ValueError("hidden must be a contiguous bf16 [B, d] (or [B, k+1, d]) tensor on the session device")
         if self.d is None:
-            self._p_dbg.d = self._p_fast.d = hidden.shape[1]
+            for p in (self._p_dbg, self._p_fast, self._ps_dbg, self._ps_fast):
+                p.d = hidden.shape[1]
             self.d = hidden.shape[1]
+            self._hidden_shape = (self.B, self.d)
 
     def step(self, hidden: torch.Tensor, debug: bool = True) -> None:
         """switchsd_step (no verification): hidden is [B, d] whatever hidden_rows is."""
         self._check_hidden(hidden)
-        p = self._p_dbg if debug else self._p_fast
-        rows, p.hidden_rows = p.hidden_rows, 0
-        code = self.lib.switchsd_step(*self._step_head, hidden.data_ptr(), *self._step_tail,
-                                      ctypes.byref(p), *self._step_outs)
-        p.hidden_rows = rows
+        code = self._step_fn(*self._step_head, hidden.data_ptr(), *self._step_tail, self._step_refs[bool(debug)],
+                             *self._step_outs)
         if code != bd.OK:
             raise RuntimeError(f"switchsd_step failed: {code} ({bd.strerror(code)})")
 
@@ -271,11 +280,8 @@ class Session:
         call.  With synchronize the call returns when results_host is filled.  Returns its views."""
         self._check_hidden(hidden)
         io = self._host_io(hidden_host, hidden, results_host, synchronize)
-        p = self._p_dbg if debug else self._p_fast
-        rows, p.hidden_rows = p.hidden_rows, 0
         code = self.lib.switchsd_step_host(ctypes.byref(io), *self._step_head, hidden.data_ptr(), *self._step_tail,
-                                           ctypes.byref(p), *self._step_outs)
-        p.hidden_rows = rows
+                                           self._step_refs[bool(debug)], *self._step_outs)
         if code != bd.OK:
             raise RuntimeError(f"switchsd_step_host failed: {code} ({bd.strerror(code)})")
         return self._host_views(results_host)
