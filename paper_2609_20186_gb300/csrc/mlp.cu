@@ -3,9 +3,9 @@
 // The paper's probe is linear (Eq. 3); this two-layer form is an extension used with probe_kind
 // SWITCHSD_PROBE_MLP.  Its first layer is a real contraction, Z1[B, H1] = H[B, d] . W1[H1, d]^T, so it
 // runs on tcgen05.  K = d is split into P = mlp_split(d) parts, of which a CTA takes A = P / S: CTA (s, n, m)
-// stages the K chunks of its parts of H rows [128 m, +128) and W1 units [64 n, +64) in shared memory with TMA
+// stages the K chunks of its parts of H rows [128 m, +128) and W1 units [N n, +N) in shared memory with TMA
 // (128-byte swizzle, zero fill past the tensor edges), one thread issues tcgen05.mma (bf16 x bf16, fp32
-// accumulators in 64 TMEM columns a part), the four warps read their 32 rows of the A parts back with
+// accumulators in N TMEM columns a part), the four warps read their 32 rows of the A parts back with
 // tcgen05.ld, add them in order and store the partial sums
 //     part[s][b][u]  (fp32, s < S, b < B, u < H1p = H1 rounded up to 64; units >= H1 hold zeros).
 // The step kernel that follows adds the S partials of its row in order, then b1, ReLU, w2 and b2: every
@@ -24,18 +24,17 @@
 namespace switchsd {
 
 constexpr int kMlpM = 128;             // rows (sequences) per tile: the MMA's M
-constexpr int kMlpN = 64;              // hidden units per tile: the MMA's N
 constexpr int kMlpKc = 64;             // K elements per staged chunk: one 128-byte swizzle row
 constexpr int kMlpThreads = 128;       // four warps: one per 32 TMEM lanes
 constexpr uint32_t kAChunk = kMlpM * kMlpKc * 2;    // 16 KB
-constexpr uint32_t kBChunk = kMlpN * kMlpKc * 2;    // 8 KB
-static_assert(kMaxMlpChunks * (kAChunk + kBChunk) + 1024 + 64 <= 227 * 1024,
-              "operands, alignment slack and static shared memory must fit one CTA");
-static_assert(kMlpThreads == kMlpM && kMlpN == 64, "one thread per tile row; 16 chunks of 16 bytes per row");
+static_assert(kMlpThreads == kMlpM, "one thread per tile row");
 
-// Instruction descriptor of tcgen05.mma kind::f16: D fp32, A and B bf16, both K-major, M = 128, N = 64.
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(kMlpN >> 3) << 17) |
-                            (uint32_t(kMlpM >> 4) << 24);
+// Of a tile of N hidden units (the MMA's N): a staged chunk of W1, and the instruction descriptor of
+// tcgen05.mma kind::f16 (D fp32, A and B bf16, both K-major, M = 128).
+template <int N>
+constexpr uint32_t kBChunk = uint32_t(N * kMlpKc * 2);
+template <int N>
+constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(N >> 3) << 17) | (uint32_t(kMlpM >> 4) << 24);
 
 struct MlpArgs {
     float *part;   // [S][B][H1p]
@@ -73,6 +72,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+template <int N>
 __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_constant__ CUtensorMap tm_h,
                                                              const __grid_constant__ CUtensorMap tm_w,
                                                              const MlpArgs a) {
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int S = int(gridDim.x), ks = blockIdx.x;
-    const int n_tile = blockIdx.y, m0 = blockIdx.z * kMlpM, n0 = n_tile * kMlpN;
+    const int n_tile = blockIdx.y, m0 = blockIdx.z * kMlpM, n0 = n_tile * N;
     const int A = a.parts / S;                           // this CTA's parts
     const int per = (a.nchunks + a.parts - 1) / a.parts;  // chunks of a part (fewer, or none, at the end of K)
     const int c0 = ks * A * per;
@@ -94,9 +94,9 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
     uint8_t *opB = base + size_t(st) * kAChunk;
     auto issue = [&](int c) {  // chunk c of this CTA's K slice into stage c % st
         const int sg = c % st;
-        mbar_arrive_expect_tx(&full[sg], kAChunk + kBChunk);
+        mbar_arrive_expect_tx(&full[sg], kAChunk + kBChunk<N>);
         tma_load_2d(opA + size_t(sg) * kAChunk, &tm_h, (c0 + c) * kMlpKc, m0, &full[sg]);
-        tma_load_2d(opB + size_t(sg) * kBChunk, &tm_w, (c0 + c) * kMlpKc, n0, &full[sg]);
+        tma_load_2d(opB + size_t(sg) * kBChunk<N>, &tm_w, (c0 + c) * kMlpKc, n0, &full[sg]);
     };
     const int first = min(nck, st);  // chunks issued up front
 
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
             landed = c + 1;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const uint64_t da = sw128_desc(smem_addr(opA + size_t(sg) * kAChunk));
-            const uint64_t db = sw128_desc(smem_addr(opB + size_t(sg) * kBChunk));
+            const uint64_t db = sw128_desc(smem_addr(opB + size_t(sg) * kBChunk<N>));
 #pragma unroll
             for (int j = 0; j < kMlpKc / 16; ++j) {
                 const uint32_t acc = ((c % per) | j) != 0;  // a part starts from zero in its own columns
@@ -158,8 +158,8 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
                     ".reg .pred p;\n"
                     "setp.ne.b32 p, %4, 0;\n"
                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
-                    "}\n" ::"r"(tmem + uint32_t(kMlpN * (c / per))),
-                    "l"(da + uint64_t(2 * j)), "l"(db + uint64_t(2 * j)), "r"(kIdesc), "r"(acc)
+                    "}\n" ::"r"(tmem + uint32_t(N * (c / per))),
+                    "l"(da + uint64_t(2 * j)), "l"(db + uint64_t(2 * j)), "r"(kIdesc<N>), "r"(acc)
                     : "memory");
             }
             if (c + st < nck) {
@@ -193,13 +193,14 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
     // Row tid of the tile: its 64 accumulators, the parts added in order (zero when this CTA had no K chunk;
     // NaN when a copy or the MMAs did not complete in time, so the row's logit shows the failure).  The tile
     // goes out through shared memory (the operand stages are free: every MMA has completed), so that each warp
-    // store writes two whole 256-byte rows instead of one 16-byte piece of 32 rows.  Row r keeps its 16-byte
+    // store writes whole rows instead of one 16-byte piece of 32 rows.  Row r keeps its 16-byte
     // chunk q at position q ^ (r % 16): both the row-wise writes here and the reads across rows below hit
     // distinct banks.
-    float4 *tile = reinterpret_cast<float4 *>(base);  // [kMlpM rows][16 chunks]
+    constexpr int kQ = N / 4;  // 16-byte chunks of a row
+    float4 *tile = reinterpret_cast<float4 *>(base);  // [kMlpM rows][kQ]
     const uint32_t taddr = tmem + (uint32_t(warp * 32) << 16);
 #pragma unroll 1
-    for (int g = 0; g < kMlpN; g += 32) {
+    for (int g = 0; g < N; g += 32) {
         float v[32];
         if (nck > 0 && ok) {
             tmem_ld32(taddr + uint32_t(g), v);
@@ -207,7 +208,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
 #pragma unroll 1
             for (int p = 1; p * per < nck; ++p) {
                 float w[32];
-                tmem_ld32(taddr + uint32_t(kMlpN * p + g), w);
+                tmem_ld32(taddr + uint32_t(N * p + g), w);
                 asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
                 for (int i = 0; i < 32; ++i) v[i] += w[i];
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
         }
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-            tile[tid * 16 + ((g / 4 + q) ^ (tid & 15))] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            tile[tid * kQ + ((g / 4 + q) ^ (tid & 15))] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
     }
     // The partial sums overwrite what an earlier step kernel may still read: with the prefetch bit the copies
     // and the MMAs above ran before the wait, the stores come after it.
@@ -227,11 +228,11 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
 #pragma unroll 4
-    for (int i = 0; i < 16; ++i) {  // warp w writes rows 32 w .. 32 w + 31, two per store
-        const int r = warp * 32 + 2 * i + (lane >> 4), c = lane & 15;
+    for (int i = lane; i < kWarp * kQ; i += kWarp) {  // warp w writes rows 32 w .. 32 w + 31, whole rows at a time
+        const int r = warp * kWarp + i / kQ, c = i % kQ;
         if (m0 + r < a.B)
             reinterpret_cast<float4 *>(a.part + (size_t(ks) * a.B + size_t(m0 + r)) * a.H1p + n0)[c] =
-                tile[r * 16 + (c ^ (r & 15))];
+                tile[r * kQ + (c ^ (r & 15))];
     }
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(a.columns) : "memory");
@@ -273,6 +274,10 @@ int mlp_split(int d) {
     return s;
 }
 
+static size_t mlp_most_partials(int B, int d, int H1) {  // bytes, with every part its own CTA
+    return size_t(mlp_split(d)) * size_t(B) * size_t(mlp_hidden_padded(H1)) * sizeof(float);
+}
+
 int mlp_ctas_per_tile(int B, int d, int H1) {
     const int parts = mlp_split(d);
     // With every part its own CTA, parts x B x H1p floats go through memory.  Past 10 MB two parts a CTA are
@@ -280,15 +285,22 @@ int mlp_ctas_per_tile(int B, int d, int H1) {
     // 256 units (4 MB) 10.3 and 13.6 us, 512 x 256 (8 MB) 11.8 and 14.2, 130 x 1024 (8.5 MB) 13.2 and 14.4,
     // 768 x 256 (12.6 MB) 18.6 and 17.2, 400 x 512 (13 MB) 20.7 and 15.3, 768 x 512 (25 MB) 25.1 and 21.0 (four
     // parts a CTA: 23.3).
-    const size_t bytes = size_t(parts) * size_t(B) * size_t(mlp_hidden_padded(H1)) * sizeof(float);
-    return parts > 1 && bytes > 10u * 1000u * 1000u ? parts / 2 : parts;
+    return parts > 1 && mlp_most_partials(B, d, H1) > 10u * 1000u * 1000u ? parts / 2 : parts;
+}
+
+// Tiles of 128 units where H1p divides into them and the partial sums call for two parts a CTA: the operands' L2
+// traffic, which bounds those grids, falls by a third (a step of 768
+// rows x 512 units 21.1 us with tiles of 64, 19.0 of 128; 400 x 512 15.4 and 14.9; 768 x 256 16.9 and 16.6).
+static bool mlp_wide(int B, int d, int H1) {
+    return mlp_hidden_padded(H1) % (2 * kMlpNMin) == 0 && mlp_ctas_per_tile(B, d, H1) < mlp_split(d);
 }
 
 // A grid of at most half the SMs stages all its chunks at once, one of at most a CTA an SM three, a larger one
 // two: a step of 64 rows x 256 units (64 CTAs) takes 8.4 us with two, 7.3 with all five; 256 x 256 (128 CTAs)
 // 10.3 with two, 9.9 with three, 11.6 with five; 512 x 256 (256 CTAs) 11.9 with two, 13.6 with three.
-int mlp_stages_beside(int B, int H1, int S, int sms) {
-    const int64_t ctas = int64_t((B + kMlpM - 1) / kMlpM) * ((H1 + kMlpN - 1) / kMlpN) * S;
+int mlp_stages_beside(int B, int d, int H1, int S, int sms) {
+    const int N = mlp_wide(B, d, H1) ? 2 * kMlpNMin : kMlpNMin;
+    const int64_t ctas = int64_t((B + kMlpM - 1) / kMlpM) * ((H1 + N - 1) / N) * S;
     return 2 * ctas <= sms ? 0 : (ctas <= sms ? 3 : 2);
 }
 
@@ -298,26 +310,28 @@ bool mlp_shape_ok(int d, int H1) {
     return (nchunks + s - 1) / s <= kMaxMlpChunks && H1 >= 1 && H1 <= kMaxMlpHidden && d >= 8 && d % 8 == 0;
 }
 
-int mlp_hidden_padded(int H1) { return (H1 + kMlpN - 1) / kMlpN * kMlpN; }
+int mlp_hidden_padded(int H1) { return (H1 + kMlpNMin - 1) / kMlpNMin * kMlpNMin; }
 
-cudaError_t launch_mlp_tc(const uint16_t *hidden, const uint16_t *W1, float *part, int B, int d, int H1, int S,
-                          bool prefetch, cudaStream_t stream, int stages) {
+template <int N>
+static cudaError_t launch_mlp_n(const uint16_t *hidden, const uint16_t *W1, float *part, int B, int d, int H1, int S,
+                                bool prefetch, cudaStream_t stream, int stages) {
     CUtensorMap tm_h, tm_w;
-    if (!encode_rows(&tm_h, hidden, B, d, kMlpM) || !encode_rows(&tm_w, W1, H1, d, kMlpN))
-        return cudaErrorInvalidValue;
+    if (!encode_rows(&tm_h, hidden, B, d, kMlpM) || !encode_rows(&tm_w, W1, H1, d, N)) return cudaErrorInvalidValue;
     const int nchunks = (d + kMlpKc - 1) / kMlpKc;
     const int parts = mlp_split(d);
     const int per = (parts / S) * ((nchunks + parts - 1) / parts);  // a CTA's chunks
-    const int most = stages >= 1 && stages < kMaxMlpChunks ? stages : kMaxMlpChunks;
+    constexpr int kFit = int((226 * 1024 - 1024) / (kAChunk + kBChunk<N>));  // chunks that fit a CTA
+    const int fit = kFit < kMaxMlpChunks ? kFit : kMaxMlpChunks;
+    const int most = stages >= 1 && stages < fit ? stages : fit;
     const int st = per < most ? per : most;
-    // the operand stages, which also hold the output tile (kMlpM x kMlpN fp32) once the MMAs are done
-    const size_t smem = 1024 + std::max(size_t(st) * (kAChunk + kBChunk), size_t(kMlpM) * kMlpN * 4);
+    // the operand stages, which also hold the output tile (kMlpM x N fp32) once the MMAs are done
+    const size_t smem = 1024 + std::max(size_t(st) * (kAChunk + kBChunk<N>), size_t(kMlpM) * N * 4);
     static bool attr_done[64] = {false};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-        const cudaError_t e = cudaFuncSetAttribute(mlp_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   int(1024 + size_t(kMaxMlpChunks) * (kAChunk + kBChunk)));
+        const cudaError_t e = cudaFuncSetAttribute(mlp_tc_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   int(1024 + size_t(fit) * (kAChunk + kBChunk<N>)));
         if (e != cudaSuccess) return e;
         attr_done[dev] = true;
     }
@@ -329,10 +343,16 @@ cudaError_t launch_mlp_tc(const uint16_t *hidden, const uint16_t *W1, float *par
     a.prefetch = prefetch ? 1 : 0;
     a.stages = st;
     a.parts = parts;
-    a.columns = kMlpN * (parts / S);
-    const dim3 grid(unsigned(S), unsigned(a.H1p / kMlpN), unsigned((B + kMlpM - 1) / kMlpM));
+    a.columns = N * (parts / S);
+    const dim3 grid(unsigned(S), unsigned(a.H1p / N), unsigned((B + kMlpM - 1) / kMlpM));
     // An explicit one-CTA cluster: the copies and the MMA commit address shared::cluster.
-    return launch_pdl(mlp_tc_kernel, grid, dim3(kMlpThreads), smem, stream, 1u, tm_h, tm_w, a);
+    return launch_pdl(mlp_tc_kernel<N>, grid, dim3(kMlpThreads), smem, stream, 1u, tm_h, tm_w, a);
+}
+
+cudaError_t launch_mlp_tc(const uint16_t *hidden, const uint16_t *W1, float *part, int B, int d, int H1, int S,
+                          bool prefetch, cudaStream_t stream, int stages) {
+    return mlp_wide(B, d, H1) ? launch_mlp_n<2 * kMlpNMin>(hidden, W1, part, B, d, H1, S, prefetch, stream, stages)
+                              : launch_mlp_n<kMlpNMin>(hidden, W1, part, B, d, H1, S, prefetch, stream, stages);
 }
 
 }  // namespace switchsd

@@ -8,7 +8,8 @@ namespace switchsd {
 
 constexpr int kMaxMlpSplit = 16;    // parts of K
 constexpr int kMaxMlpChunks = 8;    // 64-element K chunks staged per CTA: d <= 16 * 8 * 64 = 8192
-constexpr int kMaxMlpHidden = 1024; // H1: at most 16 tiles of 64 units
+constexpr int kMaxMlpHidden = 1024; // H1
+constexpr int kMlpNMin = 64;        // hidden units of the smaller tile (the larger has twice as many)
 
 // Parts of K for hidden size d: the most partial sums per (row, unit).
 int mlp_split(int d);
@@ -16,7 +17,7 @@ int mlp_split(int d);
 // of a launch.  A power of two, at most mlp_split(d).
 int mlp_ctas_per_tile(int B, int d, int H1);
 // Chunks a CTA stages at once when the rescan kernel runs beside the launch (0: all of them).
-int mlp_stages_beside(int B, int H1, int S, int sms);
+int mlp_stages_beside(int B, int d, int H1, int S, int sms);
 // Whether (d, H1) is within the kernel's limits.
 bool mlp_shape_ok(int d, int H1);
 // H1 rounded up to the 64-unit tile: the row stride of the partial sums.

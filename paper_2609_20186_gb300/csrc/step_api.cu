@@ -311,7 +311,7 @@ static int step_entry(int32_t *ctx_tokens, int32_t *ctx_lens, const uint16_t *hi
         const int sms = sm_count_cached() > 0 ? sm_count_cached() : 148;
         args.mlp_S = mlp_ctas_per_tile(p->B, p->d, p->probe_hidden);
         if (launch_mlp_tc(probe_in, probe_w, part, p->B, p->d, p->probe_hidden, args.mlp_S, probe_pf, stream,
-                          p->index == nullptr ? mlp_stages_beside(p->B, p->probe_hidden, args.mlp_S, sms) : 0) != cudaSuccess)
+                          p->index == nullptr ? mlp_stages_beside(p->B, p->d, p->probe_hidden, args.mlp_S, sms) : 0) != cudaSuccess)
             return SWITCHSD_ERR_CUDA;
         args.z1_part = part;
         mlp_early = probe_pf;
