@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     const int nv = a.d >> 3;
     const int vper = (nv + int(C) - 1) / int(C);
     const int v0 = min(nv, int(rank) * vper), v1 = min(nv, v0 + vper);
-    const int v_staged = (gather || mlp) ? 0 : min(v1 - v0, a.probe_words);
+    const int v_staged = mlp ? 0 : min(v1 - v0, a.probe_words);
     const uint4 *w4 = reinterpret_cast<const uint4 *>(a.probe_w);
     const uint4 *h4 = reinterpret_cast<const uint4 *>(a.hidden + size_t(b) * size_t(gather ? a.hidden_rows : 1) *
                                                                   size_t(a.d));
@@ -613,15 +613,10 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
         mlp_finish(u_first + kRescanThreads);
     }
     // The probed state of a fused verification with hidden_rows = k + 1: row a_b (row 0 when nothing was
-    // appended).  Its words are loaded now and used after the scan.
-    uint4 gw = make_uint4(0, 0, 0, 0), gh = make_uint4(0, 0, 0, 0);
+    // appended).  Its slice is staged now and used after the scan.
     if (gather) {
         h4 += size_t(acc > 0 ? acc : 0) * size_t(nv);
-        const int v = v0 + tid - kWarp;
-        if (warp >= 1 && v < v1) {
-            gw = __ldg(w4 + v);
-            gh = __ldg(h4 + v);
-        }
+        if (tid == 0) issue_probe();
     }
 
     // ---- this warp's window: y[L_old - kHalo + j], the old tail then the appended tokens ----
@@ -842,10 +837,6 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     } else if (warp >= 1) {
         if (mlp) {
             // finished after the verification (mlp_early)
-        } else if (gather) {
-            zp = dot8_bf16(gw, gh, 0.f);  // zero words for a thread past the slice
-            for (int v = v0 + tid - kWarp + (kRescanThreads - kWarp); v < v1; v += kRescanThreads - kWarp)
-                zp = dot8_bf16(__ldg(w4 + v), __ldg(h4 + v), zp);
         } else if (!pf_probe) {
             probe_dot(h4);
         }
