@@ -45,6 +45,7 @@ constexpr int kKeyShift = 25;
 constexpr uint32_t kKeyEndMask = (1u << kKeyShift) - 1u;
 constexpr uint32_t kKeyTimeout = 1u << 31;
 static_assert(SWITCHSD_NMAX < (1 << (31 - kKeyShift)), "m must fit below the timeout bit");
+static_assert(SWITCHSD_WMAX * SWITCHSD_KMAX <= 1024 && SWITCHSD_KMAX <= 64, "the candidates' division by D");
 // The scan: kScanWords words per thread per round; a thread's words of a CTA range fit the 32 bits of its
 // pass mask.
 constexpr int kScanWords = 4;
@@ -315,6 +316,10 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
         }
         fence_mbar_init();
     }
+    // Candidate mode: i / D for i < W D <= 1024 as (i inv_d) >> 16 (inv_d D - 2^16 < 64, so the error term stays
+    // below 2^16): the divisions leave the chain after the wait.
+    const uint32_t inv_d = kCand ? (65536u + uint32_t(a.D) - 1u) / uint32_t(a.D) : 0u;
+    auto over_d = [&](int i) { return int((uint32_t(i) * inv_d) >> 16); };
     if (kCand) {
         for (int i = tid; i < cl.bm_words; i += kRescanThreads) bm[i] = 0u;
         if (tid < kMaxCand) s_miss[tid] = SWITCHSD_KMAX;
@@ -545,14 +550,14 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
                 c[u] = t[u] = 0;
                 if (i < n_d) {
                     c[u] = __ldcg(a.pv_draft + o * D + i);
-                    t[u] = __ldcg(a.pv_target + o * (D + 1) + i + i / D);
+                    t[u] = __ldcg(a.pv_target + o * (D + 1) + i + over_d(i));
                 }
             }
 #pragma unroll
             for (int u = 0; u < kVerifyLoads; ++u) {
                 const int i = base + u * kRescanThreads;
                 if (i < n_d) {
-                    const int w = i / D;
+                    const int w = over_d(i);
                     vc[i] = c[u];
                     vt[i + w] = t[u];
                     if (c[u] != t[u]) atomicMin(&s_miss[w], i - w * D);
@@ -813,8 +818,8 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
             int32_t *ct = reinterpret_cast<int32_t *>(cstage + 16 + 16 * ((a.W + 3) / 4));
             if (lane == 0) *reinterpret_cast<int4 *>(cstage) = make_int4(nsel, 0, 0, 0);
             if (lane < nsel) ce[lane] = s_sel[lane];
-            const int dw = kWarp / a.D, di = kWarp - dw * a.D;  // (candidate, token) step of 32 slots
-            int w = lane / a.D, i = lane - w * a.D;
+            const int dw = over_d(kWarp), di = kWarp - dw * a.D;  // (candidate, token) step of 32 slots
+            int w = over_d(lane), i = lane - w * a.D;
             for (int t = lane; !kRing && t < nsel * a.D; t += kWarp) {  // (the ring's tiles are gone)
                 const int32_t ew = s_sel[w];
                 const int32_t p = ew + 1 + i;
@@ -951,8 +956,8 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
             return reinterpret_cast<const int32_t *>(cmsgs + size_t(r) * cl.cslot + 16)[src - r * kMaxCand];
         };
         if (lane < nc) a.out_cand_len[size_t(b) * a.W + lane] = min(a.D, L - 1 - cand_end(s_sel[lane]));
-        const int dw = kWarp / a.D, di = kWarp - dw * a.D;  // (candidate, token) step of 32 slots
-        int w = lane / a.D, i = lane - w * a.D;
+        const int dw = over_d(kWarp), di = kWarp - dw * a.D;  // (candidate, token) step of 32 slots
+        int w = over_d(lane), i = lane - w * a.D;
         for (int t = lane; t < nc * a.D; t += kWarp, w += dw, i += di) {
             if (i >= a.D) {
                 i -= a.D;
