@@ -434,15 +434,15 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
 // from the table its own bins' warp wrote (same warp, earlier chunk) and updates only the heads it moved.
 //
 // Why: one warp per item walking its row 32 positions at a time (a dependent head read and write each) took
-// 1210 us for 64 rows of 32K tokens, n = 3..8 (build and one step); this takes 150 us.  Ranks by eight ballots a
+// 1210 us for 64 rows of 32K tokens, n = 3..8 (build and one step); this takes 144 us.  Ranks by eight ballots a
 // position, counted in a pass of their own: 177 us; the groups of equal keys in a round of step 4 by nine ballots
 // (six rounds in ten hold one): 155 us.  The tokens staged in shared memory by one copy made no difference.  The
 // table written sets the floor (201 MB of heads + 50 MB of links: 37 us at the measured copy bandwidth); what
-// bounds it is the issue rate (ALU and shared-memory pipes each at half of their peak) at one 1024-thread CTA an
-// SM, 2.5 waves of them here.
+// bounds it is the shared-memory pipe (random accesses, three to four wavefronts each: 70 % of its peak while a
+// CTA runs) and the issue rate, at one 1024-thread CTA an SM, 2.5 waves of them here.
 // ------------------------------------------------------------------------------------------------
 constexpr int kBuildKeyBits = 9;
-constexpr int kBuildBins = 256;
+constexpr int kBuildBins = 256;  // 1 << 8
 constexpr int kLocalBits = kBuildKeyBits + 8;  // a bucket within its part: bin and key.  A position's rank within
                                                // its segment and bin (below 1024), and in the queue its place in
                                                // the chunk (15 bits), stand above it.
@@ -582,6 +582,9 @@ __global__ void __launch_bounds__(kT, 1024 / kT) index_build_kernel(const BuildA
                 s_bin[1 + lane * (kBuildBins / kWarp) + j] = incl - sum + v[j];
         }
         __syncthreads();
+        for (int i = tid; i < kW * kBuildBins; i += kT)  // a (bin, warp)'s place in the queue
+            cnt[(i >> 8) * (kBuildBins + 1) + (i & (kBuildBins - 1))] += s_bin[i & (kBuildBins - 1)];
+        __syncthreads();
 
         // 3. scatter into the queue, in position order within a bin
 #pragma unroll
@@ -590,7 +593,7 @@ __global__ void __launch_bounds__(kT, 1024 / kT) index_build_kernel(const BuildA
             if (c != 0xffffffffu) {
                 const uint32_t local = c & ((1u << kLocalBits) - 1u), bin = local >> keybits;
                 const uint32_t lp = uint32_t(p_seg - c0 + 32 * i + lane);
-                q[s_bin[bin] + my[bin] + (c >> kLocalBits)] = lp << kLocalBits | local;
+                q[my[bin] + (c >> kLocalBits)] = lp << kLocalBits | local;
             }
         }
         __syncthreads();  // the counters are dead from here on: the links take their place
