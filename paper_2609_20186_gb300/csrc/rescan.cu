@@ -120,6 +120,7 @@ __device__ __forceinline__ uint32_t scan_ends(const int32_t *stage, int32_t e_lo
     const int32_t n4 = (e_end - e_lo + 3) >> 2;
     const int4 *g4 = reinterpret_cast<const int4 *>(stage + kHalo);
     const int32_t off = kHalo - e_lo;
+    constexpr int kWords = kPre ? 2 * kScanWords : kScanWords;  // a round's words a thread: 4-byte or 16-byte loads
     uint32_t passed = 0u;  // bit i: word tid + i * kRescanThreads holds an end that passes
     int rnd = 0;
     int32_t g0 = tid;
@@ -131,30 +132,30 @@ __device__ __forceinline__ uint32_t scan_ends(const int32_t *stage, int32_t e_lo
         if constexpr (kPre) {
             const uint32_t *w = hb + g0;
 #pragma unroll
-            for (int u = 0; u < kScanWords; ++u)
+            for (int u = 0; u < kWords; ++u)
                 if ((kAll || g0 + u * kRescanThreads < n4) && has_zero_byte(w[u * kRescanThreads] ^ hs4) != 0u) hit |= 1u << u;
         } else {
             const int4 *w = g4 + g0;
-            int4 v[kScanWords];
-            int2 pv[kScanWords];  // x[4g - 2], x[4g - 1]
+            int4 v[kWords];
+            int2 pv[kWords];  // x[4g - 2], x[4g - 1]
 #pragma unroll
-            for (int u = 0; u < kScanWords; ++u) {
+            for (int u = 0; u < kWords; ++u) {
                 const bool in = kAll || g0 + u * kRescanThreads < n4;
                 v[u] = in ? w[u * kRescanThreads] : make_int4(0, 0, 0, 0);
                 pv[u] = (F >= 2 && in) ? reinterpret_cast<const int2 *>(w + u * kRescanThreads)[-1] : make_int2(0, 0);
             }
 #pragma unroll
-            for (int u = 0; u < kScanWords; ++u) {
+            for (int u = 0; u < kWords; ++u) {
                 const uint32_t h0 = end_hash<F>(v[u].x, pv[u].y, pv[u].x), h1 = end_hash<F>(v[u].y, v[u].x, pv[u].y);
                 const uint32_t h2 = end_hash<F>(v[u].z, v[u].y, v[u].x), h3 = end_hash<F>(v[u].w, v[u].z, v[u].y);
                 if ((h0 == hs) | (h1 == hs) | (h2 == hs) | (h3 == hs)) hit |= 1u << u;
             }
         }
         passed |= hit << (rnd & 31);
-        g0 += kScanWords * kRescanThreads;
-        rnd += kScanWords;
+        g0 += kWords * kRescanThreads;
+        rnd += kWords;
     };
-    while (g0 - lane + (kScanWords - 1) * kRescanThreads + kWarp <= n4) round(std::true_type{});
+    while (g0 - lane + (kWords - 1) * kRescanThreads + kWarp <= n4) round(std::true_type{});
     while (g0 - lane < n4) round(std::false_type{});
     uint32_t mine = 0u;
     // m(e) from F for an end whose last F tokens match: x[e - q] against suf[-q], eight positions per step,
@@ -907,6 +908,12 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     const uint32_t best_e = kRing ? __reduce_max_sync(kFull, k_r == best ? e_r : 0u) : 0u;
     const unsigned at = __ballot_sync(kFull, k_r == best && (!kRing || e_r == best_e));
     const int32_t win = __shfl_sync(kFull, i_r, at != 0u ? __ffs(at) - 1 : 0);
+    // The winner's continuation is read beside the logit's sum (8K rows 3.54 -> 3.45 us a launch; not in the hash
+    // instance, whose register file is full: 32K rows 4.20 -> 4.22).
+    constexpr bool kDraftEarly = !kCand && !kPre && !kMlp;
+    const int32_t *wd = reinterpret_cast<const int32_t *>(msgs + size_t(win) * slot_bytes + 16);
+    const int32_t w_lo = kDraftEarly && lane < 4 * kw ? wd[lane] : 0;
+    const int32_t w_hi = kDraftEarly && lane + kWarp < 4 * kw ? wd[lane + kWarp] : 0;
     const float z = warp_sum_f32(z_r) + (mlp ? a.b2 : 0.f);
     const bool timeout = best == kKeyTimeout;
     const bool hit = len_ok && !timeout && best != 0u;
@@ -994,7 +1001,6 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
                 a.status[b] = st;
             }
         }
-        (void)win;
     } else {
         const int32_t kappa = a.kappa > 0 ? a.kappa : a.n_min;
         int32_t mode = SWITCHSD_MODE_NO_REP;
@@ -1014,8 +1020,9 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
                 a.status[b] = st;
             }
         }
-        const int32_t *wd = reinterpret_cast<const int32_t *>(msgs + size_t(win) * slot_bytes + 16);
-        for (int i = lane; i < len; i += kWarp) a.out_draft[size_t(b) * a.k + i] = wd[i];
+        int32_t *out = a.out_draft + size_t(b) * a.k;
+        if (lane < len) out[lane] = kDraftEarly ? w_lo : wd[lane];
+        if (lane + kWarp < len) out[lane + kWarp] = kDraftEarly ? w_hi : wd[lane + kWarp];
     }
     if (!all_in && lane == 0) (void)mbar_wait(&bars[3], 0);  // messages still in flight: a second bounded wait
     if (timed_out && lane == 0) {
