@@ -1108,6 +1108,10 @@ static cudaError_t choose_hash(StepArgs &args, int split, int sms) {
     // grid of fewer CTAs than SMs is not, measured: the 8K rows (two CTAs a row, 128 CTAs) lose 0.1 us a
     // launch with it, the 32K rows (512 CTAs) gain 0.1 us and the 128K rows (256 CTAs of 8.5K ends) 0.8 us.
     if (int64_t(split) * args.B < int64_t(sms)) return cudaSuccess;
+    // Without the context prefetch the tiles land after the wait, and the hashing would only stand before the
+    // scan: one batch of 64 rows of 32K tokens takes 6.20 us a launch without it and 7.00 with it, 16 of 128K
+    // 8.55 and 9.69, 768 of 4K with the two-layer probe 18.4 and 19.3.
+    if ((args.prefetch & SWITCHSD_PREFETCH_CONTEXT) == 0) return cudaSuccess;
     int without = 0, with = 0;
     cudaError_t e = rescan_per_sm<kSampled, kCand, kScanTokens, kMlp>(rescan_smem_bytes(args, split), without);
     if (e != cudaSuccess) return e;
