@@ -35,10 +35,17 @@ static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 // benchmark's launch graph (256 launches): the 32K-context rows 8 CTAs 4.36 us per launch (4: 4.54,
 // 16: 6.59), the 8K rows 2 CTAs 3.06 us (1: 3.41, 4: 3.28), the 128K rows 16 CTAs 5.17 us (8: 8.74),
 // the 16K rows with the two-layer probe 2 CTAs 10.15 us per step (1: 15.83, 4: 11.45).
+// A grid of at most one CTA per SM goes further, down to 2048 ends a CTA, and of at most half the SMs down to 256:
+// its copies and scans get shorter and nothing waits for a slot.  A launch, with the limit of 4096 and without:
+// one row of 16K tokens 2.99 and 2.61 us, one of 2K 2.95 and 2.78, 8 of 4K 3.16 and 2.98, sampled on 37 of 9K
+// 4.35 and 4.19, 10 candidates on 8 of 5K 5.64 and 4.96 (but 64 rows of 3K over two CTAs 3.29 and 3.34).
 static int choose_rescan_split(int B, int cap) {
     const int sms = sm_count_cached() > 0 ? sm_count_cached() : 148;
     int c = 1;
-    while (c < kMaxSplit && cap / (2 * c) >= 4096 && 2 * int64_t(B) * (2 * c) <= int64_t(kRescanMinBlocks) * sms)
+    while (c < kMaxSplit &&
+           ((cap / (2 * c) >= 4096 && 2 * int64_t(B) * (2 * c) <= int64_t(kRescanMinBlocks) * sms) ||
+            (cap / (2 * c) >= 2048 && int64_t(B) * (2 * c) <= sms) ||
+            (cap / (2 * c) >= 256 && 2 * int64_t(B) * (2 * c) <= sms)))
         c *= 2;
     return c;
 }
