@@ -4,7 +4,8 @@
 // starting at an earlier position of the row (the paper trains its probe on these labels with
 // n = n_train = 5).
 //
-// Rows up to kLabelClusterCap tokens of capacity: one kernel, a cluster of P CTAs per row.  The windows are
+// Short rows, and longer ones where the batch is large (label_one_kernel): one kernel, a cluster of P CTAs
+// per row.  The windows are
 // split over the CTAs by hash; each CTA hashes every window of the row and inserts its own into an
 // open-addressing table in its shared memory.  A slot holds hash bits above the smallest start so far of one
 // window: an empty slot is claimed with an atomicCAS, a slot whose bits and tokens agree takes an atomicMin,
@@ -19,9 +20,9 @@
 // tokens, n = 5: 55.9 us with the two kernels below and their table in memory (a chain of dependent random L2
 // atomics a window), 36.5 us with each lane following its own probe sequence, 27.5 us with the stacks, 29.1 us
 // with hash sums of 64 bits instead of 32 (kept, so that ids that differ in their high bits alone still spread).
-// The two kernels are still taken past kLabelClusterCap, where P would exceed a portable cluster.
 //
-// Longer rows: two kernels over a per-row table in the caller's workspace.
+// A few long rows: two kernels over a per-row table in the caller's workspace, which spread a row's windows over
+// the whole chip.
 //   insert  thread per window start s: hash the n tokens, probe linearly; an empty slot is claimed with
 //           atomicCAS, a slot whose window holds the same tokens takes atomicMin(slot, s).  Every slot
 //           then holds the smallest start among the windows with its tokens -- the same value whatever
@@ -121,11 +122,12 @@ __global__ void __launch_bounds__(kLabelThreads) label_mark_kernel(const LabelAr
 }
 
 // ------------------------------------------------------------------------------------------------
-// Rows of at most kLabelClusterCap tokens of capacity.
+// One kernel: short rows, and longer ones in large batches (label_one_kernel).
 // ------------------------------------------------------------------------------------------------
 constexpr int kLabelMaxParts = 8;          // CTAs a row: the portable cluster size
 constexpr int kLabelPartWindows = 32768;   // windows a CTA's table is meant for
-constexpr int kLabelClusterCap = kLabelMaxParts * kLabelPartWindows;
+constexpr int kLabelClusterCap = 65536;    // the largest capacity of the one-kernel form
+constexpr int kLabelShortCap = 16384;      // up to here for any number of rows
 constexpr int kLabelClusterThreads = 1024;
 constexpr size_t kLabelSmemMax = 224 * 1024;
 // The stacks' sizes: fewer than 32 windows are left when 32 more come from the hash or a round of tries, and a
@@ -326,12 +328,26 @@ __global__ void __launch_bounds__(kLabelClusterThreads, 1) label_cluster_kernel(
 }
 
 // CTAs a row: enough that a CTA's windows fit its table, and more while the grid leaves SMs idle (every CTA
-// hashes the whole row, so more only pay while they add SMs).
+// hashes the whole row, so more only pay while they add SMs).  SMs that do not fill a cluster in their part of
+// the chip stay idle, the more the larger the cluster: 5 clusters' worth is left for them.
 static int label_parts(int32_t B, int32_t cap, int sms) {
     int P = 1;
     while (int64_t(P) * kLabelPartWindows < cap) P *= 2;
-    while (P < kLabelMaxParts && 2 * int64_t(P) * B <= sms && cap / (2 * P) >= 512) P *= 2;
+    while (P < kLabelMaxParts && 2 * int64_t(P) * (B + 5) <= sms && cap / (2 * P) >= 512) P *= 2;
     return P;
+}
+
+// The one-kernel form costs what its longest row does -- a CTA hashes the whole row, about 11 us per 32K tokens --
+// and the two kernels what the batch does, spread over the chip.  Measured (us a call, host included, two kernels
+// -> one; zipf | few distinct windows), n = 5:
+//   1 x 1K 15.0 -> 10.4 | 16.4 -> 10.4     64 x 8K 33.3 -> 15.9 | 20.6 -> 10.6    1 x 16K 18.4 -> 12.7 | 15.5 -> 10.9
+//   4 x 16K 22.8 -> 15.7 | 15.7 -> 11.2    20 x 20K 22.3 -> 22.3 | 18.3 -> 16.2
+//   1 x 32K 17.2 -> 22.1 | 15.8 -> 17.8    8 x 32K 24.7 -> 24.9 | 15.1 -> 18.7    14 x 32K 32.8 -> 23.1 | 18.5 -> 18.8
+//   8 x 64K 34.6 -> 37.5 | 19.6 -> 33.3    24 x 64K 62.5 -> 41.0 | 39.2 -> 43.7   32 x 64K 72.4 -> 41.4 | 49.3 -> 43.8
+//   64 x 32K 72.8 -> 30.4 | 50.8 -> 32.4
+// Past 64K the one kernel would want 64 rows and more to pay (8 x 128K 44 -> 63, 16 x 128K 71 -> 116).
+static bool label_one_kernel(int32_t B, int32_t cap) {
+    return cap <= kLabelShortCap || (cap <= kLabelClusterCap && int64_t(B) * 2048 >= cap);
 }
 
 static cudaError_t launch_label_cluster(const int32_t *ctx, const int32_t *lens, int32_t B, int32_t cap, int32_t n,
@@ -360,7 +376,9 @@ static cudaError_t launch_label_cluster(const int32_t *ctx, const int32_t *lens,
     a.bm_words = (cap + 31) / 32;
     // twice the windows a CTA expects, as far as the shared memory goes (load 1/2 to 3/4)
     const int windows = (cap + P - 1) / P;
-    const int threads = windows < 2048 ? 128 : (windows < 8192 || cap > kLabelClusterCap / 2 ? 512 : kLabelClusterThreads);
+    // threads by the row, which every CTA hashes: four windows each
+    int threads = 128;
+    while (threads < kLabelClusterThreads && 4 * threads < cap) threads *= 2;
     const size_t fixed = size_t((a.bm_words + 3) & ~3) * 4 + size_t(threads / kWarp) * (kLabelTries + kLabelCompares) * sizeof(uint2) + 16;
     const size_t most = (kLabelSmemMax - fixed) / 4;
     const size_t want = size_t(2) * size_t(windows) + 64;
@@ -393,7 +411,7 @@ extern "C" int switchsd_copy_labels(const int32_t *ctx_tokens, const int32_t *ct
     if (B < 1 || B > 65535 || cap < 1 || cap > (1 << 30) || n < 1 || n > SWITCHSD_NMAX) return SWITCHSD_ERR_SHAPE;
     if (workspace_bytes < switchsd_labels_workspace_bytes(B, cap)) return SWITCHSD_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cap <= kLabelClusterCap)
+    if (label_one_kernel(B, cap))
         return launch_label_cluster(ctx_tokens, ctx_lens, B, cap, n, out_labels, s) == cudaSuccess ? SWITCHSD_OK
                                                                                                    : SWITCHSD_ERR_CUDA;
     const uint32_t T = table_slots(cap);

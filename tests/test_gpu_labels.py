@@ -127,8 +127,11 @@ def _first_occurrence_labels(x: np.ndarray, n: int) -> np.ndarray:
 
 
 # (rows, capacity, n): one and several CTAs a row, tables of every size class, capacities that are no multiple
-# of 16, the largest capacity of the one-kernel form and the first one past it
-@pytest.mark.parametrize("B,cap,n", [(200, 3001, 5), (3, 513, 32), (40, 8209, 2), (2, 32769, 5), (70, 16389, 3),
+# of 16, both sides of the lines between the one-kernel form and the two kernels (16,384 tokens for any number
+# of rows, then a row per 2,048, up to 65,536), and rows past them
+@pytest.mark.parametrize("B,cap,n", [(200, 3001, 5), (3, 513, 32), (40, 8209, 2), (1, 4097, 5), (1, 16384, 5),
+                                     (8, 16385, 5), (9, 16385, 5), (2, 32769, 5), (17, 32769, 5), (70, 16389, 3),
+                                     (31, 65536, 5), (32, 65536, 5), (40, 65521, 8), (33, 65537, 5),
                                      (1, 131075, 5), (2, 262144, 7), (1, 262145, 5)])
 def test_size_classes(B, cap, n):
     rng = np.random.default_rng(cap)
