@@ -128,6 +128,7 @@ constexpr int kLabelMaxParts = 8;          // CTAs a row: the portable cluster s
 constexpr int kLabelPartWindows = 32768;   // windows a CTA's table is meant for
 constexpr int kLabelClusterCap = 65536;    // the largest capacity of the one-kernel form
 constexpr int kLabelShortCap = 16384;      // up to here for any number of rows
+constexpr int kLabelRows = 32;             // up to kLabelClusterCap from this many rows
 constexpr int kLabelClusterThreads = 1024;
 constexpr size_t kLabelSmemMax = 224 * 1024;
 // The stacks' sizes: fewer than 32 windows are left when 32 more come from the hash or a round of tries, and a
@@ -337,17 +338,18 @@ static int label_parts(int32_t B, int32_t cap, int sms) {
     return P;
 }
 
-// The one-kernel form costs what its longest row does -- a CTA hashes the whole row, about 11 us per 32K tokens --
-// and the two kernels what the batch does, spread over the chip.  Measured (us a call, host included, two kernels
-// -> one; zipf | few distinct windows), n = 5:
-//   1 x 1K 15.0 -> 10.4 | 16.4 -> 10.4     64 x 8K 33.3 -> 15.9 | 20.6 -> 10.6    1 x 16K 18.4 -> 12.7 | 15.5 -> 10.9
-//   4 x 16K 22.8 -> 15.7 | 15.7 -> 11.2    20 x 20K 22.3 -> 22.3 | 18.3 -> 16.2
-//   1 x 32K 17.2 -> 22.1 | 15.8 -> 17.8    8 x 32K 24.7 -> 24.9 | 15.1 -> 18.7    14 x 32K 32.8 -> 23.1 | 18.5 -> 18.8
-//   8 x 64K 34.6 -> 37.5 | 19.6 -> 33.3    24 x 64K 62.5 -> 41.0 | 39.2 -> 43.7   32 x 64K 72.4 -> 41.4 | 49.3 -> 43.8
-//   64 x 32K 72.8 -> 30.4 | 50.8 -> 32.4
-// Past 64K the one kernel would want 64 rows and more to pay (8 x 128K 44 -> 63, 16 x 128K 71 -> 116).
+// The one-kernel form costs what its longest row does -- a CTA hashes the whole row -- and the two kernels what
+// the batch does, spread over the chip, least where few windows are distinct.  Measured (us a call, host
+// included, two kernels -> one; zipf | few distinct windows):
+//   n = 5   1 x 1K 15.0 -> 10.4 | 16.4 -> 10.4     64 x 8K 33.3 -> 15.9 | 20.6 -> 10.6    1 x 32K 17.2 -> 22.1 | 15.8 -> 17.8
+//           8 x 64K 34.6 -> 37.5 | 19.6 -> 33.3    64 x 32K 72.8 -> 30.4 | 50.8 -> 32.4
+//   n = 8   4 x 16K 18.7 -> 18.0 | 13.3 -> 12.3    12 x 16K 26.8 -> 17.5 | 13.9 -> 12.6   20 x 20K 24.4 -> 21.5 | 18.7 -> 16.8
+//           16 x 32K 41.1 -> 27.5 | 20.7 -> 24.6   24 x 32K 38.9 -> 29.8 | 26.8 -> 24.8
+//           24 x 48K 43.0 -> 35.5 | 33.8 -> 35.1   32 x 48K 49.6 -> 37.5 | 41.2 -> 35.0   32 x 64K 72.7 -> 46.6 | 51.4 -> 46.1
+// The line is where it wins on both texts.  Past 64K it would want far more rows (8 x 128K 44 -> 63).
 static bool label_one_kernel(int32_t B, int32_t cap) {
-    return cap <= kLabelShortCap || (cap <= kLabelClusterCap && int64_t(B) * 2048 >= cap);
+    if (cap <= kLabelShortCap) return true;
+    return cap <= kLabelClusterCap && (B >= kLabelRows || int64_t(B) * 4096 >= int64_t(cap) * 3);
 }
 
 static cudaError_t launch_label_cluster(const int32_t *ctx, const int32_t *lens, int32_t B, int32_t cap, int32_t n,
