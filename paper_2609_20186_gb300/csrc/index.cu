@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
 // Build.  One item = one (row, n); its buckets are split over P CTAs (part = the bucket's top bits).  A CTA
 // goes over the row in chunks of kChunk positions; per chunk, warp w owns a contiguous segment:
 //   1. hash and rank: every position's bucket, positions of other parts dropped, and its rank within the
-//      segment's positions of its bin (the next 8 bits of the bucket), kept in registers; the lanes of a bin
+//      segment's positions of its bin (the next 6 to 8 bits of the bucket), kept in registers; the lanes of a bin
 //      find each other through a mask per bin in shared memory (an atomicOr, a read), and the segment's counts
 //      per bin run along;
 //   2. scan: offsets of every (bin, warp), so that a bin's entries lie in position order;
@@ -434,18 +434,17 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
 // from the table its own bins' warp wrote (same warp, earlier chunk) and updates only the heads it moved.
 //
 // Why: one warp per item walking its row 32 positions at a time (a dependent head read and write each) took
-// 1210 us for 64 rows of 32K tokens, n = 3..8 (build and one step); this takes 144 us.  Ranks by eight ballots a
-// position, counted in a pass of their own: 177 us; the groups of equal keys in a round of step 4 by nine ballots
-// (six rounds in ten hold one): 155 us.  The tokens staged in shared memory by one copy made no difference.  The
+// 1210 us for 64 rows of 32K tokens, n = 3..8 (build and one step); this takes 120 us, and 144 with 256 bins
+// instead of 128.  With 256: ranks by eight ballots a position, counted in a pass of their own 177 us; the groups
+// of equal keys in a round of step 4 by nine ballots
+// (six rounds in ten hold one) 155 us.  The tokens staged in shared memory by one copy made no difference.  The
 // table written sets the floor (201 MB of heads + 50 MB of links: 37 us at the measured copy bandwidth); what
 // bounds it is the shared-memory pipe (random accesses, three to four wavefronts each: 70 % of its peak while a
 // CTA runs) and the issue rate, at one 1024-thread CTA an SM, 2.5 waves of them here.
 // ------------------------------------------------------------------------------------------------
-constexpr int kBuildKeyBits = 9;
-constexpr int kBuildBins = 256;  // 1 << 8
-constexpr int kLocalBits = kBuildKeyBits + 8;  // a bucket within its part: bin and key.  A position's rank within
-                                               // its segment and bin (below 1024), and in the queue its place in
-                                               // the chunk (15 bits), stand above it.
+// A bucket within its part: bin (at most 8 bits) and key (at most 9).  A position's rank within its segment and bin
+// (below 1024), and in the queue its place in the chunk (15 bits), stand above it.
+constexpr int kLocalBits = 17;
 constexpr uint32_t kNone16 = 0xffffu;  // no earlier entry; kDone16: the link is in global memory already
 constexpr uint32_t kDone16 = 0xfffeu;
 
@@ -455,29 +454,30 @@ struct BuildArgs {
     int32_t B, cap, n_min, nn, log2_buckets, log2_parts;
 };
 
-template <int kT, int kChunk>
+template <int kT, int kChunk, int kBinBits, int kKeyBits>
 struct BuildLayout {
-    static constexpr int kW = kT / kWarp;
+    static constexpr int kW = kT / kWarp, kBins = 1 << kBinBits;
     static constexpr size_t queue = size_t(kChunk) * 4;
-    static constexpr size_t counts = size_t(kW) * (kBuildBins + 1) * 4;
-    static constexpr size_t links = size_t(kChunk) * 2 > counts ? size_t(kChunk) * 2 : counts;  // counts, then links
-    static constexpr size_t heads = size_t(kW) * (2 << kBuildKeyBits);  // step 1's masks, then the bins' heads
-    static_assert(heads == size_t(kW) * kBuildBins * 4, "a mask per bin and warp");
+    static constexpr size_t counts = size_t(kW) * (kBins + 1) * 4;
+    static constexpr size_t links = ((size_t(kChunk) * 2 > counts ? size_t(kChunk) * 2 : counts) + 15) & ~size_t(15);  // then links
+    static constexpr int warp_heads = (2 << kKeyBits) > 4 * kBins ? 2 << kKeyBits : 4 * kBins;
+    static constexpr size_t heads = size_t(kW) * warp_heads;  // per warp step 1's masks, then a bin's heads
     static constexpr size_t bytes = queue + links + heads;
 };
 
-template <int kT, int kChunk>
+template <int kT, int kChunk, int kBinBits, int kKeyBits>
 __global__ void __launch_bounds__(kT, 1024 / kT) index_build_kernel(const BuildArgs a) {
-    using Lay = BuildLayout<kT, kChunk>;
-    constexpr int kW = Lay::kW;
+    using Lay = BuildLayout<kT, kChunk, kBinBits, kKeyBits>;
+    static_assert(kBinBits + kKeyBits <= kLocalBits, "a bucket's bits");
+    constexpr int kW = Lay::kW, kBins = Lay::kBins;
     constexpr int kIts = kChunk / kT;  // positions a thread holds
     static_assert(kIts % 8 == 0 && kChunk <= 32768, "15-bit chunk positions, rounds of eight");
     extern __shared__ __align__(16) unsigned char build_smem[];
     uint32_t *q = reinterpret_cast<uint32_t *>(build_smem);
-    uint32_t *cnt = reinterpret_cast<uint32_t *>(build_smem + Lay::queue);     // [kW][kBuildBins + 1]
+    uint32_t *cnt = reinterpret_cast<uint32_t *>(build_smem + Lay::queue);     // [kW][kBins + 1]
     uint16_t *links = reinterpret_cast<uint16_t *>(build_smem + Lay::queue);   // [kChunk]
     uint16_t *heads16 = reinterpret_cast<uint16_t *>(build_smem + Lay::queue + Lay::links);
-    __shared__ uint32_t s_bin[kBuildBins + 1];
+    __shared__ uint32_t s_bin[kBins + 1];
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int part = int(blockIdx.x) & ((1 << a.log2_parts) - 1);
@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(kT, 1024 / kT) index_build_kernel(const BuildA
     const int w = item / a.B, b = item - w * a.B;
     const int n = a.n_min + w;
     const int lg = a.log2_buckets, lgp = lg - a.log2_parts;  // bucket bits, and those within the part
-    const int binbits = lgp < 8 ? lgp : 8, keybits = lgp - binbits;
+    const int binbits = lgp < kBinBits ? lgp : kBinBits, keybits = lgp - binbits;
     const uint32_t keymask = (1u << keybits) - 1u, localmask = (1u << lgp) - 1u;
     pdl_wait();
     pdl_trigger();
@@ -494,18 +494,18 @@ __global__ void __launch_bounds__(kT, 1024 / kT) index_build_kernel(const BuildA
     const int32_t *row = a.ctx + size_t(b) * size_t(a.cap);
     int32_t L = a.lens[b];
     if (L < 0 || L > a.cap) L = 0;
-    uint16_t *H = heads16 + (warp << kBuildKeyBits);
+    uint16_t *H = heads16 + warp * (Lay::warp_heads / 2);
 
     for (int32_t c0 = 0; c0 == 0 || c0 < L; c0 += kChunk) {
         const int32_t clen = min(kChunk, L - c0);
         const int32_t seg = ((clen + kW - 1) / kW + 31) & ~31;  // a warp's positions: <= kChunk / kW
         const int32_t p_seg = c0 + warp * seg;
-        for (int i = tid; i < kW * (kBuildBins + 1); i += kT) cnt[i] = 0u;
-        for (int i = tid; i < kW * kBuildBins; i += kT) reinterpret_cast<uint32_t *>(heads16)[i] = 0u;
+        for (int i = tid; i < kW * (kBins + 1); i += kT) cnt[i] = 0u;
+        for (int i = tid; i < int(Lay::heads / 4); i += kT) reinterpret_cast<uint32_t *>(heads16)[i] = 0u;
         __syncthreads();
 
         // 1. hash and rank
-        uint32_t *mask = reinterpret_cast<uint32_t *>(H), *my = cnt + warp * (kBuildBins + 1);
+        uint32_t *mask = reinterpret_cast<uint32_t *>(H), *my = cnt + warp * (kBins + 1);
         uint32_t code[kIts];  // rank << kLocalBits | the bucket in the part, all ones for a dropped position
         const int32_t p_end = min(L, p_seg + seg);
 #pragma unroll
@@ -551,24 +551,24 @@ __global__ void __launch_bounds__(kT, 1024 / kT) index_build_kernel(const BuildA
         __syncthreads();
 
         // 2. offsets: within a bin over the warps, then over the bins
-        for (int bin = warp; bin < kBuildBins; bin += kW) {
-            const uint32_t v = lane < kW ? cnt[lane * (kBuildBins + 1) + bin] : 0u;
+        for (int bin = warp; bin < kBins; bin += kW) {
+            const uint32_t v = lane < kW ? cnt[lane * (kBins + 1) + bin] : 0u;
             uint32_t incl = v;
 #pragma unroll
             for (int o = 1; o < kWarp; o <<= 1) {
                 const uint32_t t = __shfl_up_sync(kFull, incl, o);
                 if (lane >= o) incl += t;
             }
-            if (lane < kW) cnt[lane * (kBuildBins + 1) + bin] = incl - v;
+            if (lane < kW) cnt[lane * (kBins + 1) + bin] = incl - v;
             if (lane == kWarp - 1) s_bin[bin + 1] = incl;
         }
         if (tid == 0) s_bin[0] = 0u;
         __syncthreads();
         if (warp == 0) {
-            uint32_t v[kBuildBins / kWarp], sum = 0u;
+            uint32_t v[kBins / kWarp], sum = 0u;
 #pragma unroll
-            for (int j = 0; j < kBuildBins / kWarp; ++j) {
-                sum += s_bin[1 + lane * (kBuildBins / kWarp) + j];
+            for (int j = 0; j < kBins / kWarp; ++j) {
+                sum += s_bin[1 + lane * (kBins / kWarp) + j];
                 v[j] = sum;
             }
             uint32_t incl = sum;
@@ -578,12 +578,12 @@ __global__ void __launch_bounds__(kT, 1024 / kT) index_build_kernel(const BuildA
                 if (lane >= o) incl += t;
             }
 #pragma unroll
-            for (int j = 0; j < kBuildBins / kWarp; ++j)
-                s_bin[1 + lane * (kBuildBins / kWarp) + j] = incl - sum + v[j];
+            for (int j = 0; j < kBins / kWarp; ++j)
+                s_bin[1 + lane * (kBins / kWarp) + j] = incl - sum + v[j];
         }
         __syncthreads();
-        for (int i = tid; i < kW * kBuildBins; i += kT)  // a (bin, warp)'s place in the queue
-            cnt[(i >> 8) * (kBuildBins + 1) + (i & (kBuildBins - 1))] += s_bin[i & (kBuildBins - 1)];
+        for (int i = tid; i < kW * kBins; i += kT)  // a (bin, warp)'s place in the queue
+            cnt[(i >> kBinBits) * (kBins + 1) + (i & (kBins - 1))] += s_bin[i & (kBins - 1)];
         __syncthreads();
 
         // 3. scatter into the queue, in position order within a bin
@@ -601,7 +601,7 @@ __global__ void __launch_bounds__(kT, 1024 / kT) index_build_kernel(const BuildA
         // 4. link each bin's entries in order
         const int nbins = 1 << binbits, kb = 1 << keybits;
         for (int bin = warp; bin < nbins; bin += kW) {
-            for (int i = lane; i < (kb + 7) / 8; i += kWarp)  // H holds 1 << kBuildKeyBits entries
+            for (int i = lane; i < (kb + 7) / 8; i += kWarp)  // H holds 1 << kKeyBits entries
                 reinterpret_cast<uint4 *>(H)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
             __syncwarp();
             int32_t *hb = heads + (size_t(bin) << keybits);
@@ -690,32 +690,40 @@ __global__ void __launch_bounds__(kT, 1024 / kT) index_build_kernel(const BuildA
 // ------------------------------------------------------------------------------------------------
 // Host side.
 // ------------------------------------------------------------------------------------------------
-// The build's parts per item: enough that a part's buckets fit kBuildBins bins of 1 << kBuildKeyBits heads,
+// The build's parts per item: enough that a part's buckets fit 1 << kBinBits bins of 1 << kKeyBits heads,
 // and more (up to 8) while the grid leaves SMs idle -- every part hashes the whole row, so more parts only
-// pay while they add CTAs.  Rows up to kBuildSmallChunk tokens of capacity take half-sized CTAs, two an SM.
-constexpr int kBuildSmallChunk = 16384;
-
-template <int kT, int kChunk>
+// pay while they add CTAs.
+//
+// The instance by the row's capacity: the smallest chunk that takes it whole, with as many CTAs an SM as make 1024
+// threads (four, two, one), and the fewest bins whose heads fit (a bin costs its round trips whatever it holds).
+// Build and one step, n = 3..8 unless given, us (the warp-per-item walk; 512 threads, 16384, 8 bin bits up to 16K
+// rows and 1024, 32768, 8 above; now):
+//   44 rows of 1.4K, n = 2..9   57.8, 65.6, 23.2      64 of 4K, n = 2..12   158.6, about 95, 48.6
+//   64 rows of 8K, n = 2..12    305.6, 160.4, 91.0    64 of 16K             567.8, 124.5, 77.5    64 of 32K  1203, 144, 120
+// (With 8 bin bits two CTAs of 512 threads do not fit an SM.)  Where the repeats fall on few buckets, more bins would
+// be a little quicker: 64 rows of 32K tokens of code 219 with 8 bits, 232 with 7.  Past 2^16 buckets 7 bits would
+// need twice the parts: 16 rows of 128K, n = 2..5, 188 with 8, 219 with 7.  Chunks of 16384 for 32K rows: 179.
+template <int kT, int kChunk, int kBinBits, int kKeyBits>
 static cudaError_t launch_index_build(BuildArgs a, cudaStream_t stream) {
+    constexpr auto kernel = index_build_kernel<kT, kChunk, kBinBits, kKeyBits>;
+    constexpr size_t smem = BuildLayout<kT, kChunk, kBinBits, kKeyBits>::bytes;
     static int sms[64] = {0};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     int n_sm = dev >= 0 && dev < 64 ? sms[dev] : 0;
     if (n_sm == 0) {
-        e = cudaFuncSetAttribute(index_build_kernel<kT, kChunk>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 int(BuildLayout<kT, kChunk>::bytes));
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
         if (e != cudaSuccess) return e;
         e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) sms[dev] = n_sm;
     }
     const int64_t items = int64_t(a.nn) * a.B;
-    int lp = a.log2_buckets > 8 + kBuildKeyBits ? a.log2_buckets - 8 - kBuildKeyBits : 0;
+    int lp = a.log2_buckets > kBinBits + kKeyBits ? a.log2_buckets - kBinBits - kKeyBits : 0;
     while (lp < 3 && (items << (lp + 1)) <= n_sm && a.log2_buckets - lp > 8) ++lp;
     a.log2_parts = lp;
-    return launch_pdl(index_build_kernel<kT, kChunk>, dim3(unsigned(items << lp)), dim3(kT),
-                      BuildLayout<kT, kChunk>::bytes, stream, 0u, a);
+    return launch_pdl(kernel, dim3(unsigned(items << lp)), dim3(kT), smem, stream, 0u, a);
 }
 
 int index_n_min(const switchsd_index *idx) { return idx->n_min; }
@@ -833,9 +841,13 @@ extern "C" int switchsd_index_build(switchsd_index *idx, const int32_t *ctx_toke
     a.n_min = idx->n_min;
     a.nn = idx->nn;
     a.log2_buckets = idx->log2_buckets;
-    const cudaError_t e = idx->cap <= kBuildSmallChunk
-                              ? launch_index_build<512, kBuildSmallChunk>(a, static_cast<cudaStream_t>(stream))
-                              : launch_index_build<1024, 2 * kBuildSmallChunk>(a, static_cast<cudaStream_t>(stream));
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const cudaError_t e =
+        idx->cap <= 4096           ? launch_index_build<256, 4096, 6, 7>(a, st)
+        : idx->cap <= 8192         ? launch_index_build<256, 8192, 7, 8>(a, st)
+        : idx->cap <= 16384        ? launch_index_build<512, 16384, 7, 8>(a, st)
+        : idx->log2_buckets <= 16  ? launch_index_build<1024, 32768, 7, 9>(a, st)
+                                   : launch_index_build<1024, 32768, 8, 9>(a, st);
     return e == cudaSuccess ? SWITCHSD_OK : SWITCHSD_ERR_CUDA;
 }
 

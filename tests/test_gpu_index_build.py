@@ -1,6 +1,6 @@
 """switchsd_index_build against the oracle at the sizes where its chunked radix pass can go wrong.
 
-The build takes a row in chunks (16,384 positions of capacity up to that size, else 32,768), splits the
+The build takes a row in chunks (4,096, 8,192 or 16,384 positions for capacities up to those, else 32,768), splits the
 buckets over several CTAs (few rows, or more than 2^17 buckets), and drops the positions below n - 1.  The
 rows here end just below, at and above those sizes, and hold a period-1 and a period-7 run (one bucket takes
 everything), a small alphabet (dense repeats) and uniform ids.  Every chain is read back through the
@@ -17,7 +17,8 @@ import oracle
 pytestmark = pytest.mark.gpu
 
 # (length, rows, n_min, n_max)
-SHAPES = [(1, 2, 1, 3), (7, 3, 3, 8), (33, 5, 2, 12), (1000, 40, 3, 8), (16383, 4, 3, 8), (16385, 4, 3, 8),
+SHAPES = [(1, 2, 1, 3), (7, 3, 3, 8), (33, 5, 2, 12), (1000, 40, 3, 8), (4096, 5, 2, 5),
+          (4097, 4, 3, 5), (8192, 4, 3, 5), (8193, 5, 2, 4), (16383, 4, 3, 8), (16385, 4, 3, 8),
           (32768, 4, 2, 4), (32769, 5, 1, 2), (70001, 4, 3, 5), (140003, 4, 2, 3)]
 
 
