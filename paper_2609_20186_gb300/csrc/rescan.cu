@@ -25,10 +25,10 @@
 //  * every warp ships its best key, its share of the probe's dot product and its best match's
 //    continuation (from the staged tile, or from its window past the old length) to the row's leader CTA
 //    (the last one) with asynchronous DSMEM stores completing on the leader's mbarrier, and is done.
-// The leader's warp 0 publishes the append, waits (bounded) for the C x kRescanWarps messages, reduces
-// them in a fixed order and writes the outputs.  The only cluster barrier is arrived on right after the
-// length read and waited on beside the verification's loads, so the leader's message barrier is
-// initialised before anyone ships to it and no CTA reads the length after the leader rewrites it.
+// The leader's warp 0 writes the appended tokens, waits (bounded) for the C x kRescanWarps messages, reduces
+// them in a fixed order and writes the outputs and the new length.  The only cluster barrier is arrived on
+// right after the length read and waited on beside the verification's loads, so the leader's message barrier
+// is initialised before anyone ships to it; the messages order every read of the length before its rewrite.
 #include <mutex>
 #include <type_traits>
 
@@ -407,9 +407,9 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     if (!pf_ctx) load_draft();
     // Every thread reads the length itself (one L2 request per warp), then arrives on the cluster
     // barrier.  The arrive is relaxed: the barrier only has to publish the leader's message barrier (its
-    // initialisation fence is a release), and each warp's read of the length is ordered before the leader
-    // rewrites it by the data itself -- the warp's message is computed from the length, and the leader
-    // rewrites it only after every message has landed.
+    // initialisation fence is a release).  It does not order this read against the leader's store of the new
+    // length (a relaxed arrive need not wait for a load in flight); the data does: a warp's message is computed
+    // from the length it read, and the leader stores the new one after its wait for all the messages.
     const int32_t L_old = __ldcg(a.lens + b);
     cluster_arrive_relaxed();
     const bool len_ok = L_old >= 1 && L_old <= (bounded ? a.len_bound : a.cap);
@@ -489,8 +489,8 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     if (pf_ctx && !late) pdl_wait();
     if (pf_ctx) load_draft();
     pdl_trigger();
-    // Every CTA has read the length and the leader's message barrier is initialised once this returns; the arrive
-    // was long before, so it costs little beside the loads in flight (on the way out it cost the row's chain).
+    // The leader's message barrier is initialised once this returns; the arrive was long before, so it costs little
+    // beside the loads in flight (on the way out it cost the row's chain).
     cluster_wait_acquire();
     if (!pf_probe && !gather && !mlp && tid == 0) issue_probe();
 
@@ -881,14 +881,13 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     }
 
     // ---- leader, warp 0: the append, then the row's answer ----
-    if (verifying) {
+    // (the appended positions are past every end the other CTAs scan; what their copies hold there is not used)
+    if (verifying)
         for (int32_t i = lane; i <= acc; i += kWarp) row[L_old + i] = y[kHalo + i];
-        if (lane == 0 && len_ok) {
-            a.lens[b] = L;
-            a.out_accept[b] = acc;
-        }
-    }
     const bool all_in = __all_sync(kFull, mbar_wait_polls(&bars[3], 0, a.msg_wait_polls));
+    // messages still in flight get a second bounded wait: before the new length goes out, and before the CTA's
+    // memory goes away
+    if (!all_in && lane == 0) (void)mbar_wait(&bars[3], 0);
     uint32_t k_r = 0u, e_r = 0u;
     int32_t i_r = 0;
     float z_r = 0.f;
@@ -993,7 +992,10 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
             a.out_ncand[b] = nc;
             if (a.out_match_n) a.out_match_n[b] = n;
             if (a.out_match_end) a.out_match_end[b] = e;
-            if (verifying && !len_ok) a.out_accept[b] = -1;
+            if (verifying) {
+                a.out_accept[b] = acc;          // -1: nothing appended
+                if (len_ok) a.lens[b] = L;      // every warp of the row has read the old one: its message is in
+            }
             if (verifying && a.out_choice) a.out_choice[b] = len_ok ? choice : 0;
             if (a.status) {
                 int32_t st = vst;
@@ -1013,7 +1015,10 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
             a.out_score[b] = z;
             if (a.out_match_n) a.out_match_n[b] = n;
             if (a.out_match_end) a.out_match_end[b] = e;
-            if (verifying && !len_ok) a.out_accept[b] = -1;
+            if (verifying) {
+                a.out_accept[b] = acc;          // -1: nothing appended
+                if (len_ok) a.lens[b] = L;      // every warp of the row has read the old one: its message is in
+            }
             if (a.status) {
                 int32_t st = vst;
                 if (st == SWITCHSD_ROW_OK && timeout) st = SWITCHSD_ROW_TIMEOUT;
@@ -1024,7 +1029,6 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
         if (lane < len) out[lane] = kDraftEarly ? w_lo : wd[lane];
         if (lane + kWarp < len) out[lane + kWarp] = kDraftEarly ? w_hi : wd[lane + kWarp];
     }
-    if (!all_in && lane == 0) (void)mbar_wait(&bars[3], 0);  // messages still in flight: a second bounded wait
     if (timed_out && lane == 0) {
         if (!kRing) (void)mbar_wait(&bars[0], 0);
         (void)mbar_wait(&bars[1], 0);

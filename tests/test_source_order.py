@@ -1,0 +1,35 @@
+"""Orders that the kernels' sources have to keep and that no run shows reliably: a load that happens to be slow
+reads what a store ahead of it in program order has already replaced, once in very many launches.
+
+The row's length is read by every warp of the row's CTAs and replaced by the verification in the same launch.  The
+store has to stand after the point that every reader has passed.
+"""
+import os
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_20186_gb300", "csrc")
+
+
+def _source(name: str) -> str:
+    with open(os.path.join(CSRC, name)) as f:
+        return f.read()
+
+
+def _positions(text: str, what: str):
+    at, out = text.find(what), []
+    while at >= 0:
+        out.append(at)
+        at = text.find(what, at + 1)
+    return out
+
+
+# the kernel's source, the point every reader of the length has passed
+@pytest.mark.parametrize("name,passed", [("rescan.cu", "mbar_wait_polls(&bars[3], 0, a.msg_wait_polls)")],
+                         ids=["rescan"])
+def test_length_is_stored_after_every_read(name, passed):
+    text = _source(name)
+    reads, stores = _positions(text, "__ldcg(a.lens + b)"), _positions(text, "a.lens[b] = ")
+    wait = _positions(text, passed)
+    assert len(reads) == 1 and len(wait) == 1 and stores
+    assert reads[0] < wait[0] < min(stores)
