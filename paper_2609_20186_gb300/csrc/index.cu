@@ -251,18 +251,14 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
             s_ver[0] = acc;
             s_ver[1] = L;
             s_ver[2] = vst;
-            if (verifying && len_ok) {
-                a.lens[b] = L;
-                a.out_accept[b] = acc;
-            } else if (verifying) {
-                a.out_accept[b] = -1;
-            }
+            if (verifying) a.out_accept[b] = acc;  // -1: nothing appended
             if (verifying && a.W > 0 && a.out_choice) a.out_choice[b] = choice;
             if (!a.stepping && a.status) a.status[b] = vst;
         }
     }
     __syncthreads();
     const int32_t L = s_ver[1];
+    if (tid == 0 && verifying && len_ok) a.lens[b] = L;  // every warp has read the old length: behind the barrier
     const int n = a.n_min + warp;  // this warp's gram length
     const bool has_n = warp < a.n_max - a.n_min + 1;
     const size_t nb = size_t(1) << a.log2_buckets;

@@ -25,8 +25,9 @@ def _positions(text: str, what: str):
 
 
 # the kernel's source, the point every reader of the length has passed
-@pytest.mark.parametrize("name,passed", [("rescan.cu", "mbar_wait_polls(&bars[3], 0, a.msg_wait_polls)")],
-                         ids=["rescan"])
+@pytest.mark.parametrize("name,passed", [("rescan.cu", "mbar_wait_polls(&bars[3], 0, a.msg_wait_polls)"),
+                                         ("index.cu", "__syncthreads();\n    const int32_t L = s_ver[1];")],
+                         ids=["rescan", "index"])
 def test_length_is_stored_after_every_read(name, passed):
     text = _source(name)
     reads, stores = _positions(text, "__ldcg(a.lens + b)"), _positions(text, "a.lens[b] = ")
