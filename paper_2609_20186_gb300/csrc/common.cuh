@@ -160,7 +160,9 @@ __device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
 // serialization: it waits for the preceding kernel (griddepcontrol.wait) before its first read of
 // data that kernel may have written, and lets the next kernel start launching right after
 // (griddepcontrol.launch_dependents), so launch latency overlaps execution.  Both are no-ops when the
-// launch carries no programmatic dependency.
+// launch carries no programmatic dependency.  A grid may so be resident while the kernel before it writes the
+// grid's inputs: they are read with plain loads, bulk copies or through L2, never through the non-coherent path
+// (__ldg), which asks for data that nothing writes while the grid runs.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 

@@ -99,7 +99,7 @@ __device__ __forceinline__ float index_probe_partial(const IndexArgs &a, int b, 
     const uint4 *w4 = reinterpret_cast<const uint4 *>(a.probe_w);
     float zp = 0.f;
     for (int v = threadIdx.x; v < (a.d >> 3); v += blockDim.x) {
-        const uint4 w = __ldg(w4 + v), h = __ldg(h4 + v);
+        const uint4 w = w4[v], h = h4[v];
         zp = fmaf(bf16_lo(w.x), bf16_lo(h.x), zp);
         zp = fmaf(bf16_hi(w.x), bf16_hi(h.x), zp);
         zp = fmaf(bf16_lo(w.y), bf16_lo(h.y), zp);
@@ -516,12 +516,12 @@ __global__ void __launch_bounds__(kT, 1024 / kT) index_build_kernel(const BuildA
                     const int32_t *x = row + p0 + lane;
                     for (int i = 0; i < n; ++i, --x, pw *= kGramMul)
 #pragma unroll
-                        for (int u = 0; u < 8; ++u) h[u] += uint64_t(uint32_t(__ldg(x + 32 * u))) * pw;
+                        for (int u = 0; u < 8; ++u) h[u] += uint64_t(uint32_t(x[32 * u])) * pw;
                 } else {
                     for (int i = 0; i < n; ++i, pw *= kGramMul)
 #pragma unroll
                         for (int u = 0; u < 8; ++u)
-                            h[u] += uint64_t(uint32_t(__ldg(row + min(max(p0 + lane + 32 * u - i, 0), L - 1)))) * pw;
+                            h[u] += uint64_t(uint32_t(row[min(max(p0 + lane + 32 * u - i, 0), L - 1)])) * pw;
                 }
             }
 #pragma unroll

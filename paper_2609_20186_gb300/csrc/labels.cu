@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kLabelClusterThreads, 1) label_cluster_kernel(
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int i = min(i0 + u, n - 1);
-                eq &= __ldg(x + p + i) == __ldg(x + s + i);
+                eq &= x[p + i] == x[s + i];
             }
             if (!eq) return false;
         }
@@ -269,11 +269,11 @@ __global__ void __launch_bounds__(kLabelClusterThreads, 1) label_cluster_kernel(
             const int32_t *at = x + s0 + lane;
             for (int i = 0; i < n; ++i, ++at, pw *= kLabelMul)
 #pragma unroll
-                for (int u = 0; u < kW4; ++u) h[u] += uint64_t(uint32_t(__ldg(at + kWarp * u))) * pw;
+                for (int u = 0; u < kW4; ++u) h[u] += uint64_t(uint32_t(at[kWarp * u])) * pw;
         } else {
             for (int i = 0; i < n; ++i, pw *= kLabelMul)
 #pragma unroll
-                for (int u = 0; u < kW4; ++u) h[u] += uint64_t(uint32_t(__ldg(x + min(s0 + kWarp * u + lane + i, L - 1)))) * pw;
+                for (int u = 0; u < kW4; ++u) h[u] += uint64_t(uint32_t(x[min(s0 + kWarp * u + lane + i, L - 1)])) * pw;
         }
 #pragma unroll
         for (int u = 0; u < kW4; ++u) {

@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
                 for (int i = tid - kWarp; i < v_staged; i += kRescanThreads - kWarp) zp = dot8_bf16(s_pw[i], s_ph[i], zp);
         }
         for (int v = v0 + v_staged + tid - kWarp; v < v1; v += kRescanThreads - kWarp)
-            zp = dot8_bf16(__ldg(w4 + v), __ldg(h + v), zp);
+            zp = dot8_bf16(w4[v], h[v], zp);
     };
     // A prefetched probe is finished before the wait by warps 1.. (its inputs are not written by the
     // preceding kernel); warp 0 goes straight to the wait and releases the next launch.

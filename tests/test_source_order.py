@@ -1,8 +1,12 @@
 """Orders that the kernels' sources have to keep and that no run shows reliably: a load that happens to be slow
-reads what a store ahead of it in program order has already replaced, once in very many launches.
+reads what a store ahead of it in program order has already replaced, or a cache line keeps what it held, once in
+very many launches.
 
 The row's length is read by every warp of the row's CTAs and replaced by the verification in the same launch.  The
 store has to stand after the point that every reader has passed.
+
+A grid may be resident while the kernel before it still writes the grid's inputs (programmatic launches), so none
+of them is read through the non-coherent path, which asks for data that nothing writes while the grid runs.
 """
 import os
 
@@ -34,3 +38,10 @@ def test_length_is_stored_after_every_read(name, passed):
     wait = _positions(text, passed)
     assert len(reads) == 1 and len(wait) == 1 and stores
     assert reads[0] < wait[0] < min(stores)
+
+
+def test_no_load_through_the_non_coherent_path():
+    for name in sorted(os.listdir(CSRC)):
+        text = _source(name)
+        for what in ("__ldg(", "ld.global.nc"):
+            assert what not in text, (name, what)
