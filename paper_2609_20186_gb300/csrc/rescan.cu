@@ -464,11 +464,11 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
             zp = dot8_bf16(w4[v], h[v], zp);
     };
     // A prefetched probe is finished before the wait by warps 1.. (its inputs are not written by the
-    // preceding kernel); warp 0 goes straight to the wait and releases the next launch.
-    if (pf_probe) {
-        if (warp >= 1) probe_dot(h4);
-        zp = warp_sum_f32(zp);
-    }
+    // preceding kernel); warp 0 goes straight to the wait and releases the next launch.  The sum over the warp
+    // stands at the message: taken here it made every warp wait for the products before its verification (a
+    // launch without verification, 17 rows of 98 tokens 2.71 us here, 2.46 there; 66 of 572, context not
+    // prefetched, 3.86 and 3.60; 16 launches on the 32K rows 69.3 and 66.9 us).
+    if (pf_probe && warp >= 1) probe_dot(h4);
     // Warps 1.. hash this CTA's old ends once the tile has landed -- before the wait when the context is
     // prefetched -- so that the scan after it compares one byte per end (scan_ends, kPre).
     constexpr bool pre = kPre;
@@ -848,7 +848,7 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
         }
     }
     if (!probe_ok) key = kKeyTimeout;
-    const float z_w = pf_probe ? zp : warp_sum_f32(zp);
+    const float z_w = warp_sum_f32(zp);
 
     // ---- the continuation of this warp's best match (the ring has it already) ----
     if (!kRing && key != 0u && key != kKeyTimeout) gather_next(int32_t(key & kKeyEndMask), stage, off);
