@@ -832,7 +832,8 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
                     ++w;
                 }
             }
-            __syncwarp();  // the message is shipped below, a word a lane
+            fence_proxy_async();  // the bulk copy below reads the message through the async proxy
+            __syncwarp();
         }
     }
 
@@ -866,12 +867,13 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
     } else if (lane <= kw) {
         st_async_v4(map_to_rank(slot + 16 * lane, lead), cw, done_addr);
     }
-    if (kCand && warp == 0) {  // this CTA's candidates
-        const uint32_t to = map_to_rank(cmsgs + size_t(rank) * cl.cslot, lead);
-        for (uint32_t i = lane; i < cl.cslot / 16; i += kWarp)
-            st_async_v4(to + 16 * i, reinterpret_cast<const uint4 *>(cstage)[i], done_addr);
-    }
+    // This CTA's candidates, in one bulk copy (a launch without verification; a store a word a lane instead, and so: 4
+    // candidates of 8 tokens on 287 rows of 223 tokens 3.99 and 3.60 us, 14 of 20 on 146 of 177 4.77 and 4.50; 10 of
+    // 20 on the 32K rows, 8 fused launches, 50.5 and 49.3 us).
+    const bool ships_cand = kCand && warp == 0 && lane == 0;
+    if (ships_cand) bulk_s2c(map_to_rank(cmsgs + size_t(rank) * cl.cslot, lead), cstage, cl.cslot, done_addr);
     if (rank != lead || warp != 0) {
+        if (ships_cand) bulk_wait_read();  // the message has been read out
         if (timed_out && lane == 0) {  // copies still in flight get a second bounded wait
             if (!kRing) (void)mbar_wait(&bars[0], 0);
             (void)mbar_wait(&bars[1], 0);
@@ -1029,6 +1031,7 @@ __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaun
         if (lane < len) out[lane] = kDraftEarly ? w_lo : wd[lane];
         if (lane + kWarp < len) out[lane + kWarp] = kDraftEarly ? w_hi : wd[lane + kWarp];
     }
+    if (ships_cand) bulk_wait_read();  // the leader's own message has been read out
     if (timed_out && lane == 0) {
         if (!kRing) (void)mbar_wait(&bars[0], 0);
         (void)mbar_wait(&bars[1], 0);
