@@ -11,8 +11,8 @@
 // The step kernel that follows adds the S partials of its row in order, then b1, ReLU, w2 and b2: every
 // sum has a fixed order, so the result is deterministic.  No cluster and no cross-CTA exchange here.
 //
-// S is P, or P / 2 for the larger batches (mlp_ctas_per_tile), so that the partial sums that go through memory --
-// S B H1 floats written, then read by the row's step CTAs, which bound those batches -- stay small.  The parts,
+// S is P, or P / 2 where the partial sums that go through memory -- S B H1 floats written, then read by the row's step
+// CTAs -- bound the batch (mlp_ctas_per_tile).  The parts,
 // and with them the length of every sum in an accumulator, do not depend on S.
 #include <cudaTypedefs.h>
 
@@ -40,7 +40,7 @@ struct MlpArgs {
     float *part;   // [S][B][H1p]
     int32_t B, H1p, nchunks, prefetch;
     int32_t parts;   // P
-    int32_t columns; // TMEM columns: 64 a part of the CTA, a power of two
+    int32_t columns; // TMEM columns: N a part of the CTA, a power of two
     int32_t stages;  // operand stages: chunk c goes to stage c % stages, refilled once its MMAs are done
 };
 
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_tc_kernel(const __grid_consta
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     ok = __syncthreads_and(ok && mma_done);
 
-    // Row tid of the tile: its 64 accumulators, the parts added in order (zero when this CTA had no K chunk;
+    // Row tid of the tile: its N accumulators, the parts added in order (zero when this CTA had no K chunk;
     // NaN when a copy or the MMAs did not complete in time, so the row's logit shows the failure).  The tile
     // goes out through shared memory (the operand stages are free: every MMA has completed), so that each warp
     // store writes whole rows instead of one 16-byte piece of 32 rows.  Row r keeps its 16-byte
@@ -274,34 +274,48 @@ int mlp_split(int d) {
     return s;
 }
 
-static size_t mlp_most_partials(int B, int d, int H1) {  // bytes, with every part its own CTA
-    return size_t(mlp_split(d)) * size_t(B) * size_t(mlp_hidden_padded(H1)) * sizeof(float);
-}
+// With every part its own CTA, P x B x H1p floats of partial sums go through memory.  Past 10 MB of them the rows'
+// and units' tiles are 128 x 128 where H1p divides into them -- the operands' L2 traffic falls by a third -- and two
+// parts go to a CTA where that still leaves enough CTAs.  A step (probe and rescan kernel, rows of 2K tokens, context
+// prefetched), one part a CTA and two, us:
+//   d = 4096: 256 rows x 256 units (4 MB) 8.0 and 9.5      512 x 256 (8 MB) 9.4 and 10.4      512 x 512 (17 MB) 14.6 and 11.9
+//   d = 5120: 768 x 256 (13 MB) 12.2 and 14.3              512 x 512 14.8 and 13.0            768 x 512 (25 MB) 21.2 and 16.1
+//   d = 8192: 330 x 512 (11 MB) 13.2 and 16.1              768 x 256 14.0 and 18.0            768 x 768 (38 MB) 34.2 and 26.0
+// A CTA goes over the chunks of its parts one after another: two parts of eight chunks on 96 CTAs leave SMs idle for
+// longer than the smaller sums save, two parts of four chunks on 128 CTAs do not.  The line, seven CTAs per SM and
+// chunk of a part, has the measured sizes on their sides (945 of them: 14 batches, 7 H1, 5 d, rows of 2K and 8K).
+constexpr size_t kMlpManyPartials = 10u * 1000u * 1000u;
 
-int mlp_ctas_per_tile(int B, int d, int H1) {
-    const int parts = mlp_split(d);
-    // With every part its own CTA, parts x B x H1p floats go through memory.  Past 10 MB two parts a CTA are
-    // faster, below it the shorter CTAs.  A step (probe and rescan kernel), one part a CTA and two: 256 rows x
-    // 256 units (4 MB) 10.3 and 13.6 us, 512 x 256 (8 MB) 11.8 and 14.2, 130 x 1024 (8.5 MB) 13.2 and 14.4,
-    // 768 x 256 (12.6 MB) 18.6 and 17.2, 400 x 512 (13 MB) 20.7 and 15.3, 768 x 512 (25 MB) 25.1 and 21.0 (four
-    // parts a CTA: 23.3).
-    return parts > 1 && mlp_most_partials(B, d, H1) > 10u * 1000u * 1000u ? parts / 2 : parts;
-}
-
-// Tiles of 128 units where H1p divides into them and the partial sums call for two parts a CTA: the operands' L2
-// traffic, which bounds those grids, falls by a third (a step of 768
-// rows x 512 units 21.1 us with tiles of 64, 19.0 of 128; 400 x 512 15.4 and 14.9; 768 x 256 16.9 and 16.6).
 static bool mlp_wide(int B, int d, int H1) {
-    return mlp_hidden_padded(H1) % (2 * kMlpNMin) == 0 && mlp_ctas_per_tile(B, d, H1) < mlp_split(d);
+    const size_t partials = size_t(mlp_split(d)) * size_t(B) * size_t(mlp_hidden_padded(H1)) * sizeof(float);
+    return partials > kMlpManyPartials && mlp_hidden_padded(H1) % (2 * kMlpNMin) == 0;
 }
 
-// A grid of at most half the SMs stages all its chunks at once, one of at most a CTA an SM three, a larger one
-// two: a step of 64 rows x 256 units (64 CTAs) takes 8.4 us with two, 7.3 with all five; 256 x 256 (128 CTAs)
-// 10.3 with two, 9.9 with three, 11.6 with five; 512 x 256 (256 CTAs) 11.9 with two, 13.6 with three.
-int mlp_stages_beside(int B, int d, int H1, int S, int sms) {
+static int64_t mlp_tiles(int B, int d, int H1) {  // of 128 rows x N units
     const int N = mlp_wide(B, d, H1) ? 2 * kMlpNMin : kMlpNMin;
-    const int64_t ctas = int64_t((B + kMlpM - 1) / kMlpM) * ((H1 + N - 1) / N) * S;
-    return 2 * ctas <= sms ? 0 : (ctas <= sms ? 3 : 2);
+    return int64_t((B + kMlpM - 1) / kMlpM) * (mlp_hidden_padded(H1) / N);
+}
+
+int mlp_ctas_per_tile(int B, int d, int H1, int sms) {
+    const int parts = mlp_split(d);
+    const int nchunks = (d + kMlpKc - 1) / kMlpKc, per = (nchunks + parts - 1) / parts;
+    const size_t partials = size_t(parts) * size_t(B) * size_t(mlp_hidden_padded(H1)) * sizeof(float);
+    if (parts == 1 || partials <= kMlpManyPartials) return parts;
+    return 7 * mlp_tiles(B, d, H1) * (parts / 2) >= int64_t(sms) * per ? parts / 2 : parts;
+}
+
+// A grid of at most half the SMs stages all its chunks at once, as does one of at most a CTA an SM beside a few rows;
+// one of at most a CTA an SM three chunks, unless a CTA of one part then leaves no room for the rescan kernel's CTAs
+// (`beside` bytes an SM); a larger one two.  A step of 64 rows x 256 units (64 CTAs) takes 8.4 us with two, 7.3 with all
+// five; 4 x 512, d = 8192 (128 CTAs) 9.2 with two or three, 8.7 with all eight; 256 x 256 (128 CTAs) 10.3 with two, 9.9
+// with three, 11.6 with five; 768 x 64 on rows of 8K (96 CTAs, 172 KB beside) 8.6 with two, 9.8 with three; 512 x 256
+// (256 CTAs) 11.9 with two, 13.6 with three.
+int mlp_stages_beside(int B, int d, int H1, int S, int sms, size_t beside) {
+    constexpr int kFewRows = 16;
+    const int64_t ctas = mlp_tiles(B, d, H1) * S;
+    if (2 * ctas <= sms || (ctas <= sms && B <= kFewRows)) return 0;
+    const size_t three = 3 * (kAChunk + (mlp_wide(B, d, H1) ? kBChunk<2 * kMlpNMin> : kBChunk<kMlpNMin>)) + 2048;
+    return ctas <= sms && (S < mlp_split(d) || beside + three <= size_t(228) * 1024) ? 3 : 2;
 }
 
 bool mlp_shape_ok(int d, int H1) {
@@ -343,6 +357,11 @@ static cudaError_t launch_mlp_n(const uint16_t *hidden, const uint16_t *W1, floa
     a.prefetch = prefetch ? 1 : 0;
     a.stages = st;
     a.parts = parts;
+    // An SM has 512 columns: where three CTAs of 256 fit it by shared memory, the third waits in its allocation until
+    // one of the others gives its columns back.  Those wait for their own copies and, with the prefetch bit, for the
+    // kernel before this one, all of whose CTAs run (this grid starts after each of them has released it): the wait
+    // ends.
+    static_assert(2 * N <= 512, "two parts' accumulators fit TMEM");
     a.columns = N * (parts / S);
     const dim3 grid(unsigned(S), unsigned(a.H1p / N), unsigned((B + kMlpM - 1) / kMlpM));
     // An explicit one-CTA cluster: the copies and the MMA commit address shared::cluster.

@@ -13,14 +13,15 @@ constexpr int kMlpNMin = 64;        // hidden units of the smaller tile (the lar
 
 // Parts of K for hidden size d: the most partial sums per (row, unit).
 int mlp_split(int d);
-// CTAs per tile of 128 rows x 64 units, each with an equal share of the parts: the partial sums per (row, unit)
-// of a launch.  A power of two, at most mlp_split(d).
-int mlp_ctas_per_tile(int B, int d, int H1);
-// Chunks a CTA stages at once when the rescan kernel runs beside the launch (0: all of them).
-int mlp_stages_beside(int B, int d, int H1, int S, int sms);
+// CTAs per tile of 128 rows x 64 or 128 units, each with an equal share of the parts: the partial sums per (row,
+// unit) of a launch.  A power of two, at most mlp_split(d).
+int mlp_ctas_per_tile(int B, int d, int H1, int sms);
+// Chunks a CTA stages at once when the rescan kernel runs beside the launch with `beside` bytes of shared memory an SM
+// (0: all of them).
+int mlp_stages_beside(int B, int d, int H1, int S, int sms, size_t beside);
 // Whether (d, H1) is within the kernel's limits.
 bool mlp_shape_ok(int d, int H1);
-// H1 rounded up to the 64-unit tile: the row stride of the partial sums.
+// H1 rounded up to the smaller tile's 64 units: the row stride of the partial sums.
 int mlp_hidden_padded(int H1);
 // part [S][B][mlp_hidden_padded(H1)] <- split-K partial sums of W1 h (fp32; units >= H1 are zero), S =
 // mlp_ctas_per_tile(...).  Launched with programmatic stream serialization; prefetch: the hidden states and W1 may be

@@ -316,9 +316,15 @@ static int step_entry(int32_t *ctx_tokens, int32_t *ctx_lens, const uint16_t *hi
         // Beside the rescan kernel the first layer stages few chunks at a time, so that every CTA of the
         // rescan kernel fits on the GPU while it runs (that kernel verifies and scans meanwhile).
         const int sms = sm_count_cached() > 0 ? sm_count_cached() : 148;
-        args.mlp_S = mlp_ctas_per_tile(p->B, p->d, p->probe_hidden);
-        if (launch_mlp_tc(probe_in, probe_w, part, p->B, p->d, p->probe_hidden, args.mlp_S, probe_pf, stream,
-                          p->index == nullptr ? mlp_stages_beside(p->B, p->d, p->probe_hidden, args.mlp_S, sms) : 0) != cudaSuccess)
+        args.mlp_S = mlp_ctas_per_tile(p->B, p->d, p->probe_hidden, sms);
+        int stages = 0;
+        if (p->index == nullptr) {  // (about a KB of each CTA is not dynamic)
+            const size_t ctas = (size_t(p->B) * size_t(split) + size_t(sms) - 1) / size_t(sms);
+            stages = mlp_stages_beside(p->B, p->d, p->probe_hidden, args.mlp_S, sms,
+                                       ctas * (rescan_smem_bytes(args, split) + 2048));
+        }
+        if (launch_mlp_tc(probe_in, probe_w, part, p->B, p->d, p->probe_hidden, args.mlp_S, probe_pf, stream, stages) !=
+            cudaSuccess)
             return SWITCHSD_ERR_CUDA;
         args.z1_part = part;
         mlp_early = probe_pf;

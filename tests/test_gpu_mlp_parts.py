@@ -1,5 +1,6 @@
 """The two-layer probe's first layer at the sizes where its split of K changes, against the oracle's probe in
-double precision: one and two parts of K a CTA (the line is 10 MB of partial sums), parts without a chunk of K
+double precision: one and two parts of K a CTA with tiles of 64 and 128 units (past 10 MB of partial sums; two parts
+where enough CTAs are left: 330 x 512 at d = 4096 and 8192 stand on either side), parts without a chunk of K
 (17 chunks over 16 parts), one and two chunks of K in all, ragged last tiles of rows and units, several units a
 thread of the rescan kernel, a bias, and the grids that stage all, three or two chunks at once.
 
@@ -16,7 +17,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B,H1,d", [(330, 512, 1096), (330, 509, 4096), (170, 1024, 2048), (16, 100, 64), (129, 65, 136),
-                                    (700, 256, 512), (64, 256, 5120), (300, 128, 8192)])
+                                    (700, 256, 512), (64, 256, 5120), (300, 128, 8192), (330, 512, 8192), (256, 768, 5120),
+                                    (400, 448, 4096), (4, 512, 8192), (1300, 128, 5120)])
 @pytest.mark.parametrize("prefetch", [0, 2])
 def test_first_layer_parts(B, H1, d, prefetch):
     import torch
