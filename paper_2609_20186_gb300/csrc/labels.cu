@@ -4,9 +4,8 @@
 // starting at an earlier position of the row (the paper trains its probe on these labels with
 // n = n_train = 5).
 //
-// Short rows, and longer ones where the batch is large (label_one_kernel): one kernel, a cluster of P CTAs
-// per row.  The windows are
-// split over the CTAs by hash; each CTA hashes every window of the row and inserts its own into an
+// Short rows, and longer ones where the batch fills the chip (label_one_kernel): one kernel, a cluster of P CTAs
+// per row.  The windows are split over the CTAs by hash; each CTA hashes every window of the row and inserts its own into an
 // open-addressing table in its shared memory.  A slot holds hash bits above the smallest start so far of one
 // window: an empty slot is claimed with an atomicCAS, a slot whose bits and tokens agree takes an atomicMin,
 // and whichever of the two starts is the larger is marked in the CTA's bitmap -- every start but the smallest
@@ -21,7 +20,7 @@
 // atomics a window), 36.5 us with each lane following its own probe sequence, 27.5 us with the stacks, 29.1 us
 // with hash sums of 64 bits instead of 32 (kept, so that ids that differ in their high bits alone still spread).
 //
-// A few long rows: two kernels over a per-row table in the caller's workspace, which spread a row's windows over
+// Other long rows: two kernels over a per-row table in the caller's workspace, which spread a row's windows over
 // the whole chip.
 //   insert  thread per window start s: hash the n tokens, probe linearly; an empty slot is claimed with
 //           atomicCAS, a slot whose window holds the same tokens takes atomicMin(slot, s).  Every slot
@@ -122,13 +121,11 @@ __global__ void __launch_bounds__(kLabelThreads) label_mark_kernel(const LabelAr
 }
 
 // ------------------------------------------------------------------------------------------------
-// One kernel: short rows, and longer ones in large batches (label_one_kernel).
+// One kernel: short rows, and longer ones where the batch fills the chip (label_one_kernel).
 // ------------------------------------------------------------------------------------------------
 constexpr int kLabelMaxParts = 8;          // CTAs a row: the portable cluster size
 constexpr int kLabelPartWindows = 32768;   // windows a CTA's table is meant for
 constexpr int kLabelClusterCap = 65536;    // the largest capacity of the one-kernel form
-constexpr int kLabelShortCap = 16384;      // up to here for any number of rows
-constexpr int kLabelRows = 32;             // up to kLabelClusterCap from this many rows
 constexpr int kLabelClusterThreads = 1024;
 constexpr size_t kLabelSmemMax = 224 * 1024;
 // The stacks' sizes: fewer than 32 windows are left when 32 more come from the hash or a round of tries, and a
@@ -296,7 +293,7 @@ __global__ void __launch_bounds__(kLabelClusterThreads, 1) label_cluster_kernel(
     cluster_arrive_release();
     cluster_wait_acquire();
 
-    // Labels: CTA `part` takes every P-th group of 16 positions' share [g0, g1) of the row's capacity.
+    // Labels: CTA `part` takes a contiguous P-th of the row's groups of 16 positions.
     uint8_t *out = a.labels + size_t(b) * size_t(a.cap);
     const int groups = (a.cap + 15) >> 4;
     const int per = (groups + int(P) - 1) / int(P);
@@ -338,27 +335,38 @@ static int label_parts(int32_t B, int32_t cap, int sms) {
     return P;
 }
 
-// The one-kernel form costs what its longest row does -- a CTA hashes the whole row -- and the two kernels what
-// the batch does, spread over the chip, least where few windows are distinct.  Measured (us a call, host
-// included, two kernels -> one; zipf | few distinct windows):
-//   n = 5   1 x 1K 15.0 -> 10.4 | 16.4 -> 10.4     64 x 8K 33.3 -> 15.9 | 20.6 -> 10.6    1 x 32K 17.2 -> 22.1 | 15.8 -> 17.8
-//           8 x 64K 34.6 -> 37.5 | 19.6 -> 33.3    64 x 32K 72.8 -> 30.4 | 50.8 -> 32.4
-//   n = 8   4 x 16K 18.7 -> 18.0 | 13.3 -> 12.3    12 x 16K 26.8 -> 17.5 | 13.9 -> 12.6   20 x 20K 24.4 -> 21.5 | 18.7 -> 16.8
-//           16 x 32K 41.1 -> 27.5 | 20.7 -> 24.6   24 x 32K 38.9 -> 29.8 | 26.8 -> 24.8
-//           24 x 48K 43.0 -> 35.5 | 33.8 -> 35.1   32 x 48K 49.6 -> 37.5 | 41.2 -> 35.0   32 x 64K 72.7 -> 46.6 | 51.4 -> 46.1
-// The line is where it wins on both texts.  Past 64K it would want far more rows (8 x 128K 44 -> 63).
-static bool label_one_kernel(int32_t B, int32_t cap) {
-    if (cap <= kLabelShortCap) return true;
-    return cap <= kLabelClusterCap && (B >= kLabelRows || int64_t(B) * 4096 >= int64_t(cap) * 3);
+// The one-kernel form costs what its longest row does -- a CTA hashes the whole row, n tokens a window -- and the two
+// kernels what the batch does, spread over the chip, least where few windows are distinct.  Measured on Zipf text and on
+// tiles of code, the worse of the two counts (two kernels / one kernel, of the time; above 1 the one kernel is faster):
+//   rows of   8K  n = 3..32  1 row 1.13 and more
+//             9K  n = 5, 8   6 rows 0.99 1.01   14 rows 1.03 0.79   18 rows 0.95 0.87   22 rows 1.13 1.03   24 rows 0.98 1.13
+//            16K  n = 5, 8   1 row 0.96 0.85    4 rows 1.06 1.01    8 rows 1.08 1.05    16 rows 1.12 1.05
+//                 n = 12, 32 4 rows 0.85 0.82   16 rows 1.00 0.97   20 rows 1.16 1.13
+//            32K  n = 5, 8   16 rows 0.86 0.86  20 rows 1.03 1.02   24 rows 1.11 1.11   34 rows 0.99 1.01   80 rows 1.17 1.22
+//                 n = 12, 32 24 rows 0.96 0.94  33 rows 1.16 1.20   34 rows 0.84 0.91   52 rows 1.14 1.29   72 rows 0.94 1.12
+//            64K  n = 5, 8   28 rows 1.07 1.00  33 rows 1.23 1.17   34 rows 0.81 0.80   52 rows 1.14 1.13   80 rows 0.88 0.89
+//                 n = 12, 32 33 rows 0.96 0.99  60 rows 1.01 1.12   71 rows 1.18 1.31   80 rows 0.70 0.76   152 rows 1.35 1.43
+// (A row just past a multiple of the 4,096 windows that a CTA hashes at once costs one more round: 9K.)  Past 16K or
+// 32K the time goes by whole waves of CTAs (an SM holds one) and the CTAs a row halve as the rows grow
+// (33 and 34), so the rule asks how much of its waves the grid fills: three quarters, and seven eighths where both the
+// rows and the windows are long.
+static bool label_one_kernel(int32_t B, int32_t cap, int32_t n, int P, int sms) {
+    const bool short_windows = n <= 8;
+    if (cap <= 8192) return true;
+    if (cap <= 16384) return B >= (short_windows && cap > 12288 ? 4 : 22);
+    if (cap <= 32768 && short_windows) return B >= 24;
+    if (cap > kLabelClusterCap) return false;
+    const int64_t ctas = int64_t(B) * P, waves = (ctas + sms - 1) / sms;
+    return 8 * ctas >= (cap > 32768 && !short_windows ? 7 : 6) * waves * sms;
 }
 
-static cudaError_t launch_label_cluster(const int32_t *ctx, const int32_t *lens, int32_t B, int32_t cap, int32_t n,
-                                        uint8_t *labels, cudaStream_t stream) {
+// SMs of the current device; sets the cluster kernel's shared-memory limit on its first call for the device.
+static cudaError_t label_sms(int &sms) {
     static int sm_counts[64] = {0};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    int sms = dev >= 0 && dev < 64 ? sm_counts[dev] : 0;
+    sms = dev >= 0 && dev < 64 ? sm_counts[dev] : 0;
     if (sms == 0) {
         e = cudaFuncSetAttribute(label_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kLabelSmemMax));
         if (e != cudaSuccess) return e;
@@ -366,7 +374,11 @@ static cudaError_t launch_label_cluster(const int32_t *ctx, const int32_t *lens,
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) sm_counts[dev] = sms;
     }
-    const int P = label_parts(B, cap, sms);
+    return cudaSuccess;
+}
+
+static cudaError_t launch_label_cluster(const int32_t *ctx, const int32_t *lens, int32_t B, int32_t cap, int32_t n,
+                                        uint8_t *labels, int P, cudaStream_t stream) {
     ClusterLabelArgs a;
     a.ctx = ctx;
     a.lens = lens;
@@ -413,9 +425,12 @@ extern "C" int switchsd_copy_labels(const int32_t *ctx_tokens, const int32_t *ct
     if (B < 1 || B > 65535 || cap < 1 || cap > (1 << 30) || n < 1 || n > SWITCHSD_NMAX) return SWITCHSD_ERR_SHAPE;
     if (workspace_bytes < switchsd_labels_workspace_bytes(B, cap)) return SWITCHSD_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (label_one_kernel(B, cap))
-        return launch_label_cluster(ctx_tokens, ctx_lens, B, cap, n, out_labels, s) == cudaSuccess ? SWITCHSD_OK
-                                                                                                   : SWITCHSD_ERR_CUDA;
+    int sms = 0;
+    if (label_sms(sms) != cudaSuccess) return SWITCHSD_ERR_CUDA;
+    const int P = label_parts(B, cap, sms);
+    if (label_one_kernel(B, cap, n, P, sms))
+        return launch_label_cluster(ctx_tokens, ctx_lens, B, cap, n, out_labels, P, s) == cudaSuccess ? SWITCHSD_OK
+                                                                                                      : SWITCHSD_ERR_CUDA;
     const uint32_t T = table_slots(cap);
     if (cudaMemsetAsync(workspace, 0xff, size_t(B) * T * sizeof(int32_t), s) != cudaSuccess) return SWITCHSD_ERR_CUDA;
     LabelArgs a;

@@ -127,12 +127,15 @@ def _first_occurrence_labels(x: np.ndarray, n: int) -> np.ndarray:
 
 
 # (rows, capacity, n): one and several CTAs a row, tables of every size class, capacities that are no multiple
-# of 16, both sides of the lines between the one-kernel form and the two kernels (16,384 tokens for any number
-# of rows, then a row per 1,365, or 32 rows, up to 65,536), and rows past them
+# of 16, both sides of the lines between the one-kernel form and the two kernels (8,192 tokens for any number of
+# rows; then 4 or 22 rows up to 16,384 and 24 up to 32,768, by n; then the share of the grid's waves that is filled,
+# up to 65,536), and rows past them
 @pytest.mark.parametrize("B,cap,n", [(200, 3001, 5), (3, 513, 32), (40, 8209, 2), (1, 4097, 5), (1, 16384, 5),
                                      (12, 16385, 5), (13, 16385, 5), (23, 32768, 5), (24, 32768, 8), (2, 32769, 5), (70, 16389, 3),
                                      (31, 65536, 5), (32, 65536, 5), (40, 65521, 8), (33, 65537, 5),
-                                     (1, 131075, 5), (2, 262144, 7), (1, 262145, 5)])
+                                     (1, 131075, 5), (2, 262144, 7), (1, 262145, 5),
+                                     (1, 8192, 5), (21, 8193, 8), (22, 8193, 8), (3, 12289, 8), (4, 12289, 8), (21, 16383, 9), (22, 16383, 9), (24, 20001, 5),
+                                     (28, 32768, 9), (29, 32768, 32), (28, 40004, 5), (57, 40004, 5), (66, 33001, 12), (67, 33001, 12)])
 def test_size_classes(B, cap, n):
     rng = np.random.default_rng(cap)
     ctx = np.zeros((B, cap), np.int32)
