@@ -411,8 +411,8 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
 }
 
 // ------------------------------------------------------------------------------------------------
-// Build.  One item = one (row, n); its buckets are split over P CTAs (part = the bucket's top bits).  A CTA
-// goes over the row in chunks of kChunk positions; per chunk, warp w owns a contiguous segment:
+// Build.  One item = one (row, n); its buckets are split over P CTAs (part = the bucket's top bits; a few calls take
+// index_walk_kernel below).  A CTA goes over the row in chunks of kChunk positions; per chunk, warp w owns a contiguous segment:
 //   1. hash and rank: every position's bucket, positions of other parts dropped, and its rank within the
 //      segment's positions of its bin (the next 6 to 8 bits of the bucket), kept in registers; the lanes of a bin
 //      find each other through a mask per bin in shared memory (an atomicOr, a read), and the segment's counts
@@ -683,6 +683,41 @@ __global__ void __launch_bounds__(kT, 1024 / kT) index_build_kernel(const BuildA
     }
 }
 
+// The same tables from one warp per item, which inserts its row's positions in increasing order, 32 at a time, into
+// heads that were set to -1 before (a dependent head read and write per 32 positions: about 1.4 us, whatever the
+// number of items up to a thousand or so).  For many short rows, where a CTA per item costs its fixed steps, and for
+// many rows so long that index_build_kernel would go over each of them once per part (index_walks).
+constexpr int kWalkWarps = 8;
+__global__ void __launch_bounds__(kWalkWarps * kWarp) index_walk_kernel(const BuildArgs a) {
+    const int lane = threadIdx.x & 31;
+    const int item = int(blockIdx.x) * kWalkWarps + int(threadIdx.x >> 5);
+    pdl_wait();
+    pdl_trigger();
+    if (item >= a.nn * a.B) return;
+    const int w = item / a.B, b = item - w * a.B;
+    const int n = a.n_min + w;
+    int32_t *heads = a.heads + (size_t(w) * a.B + b) * (size_t(1) << a.log2_buckets);
+    int32_t *prev = a.prev + (size_t(w) * a.B + b) * size_t(a.cap);
+    const int32_t *row = a.ctx + size_t(b) * size_t(a.cap);
+    int32_t L = a.lens[b];
+    if (L < 0 || L > a.cap) L = 0;
+    for (int32_t base = n - 1; base < L; base += kWarp) {
+        const int32_t p = base + lane;
+        const bool valid = p < L;
+        uint32_t bucket = 0xffffffffu;
+        if (valid) bucket = gram_hash(n, [&](int i) { return row[p - i]; }, a.log2_buckets);
+        const unsigned peers = __match_any_sync(kFull, bucket) & __ballot_sync(kFull, valid);
+        const int32_t old_head = valid ? heads[bucket] : -1;
+        __syncwarp();  // every lane has read its head before any lane replaces one
+        if (valid) {
+            const unsigned earlier = peers & ((1u << lane) - 1u);
+            prev[p] = earlier ? base + (31 - __clz(earlier)) : old_head;
+            if ((peers >> lane) == 1u) heads[bucket] = p;
+        }
+        __syncwarp();
+    }
+}
+
 // ------------------------------------------------------------------------------------------------
 // Host side.
 // ------------------------------------------------------------------------------------------------
@@ -720,6 +755,33 @@ static cudaError_t launch_index_build(BuildArgs a, cudaStream_t stream) {
     while (lp < 3 && (items << (lp + 1)) <= n_sm && a.log2_buckets - lp > 8) ++lp;
     a.log2_parts = lp;
     return launch_pdl(kernel, dim3(unsigned(items << lp)), dim3(kT), smem, stream, 0u, a);
+}
+
+// Parts that an item's buckets need (log2): a part has at most 8 bits of bins and 9 of keys.
+static int index_parts_needed(int log2_buckets) { return log2_buckets > 17 ? log2_buckets - 17 : 0; }
+
+// Whether the build takes the warp-per-item walk.  Measured, us, zipf text (walk, index_build_kernel; items = rows x n):
+//   short rows  items of 64: 1 6.1, 9.6   96 6.3, 9.9   24,576 18.6, 463      256: 6 8.9, 11.2   384 11.2, 17.3
+//               512: 6 13.2, 11.2   384 17.3, 17.6   1,536 19.1, 43.4      1K: 384 30.1, 19.4   1,536 33.2, 47.5
+//               1.5K: 384 43.7, 20.4   1,536 49.6, 50.6   6,144 150, 175   2K: 2,400 87, 92   6,144 193, 198   24,576 818, 769
+//   long rows   (ms) 300K (8 parts): 1,024 14.8, 16.3   2,048 24.9, 32.5       600K (16): 384 23.5, 22.1   768 27.0, 44.0
+//               1M (16): 384 48.5, 37.1   660 45.1, 64.3      2M (32): 192 104, 71   240 90, 89   288 84, 107
+//               4M (64): 48 183, 67   144 177, 204      8M (128): 24 372, 128   72 375, 373
+// The long rows' line is where items x parts pass about 8,192 (index_build_kernel's time per token goes by it, the
+// walk's does not); with 4 parts and fewer the walk is never ahead (2,048 items of 256K: 21.1 and 15.3).  Rows of few
+// distinct n-grams, whose heads stay in L2, would take the walk earlier (64 rows of 600K, period 64: 14.5 and 22.3).
+static bool index_walks(int32_t cap, int64_t items, int log2_buckets) {
+    const int lp = index_parts_needed(log2_buckets);
+    const bool short_rows = cap <= 256 || (cap <= 1536 && items >= cap) || (cap <= 2048 && items >= cap && items <= 8192);
+    return short_rows || (lp >= 3 && (items << lp) > 8192);
+}
+
+static cudaError_t launch_index_walk(const BuildArgs &a, cudaStream_t stream) {
+    const size_t items = size_t(a.nn) * size_t(a.B);
+    const cudaError_t e = cudaMemsetAsync(a.heads, 0xff, items * (size_t(1) << a.log2_buckets) * sizeof(int32_t), stream);
+    if (e != cudaSuccess) return e;  // (every head -1)
+    return launch_pdl(index_walk_kernel, dim3(unsigned((items + kWalkWarps - 1) / kWalkWarps)), dim3(kWalkWarps * kWarp), 0,
+                      stream, 0u, a);
 }
 
 int index_n_min(const switchsd_index *idx) { return idx->n_min; }
@@ -838,8 +900,10 @@ extern "C" int switchsd_index_build(switchsd_index *idx, const int32_t *ctx_toke
     a.nn = idx->nn;
     a.log2_buckets = idx->log2_buckets;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    a.log2_parts = 0;
     const cudaError_t e =
-        idx->cap <= 4096           ? launch_index_build<256, 4096, 6, 7>(a, st)
+        index_walks(a.cap, int64_t(a.nn) * a.B, a.log2_buckets) ? launch_index_walk(a, st)
+        : idx->cap <= 4096         ? launch_index_build<256, 4096, 6, 7>(a, st)
         : idx->cap <= 8192         ? launch_index_build<256, 8192, 7, 8>(a, st)
         : idx->cap <= 16384        ? launch_index_build<512, 16384, 7, 8>(a, st)
         : idx->log2_buckets <= 16  ? launch_index_build<1024, 32768, 7, 9>(a, st)

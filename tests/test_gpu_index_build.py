@@ -6,6 +6,9 @@ rows here end just below, at and above those sizes, and hold a period-1 and a pe
 everything), a small alphabet (dense repeats) and uniform ids.  Every chain is read back through the
 candidate step: for every gate length kappa it lists the W most recent ends of the kappa-gram, at the built
 length and at shorter ones (ends past the length are skipped).
+
+Rows of up to 256 tokens, many rows of up to 2,048, and many of more than 262,144 are built by a warp per row and n
+instead (capacity 260 with 240 and 300 of them stands on either side).
 """
 import ctypes
 
@@ -17,7 +20,8 @@ import oracle
 pytestmark = pytest.mark.gpu
 
 # (length, rows, n_min, n_max)
-SHAPES = [(1, 2, 1, 3), (7, 3, 3, 8), (33, 5, 2, 12), (1000, 40, 3, 8), (4096, 5, 2, 5),
+SHAPES = [(1, 2, 1, 3), (7, 3, 3, 8), (33, 5, 2, 12), (255, 9, 3, 8), (257, 40, 3, 8), (258, 50, 3, 8), (1000, 40, 3, 8),
+          (1001, 170, 3, 8), (1801, 310, 3, 8), (4096, 5, 2, 5),
           (4097, 4, 3, 5), (8192, 4, 3, 5), (8193, 5, 2, 4), (16383, 4, 3, 8), (16385, 4, 3, 8),
           (32768, 4, 2, 4), (32769, 5, 1, 2), (70001, 4, 3, 5), (140003, 4, 2, 3)]
 
@@ -39,7 +43,7 @@ def _rows(L, B, rng):
     return x
 
 
-@pytest.mark.parametrize("L,B,n_min,n_max", SHAPES, ids=[f"L{s[0]}" for s in SHAPES])
+@pytest.mark.parametrize("L,B,n_min,n_max", SHAPES, ids=[f"L{s[0]}_{s[1]}" for s in SHAPES])
 def test_built_chains(L, B, n_min, n_max):
     import torch
     from paper_2609_20186_gb300 import binding as bd
@@ -91,4 +95,46 @@ def test_built_chains(L, B, n_min, n_max):
                 for i in range(int(o["ncand"][b])):
                     m = int(o["cand_len"][b, i])
                     assert gl[b, i] == m and np.array_equal(g[b, i, :m], o["cand"][b, i, :m]), (cut, kappa, b, i)
+    idx.close()
+
+
+def test_many_long_rows():
+    """34 rows past 262,144 tokens with 31 n: the warp-per-item build, read back for the shortest, a middle and the
+    longest n of the first four rows and the last."""
+    import torch
+    from paper_2609_20186_gb300 import binding as bd
+    lib = bd.load()
+    B, L, n_min, n_max, W, D, d, k = 34, 262145, 2, 32, 16, 4, 8, 4
+    cap = (L + 3) // 4 * 4
+    ctx = np.zeros((B, cap), np.int32)
+    ctx[:, :L] = _rows(L, B, np.random.default_rng(L))
+    lens = np.full(B, L, np.int32)
+    c, ln = torch.from_numpy(ctx).cuda(), torch.from_numpy(lens).cuda()
+    idx = bd.NgramIndex(B, cap, n_min, n_max)
+    idx.build(c, ln)
+    h = torch.ones(B, d, dtype=torch.bfloat16, device="cuda")
+    hb = np.full((B, d), 0x3F80, np.uint16)
+
+    def ints(*s):
+        return torch.zeros(s, dtype=torch.int32, device="cuda")
+
+    for kappa in (n_min, 9, n_max):
+        cand, cl, nc, mode, mn, me = ints(B, W, D), ints(B, W), ints(B), ints(B), ints(B), ints(B)
+        score = torch.zeros(B, device="cuda")
+        p = bd.switchsd_params()
+        p.B, p.cap, p.d, p.k, p.n_min, p.n_max, p.kappa = B, cap, d, k, n_min, n_max, kappa
+        p.logit_tau = float("-inf")
+        p.index = idx.handle
+        p.out_match_n, p.out_match_end = mn.data_ptr(), me.data_ptr()
+        p.stream = torch.cuda.current_stream().cuda_stream
+        assert lib.switchsd_step_candidates(c.data_ptr(), ln.data_ptr(), h.data_ptr(), h.data_ptr(), ctypes.byref(p), W, D,
+                                            cand.data_ptr(), cl.data_ptr(), nc.data_ptr(), mode.data_ptr(),
+                                            score.data_ptr()) == bd.OK
+        for b in (0, 1, 2, 3, B - 1):
+            o = oracle.step_candidates(ctx, lens, hb, hb[0], W=W, D=D, n_min=n_min, n_max=n_max, kappa=kappa,
+                                       logit_tau=float("-inf"), rows=(b, b + 1))
+            assert (int(mn[b]), int(me[b]), int(nc[b])) == (o["match_n"][b], o["match_end"][b], o["ncand"][b]), (kappa, b)
+            for i in range(int(o["ncand"][b])):
+                m = int(o["cand_len"][b, i])
+                assert int(cl[b, i]) == m and cand[b, i, :m].tolist() == o["cand"][b, i, :m].tolist(), (kappa, b, i)
     idx.close()
