@@ -92,8 +92,8 @@ __device__ __forceinline__ float dot8_bf16(uint4 w, uint4 h, float acc) {
 // ring, probe_words and (without the ring) hash_words set.
 cudaError_t launch_rescan_kernel(const StepArgs &args, int split, cudaStream_t stream);
 size_t rescan_smem_bytes(const StepArgs &args, int split);
-// Sets args.hash_words: the pre-wait hash table when the grid has at least one CTA per SM (`sms` SMs) and
-// the table's shared memory keeps the launch's resident CTAs per SM at min(kRescanMinBlocks, what they are
+// Sets args.hash_words: the pre-wait hash table when the context is prefetched, the grid has at least one CTA per
+// SM (`sms` SMs) and the table's shared memory keeps the launch's resident CTAs per SM at min(kRescanMinBlocks, what they are
 // without it), else 0.  args.tile, args.z1_part, args.W and args.pv_p must be set.
 cudaError_t rescan_choose_hash(StepArgs &args, int split, int sms);
 

@@ -11,6 +11,7 @@ fails.
 """
 from __future__ import annotations
 
+import ctypes
 import os
 from concurrent.futures import ThreadPoolExecutor
 
@@ -110,13 +111,16 @@ def oracle_trace_rows(wl: synth.Workload, n_rows: int, steps: int, threads: int 
 
 
 def gpu_trace(wl: synth.Workload, steps: int, split: int = 0, ctx=None, lens=None, device="cuda",
-              fused: bool = False, use_index: bool = False, sampled: bool = False, extras: dict | None = None):
+              fused: bool = False, use_index: bool = False, sampled: bool = False, extras: dict | None = None,
+              prefetch: int = 0):
     """Runs the GPU loop on all rows; returns the per-step host copies of every output.
 
     fused=False: switchsd_step, target stand-in, switchsd_verify per iteration.
     fused=True:  switchsd_verify_step (verification of iteration t-1, then step t) and the target
                  stand-in per iteration; the last draft is verified by switchsd_verify.
     sampled=True: the sampled stand-in and switchsd_verify_sampled / switchsd_verify_sampled_step (T > 0).
+    prefetch: switchsd_params.prefetch; the hidden states are uploaded before the loop then, so that the
+                 kernel before each call is the target stand-in, which writes neither them nor contexts.
     extras: if given, the run keeps the per-mode counters (switchsd_params.counters) and stores them
     there under "counters" (host int64 array)."""
     import torch
@@ -127,10 +131,12 @@ def gpu_trace(wl: synth.Workload, steps: int, split: int = 0, ctx=None, lens=Non
     sess = Session(ctx, lens, wl.probe_weights(), k=wl.k, n_min=wl.n_min, n_max=wl.n_max,
                    kappa=wl.kappa, logit_tau=wl.logit_tau, probe_kind=wl.probe_kind,
                    probe_hidden=wl.probe_hidden, future=wl.future(), harness=wl.harness_params(),
-                   split=split, d=wl.d, use_index=use_index, device=device, counters=extras is not None)
+                   split=split, d=wl.d, use_index=use_index, device=device, counters=extras is not None,
+                   prefetch=prefetch)
+    states = [bf16_tensor(wl.hidden(t), sess.device) for t in range(steps)] if prefetch else None
     trace = []
     for t in range(steps):
-        hidden = bf16_tensor(wl.hidden(t), sess.device)
+        hidden = states[t] if prefetch else bf16_tensor(wl.hidden(t), sess.device)
         if fused and t > 0:
             if sampled:
                 sess.verify_sampled_step(hidden)
@@ -161,6 +167,38 @@ def gpu_trace(wl: synth.Workload, steps: int, split: int = 0, ctx=None, lens=Non
     if extras is not None:
         extras["counters"] = sess.counters.cpu().numpy()
     return trace, sess.ctx.cpu().numpy(), sess.lens.cpu().numpy()
+
+
+class _KernelNodeParams(ctypes.Structure):  # CUDA_KERNEL_NODE_PARAMS of the driver API
+    _fields_ = [("func", ctypes.c_void_p), ("dims", ctypes.c_uint * 7), ("kernel_params", ctypes.c_void_p),
+                ("extra", ctypes.c_void_p), ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+
+def kernel_names(call) -> list[str]:
+    """The (mangled) names of the kernels that `call`, which takes a stream and launches on it, would launch:
+    captured into a graph that is never replayed, and read from the graph's kernel nodes."""
+    import torch
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph, stream=stream):
+        call(stream)
+    cu = ctypes.CDLL("libcuda.so.1")
+    raw, count = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0)
+    assert cu.cuGraphGetNodes(raw, None, ctypes.byref(count)) == 0
+    nodes = (ctypes.c_void_p * count.value)()
+    assert cu.cuGraphGetNodes(raw, nodes, ctypes.byref(count)) == 0
+    names = []
+    for node in nodes:
+        kind = ctypes.c_int(-1)
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        if kind.value != 0:  # CU_GRAPH_NODE_TYPE_KERNEL
+            continue
+        p, name = _KernelNodeParams(), ctypes.c_char_p()
+        assert cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)) == 0
+        assert cu.cuFuncGetName(ctypes.byref(name), ctypes.c_void_p(p.func or p.kern)) == 0
+        names.append(name.value.decode())
+    return names
 
 
 def compare(wl: synth.Workload, o_trace, g_trace, rows, o_ctx=None, g_ctx=None):

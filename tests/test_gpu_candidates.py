@@ -55,10 +55,11 @@ def oracle_loop(wl, rows, steps, Wc, D):
     return trace, ctx
 
 
-def gpu_loop(wl, steps, Wc, D, split=0, fused=False, use_index=False):
+def gpu_loop(wl, steps, Wc, D, split=0, fused=False, use_index=False, prefetch=0):
     """fused: switchsd_verify_candidates_step verifies iteration t-1's candidates and searches step t's in
     one launch; the last iteration's candidates are verified by switchsd_verify_candidates.  use_index:
-    the incremental n-gram index (built from the initial contexts) searches, verifies and inserts."""
+    the incremental n-gram index (built from the initial contexts) searches, verifies and inserts.  prefetch:
+    switchsd_params.prefetch, with the hidden states uploaded before the loop."""
     import torch
     from paper_2609_20186_gb300 import binding as bd, bf16_tensor
     lib = bd.load()
@@ -80,7 +81,7 @@ def gpu_loop(wl, steps, Wc, D, split=0, fused=False, use_index=False):
     p = bd.switchsd_params()
     p.B, p.cap, p.d, p.k = B, cap, wl.d, wl.k
     p.n_min, p.n_max, p.kappa, p.logit_tau = wl.n_min, wl.n_max, wl.kappa, wl.logit_tau
-    p.probe_kind, p.probe_hidden, p.split = wl.probe_kind, wl.probe_hidden, split
+    p.probe_kind, p.probe_hidden, p.split, p.prefetch = wl.probe_kind, wl.probe_hidden, split, prefetch
     ws = torch.empty(max(256, bd.switchsd_workspace_bytes(B, wl.probe_kind, wl.probe_hidden, wl.d)),
                      dtype=torch.uint8, device=dev)
     p.workspace, p.workspace_bytes = ws.data_ptr(), ws.numel()
@@ -101,9 +102,10 @@ def gpu_loop(wl, steps, Wc, D, split=0, fused=False, use_index=False):
     vp.cand_len, vp.ncand, vp.ctx_tokens, vp.ctx_lens = vl.data_ptr(), vn.data_ptr(), c.data_ptr(), ln.data_ptr()
     vp.status, vp.stream = vst.data_ptr(), p.stream
     vp.index = idx.handle if idx is not None else None
+    states = [bf16_tensor(wl.hidden(t), dev) for t in range(steps)] if prefetch else None
     trace = []
     for t in range(steps):
-        hid = bf16_tensor(wl.hidden(t), dev)
+        hid = states[t] if prefetch else bf16_tensor(wl.hidden(t), dev)
         if fused and t > 0:
             assert lib.switchsd_verify_candidates_step(
                 vc.data_ptr(), tg.data_ptr(), vl.data_ptr(), vn.data_ptr(), acc.data_ptr(), ch.data_ptr(),
@@ -182,12 +184,12 @@ KAPPA_LOW = {
 }
 
 
-@pytest.mark.parametrize("split", [0, 1], ids=["rescan_kernel", "step_kernel"])
+@pytest.mark.parametrize("split", [0, 1], ids=["one_copy", "ring"])
 @pytest.mark.parametrize("name", list(KAPPA_LOW))
 def test_candidates_kappa_below_n_min(name, split):
     """kappa below n_min on the scan path: a candidate needs only kappa tokens of common suffix, fewer
     than a match that decides the mode, so the scan's filter must not test more than kappa tokens.  The
-    library's split takes the rescan kernel; one CTA over 20K-token rows takes the step kernel."""
+    library's split stages a range with one copy; one CTA over 20K-token rows takes the ring of tiles."""
     wl = KAPPA_LOW[name]
     rows = range(wl.B)
     o_trace, o_ctx = oracle_loop(wl, rows, wl.steps, 10, 20)

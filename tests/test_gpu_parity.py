@@ -50,7 +50,7 @@ def test_split_invariance(split, fused):
 
 
 def test_multi_tile_ring():
-    """Rows long enough for several kTileMax tiles per CTA (two-stage ring), fused and separate."""
+    """Rows long enough for several tiles per CTA (the ring), fused and separate."""
     wl = W["mixed_128k"].scaled(name="mixed_ring", B=2, L0=70001, steps=6)
     for fused in (False, True):
         _run_small(wl, split=2, fused=fused)
@@ -81,13 +81,13 @@ def test_planted(variant):
 FULL_ROWS = {"uniform_8k": 64, "zipf_32k": 64, "code_16k": 64, "mixed_128k": 16}
 
 
-@pytest.mark.parametrize("name", list(FULL_ROWS))
-def test_full_size_every_row(name):
-    """Full-size workload in the benchmark's launch configuration (fused verify + step), every step:
-    every row (the first 64 of the code workload's 256) against the oracle."""
-    wl = W[name]
+PREFETCHED_STEPS = 64
+
+
+def _full_size(name, steps, prefetch):
+    wl = W[name].scaled(steps=steps)
     n = FULL_ROWS[name]
-    g_trace, g_ctx, _ = lockstep.gpu_trace(wl, wl.steps, fused=True)
+    g_trace, g_ctx, _ = lockstep.gpu_trace(wl, wl.steps, fused=True, prefetch=prefetch)
     o_trace, o_ctx, _ = lockstep.oracle_trace_rows(wl, n, wl.steps)
     rows = range(n)
     flips, stats = lockstep.compare(wl, o_trace, g_trace, rows, o_ctx, g_ctx)
@@ -97,6 +97,20 @@ def test_full_size_every_row(name):
     for t in g_trace:
         assert np.all(t["status"] == 0) and np.all(t["vstatus"] == 0)
         assert np.all(t["len"] <= wl.k)
+
+
+@pytest.mark.parametrize("name", list(FULL_ROWS))
+def test_full_size_every_row(name):
+    """Full-size workload (fused verify + step), every step: every row (the first 64 of the code workload's 256)
+    against the oracle."""
+    _full_size(name, W[name].steps, 0)
+
+
+@pytest.mark.parametrize("name", list(FULL_ROWS))
+def test_full_size_every_row_prefetched(name):
+    """The same in the benchmark's launch configuration: context and probe prefetched, and rows with room for as few
+    appends, where the rescan kernel's instances are the benchmark's (held by test_gpu_hash_instance.py)."""
+    _full_size(name, PREFETCHED_STEPS, 3)
 
 
 @pytest.mark.parametrize("fused", [False, True], ids=["separate", "fused"])
