@@ -23,7 +23,11 @@ pytestmark = pytest.mark.gpu
 SHAPES = [(1, 2, 1, 3), (7, 3, 3, 8), (33, 5, 2, 12), (255, 9, 3, 8), (257, 40, 3, 8), (258, 50, 3, 8), (1000, 40, 3, 8),
           (1001, 170, 3, 8), (1801, 310, 3, 8), (4096, 5, 2, 5),
           (4097, 4, 3, 5), (8192, 4, 3, 5), (8193, 5, 2, 4), (16383, 4, 3, 8), (16385, 4, 3, 8),
-          (32768, 4, 2, 4), (32769, 5, 1, 2), (70001, 4, 3, 5), (140003, 4, 2, 3)]
+          (32768, 4, 2, 4), (32769, 5, 1, 2), (70001, 4, 3, 5), (140003, 4, 2, 3),
+          # rows enough that a CTA takes all of an item's buckets (its links go out through shared memory), of every
+          # instance, with one chunk and with a second one
+          (4095, 40, 3, 6), (8192, 40, 3, 5), (16384, 40, 3, 5), (32768, 40, 3, 5), (32770, 40, 3, 5), (40001, 40, 3, 5),
+          (65536, 40, 3, 5)]
 
 
 def _rows(L, B, rng):
