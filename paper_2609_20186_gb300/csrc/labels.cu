@@ -132,6 +132,7 @@ constexpr size_t kLabelSmemMax = 224 * 1024;
 // round of compares can return 32 in between.
 constexpr int kLabelTries = 96, kLabelCompares = 64;
 constexpr uint32_t kSlotEmpty = 0xffffffffu;
+constexpr uint32_t kLabelProbes = 512;     // slots a window tries in a pass
 constexpr uint32_t kLabelMul = 0x9E3779B1u;
 
 struct ClusterLabelArgs {
@@ -139,7 +140,7 @@ struct ClusterLabelArgs {
     uint8_t *labels;
     int32_t cap, n, pos_bits;  // cap < 1 << pos_bits: a slot's low bits hold a start, the rest hash bits
     uint32_t slots;            // of a CTA's table
-    int32_t bm_words;          // of a CTA's bitmap: ceil(cap / 32)
+    int32_t bm_words;          // of each of a CTA's two bitmaps: ceil(cap / 32)
 };
 
 __device__ __forceinline__ uint32_t label_mix(uint64_t sum) {
@@ -161,14 +162,15 @@ __global__ void __launch_bounds__(kLabelClusterThreads, 1) label_cluster_kernel(
     extern __shared__ __align__(16) uint32_t lsm[];
     uint32_t *tab = lsm;                          // [slots]
     uint32_t *bm = lsm + ((a.slots + 3) & ~3u);   // [bm_words]: starts whose window occurs earlier
-    uint2 *stacks = reinterpret_cast<uint2 *>(bm + ((a.bm_words + 3) & ~3));
+    uint32_t *left = bm + ((a.bm_words + 3) & ~3);  // [bm_words]: starts left for the next pass
+    uint2 *stacks = reinterpret_cast<uint2 *>(left + ((a.bm_words + 3) & ~3));
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthreads = blockDim.x;
     const uint32_t part = cluster_ctarank(), P = cluster_nctarank();
     const int b = blockIdx.y;
     uint2 *stack_t = stacks + (kLabelTries + kLabelCompares) * warp, *stack_c = stack_t + kLabelTries;
     for (uint32_t i = tid; i < a.slots; i += nthreads) tab[i] = kSlotEmpty;
-    for (int i = tid; i < a.bm_words; i += nthreads) bm[i] = 0u;
+    for (int i = tid; i < a.bm_words; i += nthreads) bm[i] = left[i] = 0u;
     __syncthreads();
     pdl_wait();
     pdl_trigger();
@@ -200,18 +202,19 @@ __global__ void __launch_bounds__(kLabelClusterThreads, 1) label_cluster_kernel(
         size += __popc(who);
         __syncwarp();
     };
-    // the next slot of a window; after a whole round of a full table (only tokens built against the hash fill
-    // it) every window equal to this one ends here too, since nothing leaves the table: compare with every
-    // earlier window
+    // The next slot of a window.  After kLabelProbes of them it is left for a pass over the emptied table with another
+    // hash: only tokens built against the hash, or a part with far more windows than its share, fill a table so (a row
+    // of 32K tokens with 17K or 32K distinct windows in a part of 16K slots takes 0.7 or 3.5 ms; 206 ms or 4 s when they
+    // tried every slot and were then compared with every earlier window).  Equal
+    // windows go the same way, since they try the same slots in the same order and nothing leaves the table: a slot
+    // that one of them found taken by another window is so for all that come later.
+    bool leaves = false;  // this thread left a window
     auto next_slot = [&](uint2 &e) {
         uint32_t slot = e.y & 0xffffu, probes = (e.y >> 16) + 1u;
-        if (probes >= a.slots) {
+        if (probes >= kLabelProbes) {
             const int32_t s = int32_t(e.x & pos_mask);
-            for (int32_t p = 0; p < s; ++p)
-                if (same(p, s)) {
-                    mark(s);
-                    break;
-                }
+            atomicOr(&left[s >> 5], 1u << (s & 31));
+            leaves = true;
             return false;
         }
         if (++slot == a.slots) slot = 0u;
@@ -256,6 +259,24 @@ __global__ void __launch_bounds__(kLabelClusterThreads, 1) label_cluster_kernel(
         push(stack_t, tries, again, e);
     };
 
+    // The slot entry of window s with hash m, and its first slot: the slot from another multiple than the part's, the
+    // entry's tag from the low bits.
+    auto entry = [&](uint32_t m, int32_t s) {
+        return make_uint2((m << a.pos_bits) | uint32_t(s), __umulhi(m * 0x85EBCA77u, a.slots));
+    };
+    auto full_rounds = [&]() {
+        while (tries >= kWarp) {
+            try_round();
+            if (compares >= kWarp) compare_round();
+        }
+    };
+    auto drain = [&]() {
+        while (tries > 0 || compares > 0) {
+            if (tries > 0) try_round();
+            if (compares >= kWarp || tries == 0) compare_round();
+        }
+    };
+
     constexpr int kW4 = 4;  // windows a lane hashes at once
     for (int32_t s0 = warp * (kWarp * kW4); s0 < nw; s0 += nthreads * kW4) {
         uint64_t h[kW4];  // 64-bit sums, so that tokens that differ in their high bits alone still spread
@@ -276,18 +297,35 @@ __global__ void __launch_bounds__(kLabelClusterThreads, 1) label_cluster_kernel(
         for (int u = 0; u < kW4; ++u) {
             const int32_t s = s0 + kWarp * u + lane;
             const uint32_t m = label_mix(h[u]);
-            // the part from the hash's top bits, the slot from another multiple's, the entry's tag from the low ones
-            push(stack_t, tries, s < nw && __umulhi(m, P) == part,
-                 make_uint2((m << a.pos_bits) | uint32_t(s), __umulhi(m * 0x85EBCA77u, a.slots)));
-            while (tries >= kWarp) {
-                try_round();
-                if (compares >= kWarp) compare_round();
-            }
+            push(stack_t, tries, s < nw && __umulhi(m, P) == part, entry(m, s));  // the part from the top bits
+            full_rounds();
         }
     }
-    while (tries > 0 || compares > 0) {
-        if (tries > 0) try_round();
-        if (compares >= kWarp || tries == 0) compare_round();
+    drain();
+    // The windows left, if any: each pass empties the table, where at least kLabelProbes of them then find a slot.
+    // (Word w of `left` is read and written by its warp alone within a pass.)
+    uint64_t seed = 0u;
+    while (__syncthreads_or(leaves)) {
+        leaves = false;
+        seed += 0x9E3779B97F4A7C15ull;
+        for (uint32_t i = tid; i < a.slots; i += nthreads) tab[i] = kSlotEmpty;
+        __syncthreads();
+        for (int w = warp; w < a.bm_words; w += nthreads / kWarp) {
+            const uint32_t word = left[w];
+            if (word == 0u) continue;
+            __syncwarp();
+            if (lane == 0) left[w] = 0u;
+            __syncwarp();
+            const int32_t s = 32 * w + lane;
+            const bool on = (word >> lane & 1u) != 0u;
+            uint64_t sum = 0u;
+            uint32_t pw = 1u;
+            if (on)
+                for (int i = 0; i < n; ++i, pw *= kLabelMul) sum += uint64_t(uint32_t(x[s + i])) * pw;
+            push(stack_t, tries, on, entry(label_mix(sum ^ seed), s));
+            full_rounds();
+        }
+        drain();
     }
     // every CTA's marks are in (P = 1: the cluster is this CTA)
     cluster_arrive_release();
@@ -393,7 +431,7 @@ static cudaError_t launch_label_cluster(const int32_t *ctx, const int32_t *lens,
     // threads by the row, which every CTA hashes: four windows each
     int threads = 128;
     while (threads < kLabelClusterThreads && 4 * threads < cap) threads *= 2;
-    const size_t fixed = size_t((a.bm_words + 3) & ~3) * 4 + size_t(threads / kWarp) * (kLabelTries + kLabelCompares) * sizeof(uint2) + 16;
+    const size_t fixed = 2 * size_t((a.bm_words + 3) & ~3) * 4 + size_t(threads / kWarp) * (kLabelTries + kLabelCompares) * sizeof(uint2) + 16;
     const size_t most = (kLabelSmemMax - fixed) / 4;
     const size_t want = size_t(2) * size_t(windows) + 64;
     a.slots = uint32_t(want < most ? want : most);

@@ -156,3 +156,52 @@ def test_size_classes(B, cap, n):
         L = int(lens[b])
         assert np.array_equal(got[b, :L], _first_occurrence_labels(ctx[b, :L], n)), b
         assert not got[b, L:].any()
+
+
+def _label_part(ids: np.ndarray, parts: int) -> np.ndarray:
+    """The part of a row's cluster that takes the window of one token (label_mix of csrc/labels.cu, n = 1)."""
+    with np.errstate(over="ignore"):
+        h = ids.astype(np.uint32)
+        h = (h ^ (h >> np.uint32(15))) * np.uint32(0x2C1B3C6D)
+        h = (h ^ (h >> np.uint32(12))) * np.uint32(0x297A2D39)
+        h ^= h >> np.uint32(15)
+    return ((h.astype(np.uint64) * np.uint64(parts)) >> np.uint64(32)).astype(np.int64)
+
+
+def test_full_table():
+    """More distinct windows in one part of the hash than its table has slots: those that find the table full
+    compare with every earlier window, and repeats of them, and of the ones in the table, are still marked."""
+    import torch
+    from paper_2609_20186_gb300 import binding as bd
+    from tests import lockstep
+    B, cap, n = 24, 32768, 1
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    parts = 1
+    while parts < 8 and 2 * parts * (B + 5) <= sms and cap // (2 * parts) >= 512:
+        parts *= 2
+    slots = 2 * (cap // parts) + 64
+    rng = np.random.default_rng(3)
+    ids = rng.permutation(1 << 20)[:parts * (slots + 4000) * 2].astype(np.int32)
+    mine = ids[_label_part(ids, parts) == parts - 1]
+    full = mine[:slots + 700]
+    rest = np.setdiff1d(ids, mine)
+    assert parts > 1 and len(full) == slots + 700
+    ctx = np.zeros((B, cap), np.int32)
+    for b, order in ((0, 1), (5, -1)):
+        again = np.concatenate([full[:300], full[-600:]])  # some of the table's and some of the others
+        x = np.concatenate([full[::order], rest[:2000], rng.permutation(again), rest[:50]])
+        ctx[b, :len(x)] = x
+        ctx[b, len(x):] = rest[2000:2000 + cap - len(x)]
+    lens = np.full(B, 7, np.int32)
+    lens[[0, 5]] = cap
+
+    def call(stream):
+        bd.switchsd_copy_labels(c, ln, out, n=n, workspace=ws, stream=stream)
+    c, ln = torch.from_numpy(ctx).cuda(), torch.from_numpy(lens).cuda()
+    out = torch.zeros(c.shape, dtype=torch.uint8, device="cuda")
+    ws = torch.empty(int(bd.load().switchsd_labels_workspace_bytes(B, cap)), dtype=torch.uint8, device="cuda")
+    assert any("label_cluster_kernel" in k for k in lockstep.kernel_names(call))
+    got = _labels(ctx, lens, n)
+    for b in (0, 5):
+        want = _first_occurrence_labels(ctx[b], n)
+        assert want.sum() >= 900 and np.array_equal(got[b], want), b
