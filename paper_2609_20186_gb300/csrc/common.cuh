@@ -149,12 +149,6 @@ __device__ __forceinline__ uint32_t map_to_rank(const void *p, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(out) : "r"(smem_addr(p)), "r"(rank));
     return out;
 }
-__device__ __forceinline__ void st_cluster_u64(uint32_t addr, unsigned long long v) {
-    asm volatile("st.shared::cluster.u64 [%0], %1;\n" ::"r"(addr), "l"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(addr), "f"(v) : "memory");
-}
 
 // Programmatic dependent launch.  Every kernel of the library is launched with programmatic stream
 // serialization: it waits for the preceding kernel (griddepcontrol.wait) before its first read of
@@ -191,30 +185,6 @@ __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.w
 
 // Generic accesses to shared memory before it are ordered before asynchronous accesses to it after it.
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
-
-// Remote arrive on an mbarrier in another CTA of the cluster (release, cluster scope).
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(cluster_addr) : "memory");
-}
-
-// Bounded acquire-at-cluster-scope wait for phase `parity` (pairs with mbar_arrive_remote).
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity) {
-    const uint32_t addr = smem_addr(bar);
-    for (uint32_t it = 0; it < kWaitLimit; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n"
-            ".reg .pred p;\n"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-            "selp.u32 %0, 1, 0, p;\n"
-            "}\n"
-            : "=r"(done)
-            : "r"(addr), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
 
 // Launches `kernel` on `stream` with programmatic stream serialization and, when cluster_x >= 1, an
 // explicit cluster shape of cluster_x CTAs (1 included: the cluster instructions of the rescan kernel,

@@ -420,9 +420,9 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
 //   2. scan: offsets of every (bin, warp), so that a bin's entries lie in position order;
 //   3. scatter: (position, key) into a queue in shared memory, key = the bucket's remaining bits (<= 9);
 //   4. link: warp w takes the bins w, w + kW, ... on its own (no barrier): the bin's heads (<= 512, 16-bit
-//      chunk positions) live in shared memory, the entries are linked 32 at a time in order through
-//      __match_any_sync, and the bin's heads go out in one coalesced write, the empty ones included (so
-//      nothing clears the table first);
+//      chunk positions) live in shared memory, the entries are linked 32 at a time in order (entries of one key
+//      in a round find each other through the head that one of them holds), and the bin's heads go out in one
+//      coalesced write, the empty ones included (so nothing clears the table first);
 //   5. the links, held in shared memory as 16-bit chunk positions, go out coalesced (P = 1; with P > 1 a
 //      part's positions are scattered and step 4 stores them).
 // Steps 1 to 3 are one stable radix pass, so the time does not depend on how the tokens repeat, except that
@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(kIdxMaxWarps * kWarp) index_kernel(const Index
 // instead of 128.  With 256: ranks by eight ballots a position, counted in a pass of their own 177 us; the groups
 // of equal keys in a round of step 4 by nine ballots
 // (six rounds in ten hold one) 155 us.  The tokens staged in shared memory by one copy made no difference.  The
-// table written sets the floor (201 MB of heads + 50 MB of links: 37 us at the measured copy bandwidth); what
+// table written sets the floor (101 MB of heads + 50 MB of links: 22 us at the measured copy bandwidth); what
 // bounds it is the shared-memory pipe (random accesses, three to four wavefronts each: 70 % of its peak while a
 // CTA runs) and the issue rate, at one 1024-thread CTA an SM, 2.5 waves of them here.
 // ------------------------------------------------------------------------------------------------

@@ -264,7 +264,10 @@ __host__ __device__ inline CandLayout cand_layout(int range, int W, int D, bool 
 //
 // The ring: every warp scans its share of each tile as it lands, keeps its best match's continuation while
 // that tile is staged, and counts itself out of the stage; the last warp out refills it.  No CTA barrier and
-// no producer warp: the warps drift by up to the ring's depth.
+// no producer warp: the warps drift by up to the ring's depth.  Its CTAs are sized for rows that stream from memory, a
+// few warps an SM; where the compares weigh more than the stream -- n_min = 1 and a last token that fills a seventh
+// of the row -- a ring of 256-thread CTAs, 16 a row, was faster (29 rows of 292K Zipf tokens 18.4 us a launch, 29.4 here;
+// 33 rows of random ids 16.3 and 7.2).
 enum { kScanTokens = 0, kScanHashed = 1, kScanRing = 2 };
 template <bool kSampled, bool kCand, int kScan, bool kMlp>
 __global__ void __launch_bounds__(kRescanThreads, kScan == kScanRing ? kRingLaunchBlocks : kRescanLaunchBlocks)
