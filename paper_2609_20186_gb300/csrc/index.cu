@@ -19,7 +19,9 @@
 // tokens compared, the next link and the tokens that follow it.  The lookup starts from the link that the
 // insert of the suffix's own end found, and the draft is written from the registers of the n that wins.  16
 // rows of 128K tokens, n = 2..12, 16 launches: 82.6 us with the heads and links read again for the lookup and
-// the draft gathered at the end (seven round trips), 71.7 us so.
+// the draft gathered at the end (seven round trips), 71.7 us so, over positions that the index held already (the lengths
+// were rewound between passes).  With every append new (the index rebuilt before each pass; medians of 12 texts, one
+// pass at a time): 111.7 us against 74.9, and 124.1 against 85.2 with the seven round trips.
 // Candidate mode (W > 0, as switchsd_step_candidates / switchsd_verify_candidates): the previous W
 // candidates are verified and the longest accepted one appended; the warp of n = kappa walks its
 // chain on past the first match and lists the W most recent ends whose kappa-gram equals the
